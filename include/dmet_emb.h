@@ -77,7 +77,13 @@ typedef enum {
  * Frobenius, measured): see the library's documentation; BF16X3 and FP16X2 meet 1e-6, TF32 does
  * not. */
 typedef enum {
-  DMET_PREC_FP64 = 0,    /* every product and sum in IEEE FP64 */
+  DMET_PREC_FP64 = 0,    /* FP64 inputs, results and intermediates. Small products run as IEEE FP64
+                            FMAs; larger ones round each operand row once to 58-bit integers
+                            (relative to the row's 2-norm), multiply those exactly and round each
+                            result to FP64, which is no less accurate than the chain of FMAs. An
+                            infinity or NaN in an operand row gives NaN in every result of that
+                            row there. Products whose scratch the workspace limit does not leave
+                            run as FMAs. */
   DMET_PREC_BF16X3 = 1,  /* three bf16 slices per operand, six slice products per multiply-add */
   DMET_PREC_TF32 = 2,    /* one TF32 slice, one product (about 2^-11 relative per product) */
   DMET_PREC_TF32X3 = 3,  /* two TF32 slices, three products (about 2^-22), half the 16-bit rate */

@@ -138,6 +138,9 @@ namespace dmet {
 cudaError_t make_tmap_3d(CUtensorMap* map, int prec, const void* base, unsigned long long k_elems,
                          unsigned long long rows, unsigned long long slices, unsigned long long row_stride_elems,
                          unsigned long long slice_stride_elems, int box_rows);
+// 3-D over [planes][rows][K] bf16 with K a multiple of 64, a (64, box_rows, 1) box and 128-byte swizzled rows;
+cudaError_t make_tmap_rows128(CUtensorMap* map, const void* base, unsigned long long k_elems, unsigned long long rows,
+                              unsigned long long planes, unsigned long long plane_elems, int box_rows);
 // 4-D over a slice-interleaved operand [rows][K / BK][slices][BK] (BK = 64 bytes of elements) with a
 // (BK, 1, 1, box_rows) box: one slice of one K block.
 cudaError_t make_tmap_interleaved(CUtensorMap* map, int prec, const void* base, unsigned long long k_elems,

@@ -17,6 +17,7 @@
 
 #include "../../include/dmet_emb.h"
 #include "internal.h"
+#include "rns.h"
 #include "tc_gemm.cuh"
 
 using namespace dmet;
@@ -269,6 +270,8 @@ struct Workspace {
   double* X[2] = {nullptr, nullptr};
   double2* lq_all[2] = {nullptr, nullptr};
   double2* full = nullptr;  // one complex ERI block before 4-fold packing
+  void* rns = nullptr;      // residues of the FP64 products (rns.cu); none: they run on the FP64 pipe
+  size_t rns_b = 0;
   size_t crep_b = 0, T_b = 0, Z_b = 0, S_b = 0, X_b[2] = {0, 0}, lq_all_b[2] = {0, 0}, full_b = 0;
   // split-BF16 operands
   void* Ls = nullptr;
@@ -306,6 +309,7 @@ struct GroupedPlan {
 struct dmet_emb_plan_s {
   cudaStream_t stream = nullptr;  // the caller's stream
   int device = 0;
+  int sms = 152;
   std::vector<Prob> probs;
   size_t ws_limit = 0;
   // One workspace per problem when they all fit the limit (problems then run concurrently on
@@ -374,6 +378,8 @@ struct dmet_emb_plan_s {
   }
 };
 
+
+int device_sms();
 
 namespace {
 
@@ -530,6 +536,8 @@ static dmet_status_t queue_block_copies(dmet_emb_plan_s* P, const Prob& pr, int 
   return DMET_OK;
 }
 
+constexpr size_t kRnsScratch = (size_t)1 << 30;
+
 struct Timed {
   dmet_emb_plan_s* P;
   int kc;
@@ -545,6 +553,11 @@ struct Timed {
       b = get_event(P);
       if (a) cudaEventRecord(a, P->cs);
     }
+  }
+  // n more launches than the constructor counted
+  void more(int n) {
+    P->ks[kc].launches += n;
+    if (kc != KC_COPY) P->launches += n;
   }
   ~Timed() {
     if (P->prof && a && b) {
@@ -578,6 +591,44 @@ ZgemmArgs zargs() {
   z.alpha = 1.0;
   z.batch = 1;
   return z;
+}
+
+// An FP64 complex GEMM (or real rank-K product) on the plan's current stream: through residues on the
+// tensor cores where that is faster (rns.cu), else on the FP64 pipe. `t` counts its launches.
+RnsCtx rns_ctx(dmet_emb_plan_s* P) {
+  RnsCtx c;
+  if (!P->W || !P->W->rns) return c;
+  c.scratch = P->W->rns;
+  c.bytes = P->W->rns_b;
+  c.sms = P->sms;
+  c.err = P->derr;
+  c.wait_ns = P->wait_ns;
+  c.withhold_loads = P->withhold_loads;
+  return c;
+}
+
+dmet_status_t zgemm(dmet_emb_plan_s* P, Timed& t, const ZgemmArgs& z, int al, bool cj, int bl) {
+  const RnsCtx c = rns_ctx(P);
+  if (!rns_takes_zgemm(z, c)) {
+    CK(launch_zgemm(z, al, cj, bl, P->cs));
+    return DMET_OK;
+  }
+  int n = 0;
+  CK(rns_zgemm(z, al, cj, bl, c, P->cs, &n));
+  t.more(n - 1);
+  return DMET_OK;
+}
+
+dmet_status_t dsyrk(dmet_emb_plan_s* P, Timed& t, const DsyrkArgs& a) {
+  const RnsCtx c = rns_ctx(P);
+  if (!rns_takes_dsyrk(a, c)) {
+    CK(launch_dsyrk(a, P->cs));
+    return DMET_OK;
+  }
+  int n = 0;
+  CK(rns_dsyrk(a, c, P->cs, &n));
+  t.more(n - 1);
+  return DMET_OK;
 }
 
 dmet_status_t ensure(void** p, size_t* have, size_t need) {
@@ -679,7 +730,7 @@ dmet_status_t run_half_transform(dmet_emb_plan_s* P, Prob& pr, const Tables& tb,
     // table entries carry absolute indices; T holds this block's entries only
     z.D = P->W->T - (long long)e0 * z.sD;
     Timed t(P, KC_TRANSFORM_1, 8.0 * n * (double)naux * nao * nao * E, 0.0);
-    CK(launch_zgemm(z, A_KM, false, B_NK, P->cs));
+    TRY(zgemm(P, t, z, A_KM, false, B_NK));
   }
   {
     // Z_q[P][i][j] = sum_{(r, mu)} w_r conj(C^{k1_r}_{mu i}) T_r[mu][P][j]   (bra side + FT to R=0)
@@ -704,9 +755,12 @@ dmet_status_t run_half_transform(dmet_emb_plan_s* P, Prob& pr, const Tables& tb,
     z.alpha = real ? 1.0 : pr.lq_scale;
     z.D = (real ? P->W->Z : dest) - (long long)(real ? b0 : dest_slot0) * z.sD;
     double fl = 0;
-    for (int i = b0; i < b1; ++i) fl += 8.0 * n * (double)naux * n * tb.t2[i].w;
+    for (int i = b0; i < b1; ++i) {
+      fl += 8.0 * n * (double)naux * n * tb.t2[i].w;
+      z.K = std::max(z.K, tb.t2[i].w);  // (each entry's own K is in the table)
+    }
     Timed t(P, KC_TRANSFORM_2, fl, 0.0);
-    CK(launch_zgemm(z, A_KM, true, B_KN, P->cs));
+    TRY(zgemm(P, t, z, A_KM, true, B_KN));
   }
   return DMET_OK;
 }
@@ -766,7 +820,7 @@ dmet_status_t eri_s8(dmet_emb_plan_s* P, Prob& pr, const double2* L, const doubl
       a.mode = blk == 1 ? 1 : 0;
       const double fl = a.mode == 0 ? (double)a.M * (a.M + 1.0) * K : 2.0 * a.M * (double)a.N * K;
       Timed t(P, KC_CONTRACT, fl, 0.0);
-      CK(launch_dsyrk(a, P->cs));
+      TRY(dsyrk(P, t, a));
     }
   }
   return DMET_OK;
@@ -798,7 +852,7 @@ dmet_status_t eri_full(dmet_emb_plan_s* P, Prob& pr, const double2* L, const dou
       z.alpha = 1.0 / pr.nk;
       z.beta = 1;
       Timed t(P, KC_CONTRACT_FULL, 8.0 * (double)na2 * nb2 * pr.naux, 0.0);
-      CK(launch_zgemm(z, A_KM, false, B_KN, P->cs));
+      TRY(zgemm(P, t, z, A_KM, false, B_KN));
     }
     if (s4) {
       Timed t(P, KC_PACK, 0.0, 16.0 * (double)na2 * nb2 + (double)eri_bytes_of(pr.d, blk));
@@ -861,6 +915,42 @@ WsSizes ws_for(const Prob& pr, int bq) {
   return w;
 }
 
+// Scratch with which the FP64 products of a problem run through residues in one chunk each.
+size_t rns_want(const Prob& pr, int bq) {
+  if (pr.mixed) return 0;
+  size_t need = 0;
+  const int E = std::max(max_entries(pr.nat, bq), pr.pack == DMET_PACK_S8 ? max_entries(pr.con, bq) : 0);
+  int reps = 0;
+  for (int q = 0; q < pr.nk; ++q) reps = std::max(reps, pr.s.nrep[q]);
+  for (int s = 0; s < pr.nspin; ++s) {
+    ZgemmArgs z = zargs();
+    z.M = pr.n[s];
+    z.N = pr.naux * pr.nao;
+    z.K = pr.nao;
+    z.batch = E;
+    need = std::max(need, rns_need(z));
+    z.N = pr.naux * pr.n[s];
+    z.K = reps * pr.nao;
+    z.batch = bq;
+    need = std::max(need, rns_need(z));
+    if (pr.pack == DMET_PACK_S8) {
+      DsyrkArgs a;
+      std::memset(&a, 0, sizeof(a));
+      a.M = (int)pr.npair[s];
+      a.N = (int)pr.npair[pr.nspin == 2 ? 1 : 0];
+      a.K = 2 * bq * pr.naux;
+      a.mode = pr.nspin == 2;
+      need = std::max(need, rns_need(a));
+    } else {
+      z.M = z.N = pr.n[s] * pr.n[s];
+      z.K = pr.naux;
+      z.batch = 1;
+      need = std::max(need, rns_need(z));
+    }
+  }
+  return need;
+}
+
 dmet_status_t upload_tables(Tables& t) {
   if (t.t1.empty()) return DMET_OK;
   CK(cudaMalloc(&t.d_t1, t.t1.size() * sizeof(int4)));
@@ -880,7 +970,7 @@ void free_tables(Tables& t) {
 }
 
 void free_workspace(Workspace& w) {
-  void* ptrs[] = {w.crep, w.T, w.Z, w.S, w.X[0], w.X[1], w.lq_all[0], w.lq_all[1], w.full,
+  void* ptrs[] = {w.crep, w.T, w.Z, w.S, w.X[0], w.X[1], w.lq_all[0], w.lq_all[1], w.full, w.rns,
                   w.Ls, w.Cb[0], w.Cb[1], w.Cc, w.A2, w.ZT, w.Xt[0], w.Xt[1], w.sc};
   for (void* q : ptrs) cudaFree(q);
   w = Workspace();
@@ -1724,6 +1814,7 @@ dmet_status_t dmet_emb_plan(const dmet_emb_desc_t* descs, int32_t n_problems, vo
   dmet_emb_plan_s* P = new dmet_emb_plan_s();
   P->stream = (cudaStream_t)stream;
   cudaGetDevice(&P->device);
+  P->sms = device_sms();
   P->ws_limit = workspace_limit ? workspace_limit : ((size_t)8 << 30);
   P->probs.resize(n_problems);
   std::vector<WsSizes> wneed(n_problems);
@@ -1861,6 +1952,20 @@ dmet_status_t dmet_emb_plan(const dmet_emb_desc_t* descs, int32_t n_problems, vo
       c.Xt[s] = std::max(c.Xt[s], d.Xt[s]);
     }
   }
+  // Residue scratch from what the limit leaves: shared evenly by the workspaces, at most kRnsScratch each
+  // and no more than one chunk needs; below 8 MiB the FP64 products stay on the FP64 pipe.
+  std::vector<size_t> rsz(P->ws.size(), 0);
+  {
+    size_t used = 0;
+    for (size_t i = 0; i < P->ws.size(); ++i) used += wsz[i].total() + mixed_total(msz[i]);
+    const size_t share = used < P->ws_limit ? (P->ws_limit - used) / P->ws.size() : 0;
+    for (int p = 0; p < n_problems; ++p) {
+      size_t& r = rsz[P->ws_of[p]];
+      r = std::max(r, std::min({rns_want(P->probs[p], P->probs[p].bq), share, kRnsScratch}));
+    }
+    for (auto& r : rsz)
+      if (r < ((size_t)8 << 20)) r = 0;
+  }
   dmet_status_t st = DMET_OK;
   auto alloc = [&](void** ptr, size_t* have, size_t bytes) {
     if (st == DMET_OK && bytes) st = ensure(ptr, have, bytes);
@@ -1878,6 +1983,7 @@ dmet_status_t dmet_emb_plan(const dmet_emb_desc_t* descs, int32_t n_problems, vo
       alloc((void**)&W.X[s], &W.X_b[s], need.X[s]);
       alloc((void**)&W.lq_all[s], &W.lq_all_b[s], need.lq_all[s]);
     }
+    if (st == DMET_OK && rsz[i]) alloc(&W.rns, &W.rns_b, rsz[i]);
     alloc(&W.Ls, &W.Ls_b, mn.Ls);
     alloc(&W.Cc, &W.Cc_b, mn.Cc);
     alloc(&W.A2, &W.A2_b, mn.A2);
@@ -3130,7 +3236,7 @@ dmet_status_t dmet_emb_eri_fftdf(dmet_emb_plan_t P, int32_t problem, const void*
         z.batch = kp;
         Timed tc(P, KC_FFTDF, 8.0 * (double)nx * nxb * ng * nc, kp > 1 ? 16.0 * kp * nx * nxb * 2 : 0.0,
                  kp > 1 ? 2 : 1);
-        CK(launch_zgemm(z, A_KM, false, B_KN, P->cs));
+        TRY(zgemm(P, tc, z, A_KM, false, B_KN));
         if (kp > 1) CK(launch_sum_parts(dPart, kp, nx * nxb, (double2*)eri_out[blk], P->cs));
       }
     }

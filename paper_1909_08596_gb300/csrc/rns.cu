@@ -1,0 +1,1047 @@
+// FP64 matrix products on the 16-bit tensor cores through residues.
+//
+//   D(m, n) = sum_k A(m, k) B(n, k)   for FP64 A and B, real or complex
+//
+// The FP64 pipe of this part issues 2 FMAs a clock and SM (1.26 TFLOP/s in all), the 16-bit tensor
+// cores about 1500 times that, and 16-bit integers up to 2^7 multiply and add exactly in their FP32
+// accumulators. So every row of A and of B is scaled by a power of two to integers of about kBeta
+// bits (a 2-norm of at most 2^kBeta, so that no inner product exceeds 2^(2 kBeta)), and the integer
+// product is formed exactly by the Chinese remainder theorem (the number-theoretic form of the
+// error-free matrix products of Ozaki et al.): kMods pairwise coprime moduli of at most 8 bits, one
+// GEMM of symmetric residues (bf16, |r| <= 128) per modulus, and the product recovered modulo
+// P = prod p_i > 2 * 2^(2 kBeta). The only errors are the rounding of the operands to integers, half
+// a unit of 2^-kBeta of the row's norm (5 bits below the FP64 rounding of an element of the row's
+// size), and one rounding of the result, so it is closer to the exact product than a chain of FP64
+// FMAs, whose error grows with sqrt(K).
+//
+//   1. rns_convert_kernel: per operand row, the scale from its norm; then residues [mod][batch][row][K],
+//      K-major (complex operands as interleaved (re, im) pairs along K; the column operand of a
+//      complex product as two rows, (re, -im) for the real and (im, re) for the imaginary part).
+//   2. rns_gemm_kernel: tcgen05 (128 x up to 256 tiles, TMA-fed), one job per (modulus, batch, tile).
+//      After every kSegStages K blocks the FP32 sums, exact below 2^24, are reduced modulo p and the
+//      running residue is kept as one byte per element in Y [mod][batch][row][col].
+//   3. rns_crt_kernel: recovers the signed 117-bit integer, rounds it once to FP64, undoes the scales
+//      and writes the caller's layout.
+//
+// A row with an infinity or a NaN gives NaN in every result it enters.
+
+#include <cuda.h>
+#include <cuda_bf16.h>
+#include <limits.h>
+#include <math.h>
+#include <stdint.h>
+
+#include <algorithm>
+#include <cstring>
+
+#include "rns.h"
+#include "tc_common.cuh"
+
+namespace dmet {
+
+namespace {
+
+using namespace tc;
+
+constexpr int kMods = 15;
+constexpr int kBeta = 58;
+__host__ __device__ constexpr int mod_of(int i) {
+  constexpr int p[kMods] = {256, 253, 251, 247, 241, 239, 233, 229, 227, 223, 217, 211, 199, 197, 193};
+  return p[i];
+}
+
+using u128 = unsigned __int128;
+
+__host__ __device__ constexpr u128 mod_product() {
+  u128 p = 1;
+  for (int i = 0; i < kMods; ++i) p *= (u128)mod_of(i);
+  return p;
+}
+// W_i = (P / p_i) * ((P / p_i)^-1 mod p_i): sum r_i W_i = x (mod P) for the residues r_i of x.
+__host__ __device__ constexpr u128 crt_weight(int i) {
+  const u128 m = mod_product() / (u128)mod_of(i);
+  const int p = mod_of(i), a = (int)(m % (u128)p);
+  int inv = 1;
+  while ((a * inv) % p != 1) ++inv;
+  return m * (u128)inv;
+}
+// 30-bit limbs, so that a residue times a limb is a signed 32 x 32 -> 64-bit multiply-add
+__host__ __device__ constexpr int limb(u128 x, int j) { return (int)((x >> (30 * j)) & (u128)0x3fffffff); }
+
+constexpr bool mods_ok() {
+  for (int i = 0; i < kMods; ++i)
+    for (int j = 0; j < i; ++j) {
+      int a = mod_of(i), b = mod_of(j);
+      while (b) {
+        const int t = a % b;
+        a = b;
+        b = t;
+      }
+      if (a != 1) return false;
+    }
+  return true;
+}
+static_assert(mods_ok(), "the moduli must be pairwise coprime");
+static_assert((mod_product() >> (2 * kBeta + 1)) != 0, "P must exceed 2 * 2^(2 kBeta)");
+static_assert((mod_product() >> 120) == 0, "four 30-bit limbs must hold P");
+
+template <int I>
+struct Crt {
+  static constexpr u128 W = crt_weight(I);
+  static constexpr int w0 = limb(W, 0), w1 = limb(W, 1), w2 = limb(W, 2), w3 = limb(W, 3);
+};
+
+// Symmetric residue of 2^(16 j) modulo p.
+__host__ __device__ constexpr int chunk_weight(int i, int j) {
+  const int p = mod_of(i);
+  int r = 1;
+  for (int t = 0; t < 16 * j; ++t) r = (r * 2) % p;
+  return r > p / 2 ? r - p : r;
+}
+
+constexpr int kPoison = INT_MIN;  // scale of a row that holds an infinity or a NaN
+constexpr float kMagic = 12582912.f;  // 1.5 * 2^23: adding it rounds to an integer
+
+// v - p * rint(v / p) for an integer |v| <= 2^24: a residue with |r| <= (p + 1) / 2 (the rounding of v / p
+// can pick the neighbour when v / p lies within 2^-9 of a half-integer), so at most 128 for p = 256 and
+// 127 for the others: it fits a byte, modulo 256 for p = 256. (p = 255 would reach 128 and is left out.)
+__device__ __forceinline__ float sym_mod(float v, float p, float rp) {
+  const float q = __fadd_rn(fmaf(v, rp, kMagic), -kMagic);
+  return fmaf(q, -p, v);
+}
+
+__constant__ float kModF[kMods] = {256, 253, 251, 247, 241, 239, 233, 229, 227, 223, 217, 211, 199, 197, 193};
+
+// ---------------- operand conversion ----------------
+
+enum { SRC_COMPLEX = 0, SRC_COMPLEX2 = 1, SRC_REAL = 2 };
+
+struct ConvArgs {
+  const double* src;
+  const int4* tab;  // batch z reads tab[tab0 + z].x (sel 0) or .y (sel 1) in units of sbatch, K from .w
+  int tab0, sel;
+  long long sbatch;       // batch stride, in elements (complex or real)
+  long long s_row, s_k;   // strides of a row and of a k index, in elements
+  int rows, K, Kp;        // Kp: real K, padded to the GEMM's K block
+  int conj;
+  __nv_bfloat16* R;       // [mod][batch][rows (x 2 for SRC_COMPLEX2)][Kp]
+  long long smod;         // elements per modulus plane
+  int* exps;              // [batch][rows]
+};
+
+struct RowNorm {
+  float s;  // sum of squares in units of 2^(2 e)
+  int e;    // biased exponent of the reference
+  int bad;
+};
+
+__device__ __forceinline__ float pow2f(int e) { return __uint_as_float((unsigned)(e + 127) << 23); }
+
+__device__ __forceinline__ void norm_add(RowNorm& n, double x) {
+  const unsigned hi = (unsigned)__double2hiint(x) & 0x7fffffffu;
+  int e = (int)(hi >> 20);
+  if (e == 0x7ff) n.bad = 1;
+  if (e == 0) {
+    if ((hi | (unsigned)__double2loint(x)) == 0) return;
+    e = 1;  // subnormal: counted as the smallest normal
+  }
+  int d = e - n.e;
+  if (d > 0) {
+    n.s = d < 60 ? n.s * pow2f(-2 * d) : 0.f;
+    n.e = e;
+    d = 0;
+  }
+  if (d > -60) {
+    const float f = __uint_as_float(((unsigned)(127 + d) << 23) | ((hi & 0xfffffu) << 3) | 7u);
+    n.s = fmaf(f, f, n.s);
+  }
+}
+
+__device__ __forceinline__ void norm_merge(RowNorm& a, float s, int e, int bad) {
+  a.bad |= bad;
+  const int d = e - a.e;
+  if (d > 0) {
+    a.s = (d < 60 ? a.s * pow2f(-2 * d) : 0.f) + s;
+    a.e = e;
+  } else if (d > -60) {
+    a.s += s * pow2f(2 * d);
+  }
+}
+
+// The power s for which the row times 2^s has a 2-norm of at most 2^kBeta.
+__device__ __forceinline__ int norm_scale(const RowNorm& n) {
+  if (n.bad) return kPoison;
+  if (n.s == 0.f) return 0;
+  const unsigned b = __float_as_uint(n.s * 1.001f);
+  const int se = (int)(b >> 23) - 127;                    // floor(log2 s)
+  return kBeta - (n.e - 1023 + ((se + 2) >> 1));
+}
+
+// rint(x 2^s) as a two's-complement integer (round half away from zero), |result| <= 2^kBeta.
+__device__ __forceinline__ long long to_int(double x, int s) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  const int e = (int)((b >> 52) & 0x7ff);
+  unsigned long long m = b & ((1ull << 52) - 1);
+  if (e) m |= 1ull << 52;
+  const int sh = (e ? e : 1) - 1075 + s;
+  if (sh >= 0) m <<= min(sh, 63);
+  else m = sh > -55 ? (m + (1ull << (-sh - 1))) >> -sh : 0ull;
+  return (long long)b < 0 ? -(long long)m : (long long)m;
+}
+
+// Four signed 16-bit digits of a, as floats: a = sum c_j 2^(16 j).
+__device__ __forceinline__ void digits(long long a, float (&c)[4]) {
+  const unsigned long long b = (unsigned long long)a + 0x8000800080008000ull;
+  const unsigned lo = (unsigned)b, hi = (unsigned)(b >> 32);
+  constexpr float bias = 8388608.f + 32768.f;  // 2^23 + 2^15
+  c[0] = __uint_as_float(__byte_perm(lo, 0x4B000000u, 0x7610)) - bias;
+  c[1] = __uint_as_float(__byte_perm(lo, 0x4B000000u, 0x7632)) - bias;
+  c[2] = __uint_as_float(__byte_perm(hi, 0x4B000000u, 0x7610)) - bias;
+  c[3] = __uint_as_float(__byte_perm(hi, 0x4B000000u, 0x7632)) - bias;
+}
+
+// |c_j w_j| <= 2^22 for j = 1, 2, 2^18 for j = 3 (|a| <= 2^59) and 2^15 for j = 0: the sum is exact.
+template <int I>
+__device__ __forceinline__ float residue(const float (&c)[4]) {
+  constexpr float w1 = (float)chunk_weight(I, 1), w2 = (float)chunk_weight(I, 2), w3 = (float)chunk_weight(I, 3);
+  constexpr float p = (float)mod_of(I), rp = 1.0f / p;
+  return sym_mod(fmaf(c[3], w3, fmaf(c[2], w2, fmaf(c[1], w1, c[0]))), p, rp);
+}
+
+template <int SRC, int I>
+__device__ __forceinline__ void store_residues(const float (&cr)[4], const float (&ci)[4], __nv_bfloat16* dst,
+                                               long long smod, int Kp) {
+  if constexpr (I < kMods) {
+    const float re = residue<I>(cr), im = residue<I>(ci);
+    const __nv_bfloat162 p = __floats2bfloat162_rn(re, SRC == SRC_COMPLEX2 ? -im : im);
+    *reinterpret_cast<__nv_bfloat162*>(dst) = p;
+    if constexpr (SRC == SRC_COMPLEX2) *reinterpret_cast<__nv_bfloat162*>(dst + Kp) = __floats2bfloat162_rn(im, re);
+    store_residues<SRC, I + 1>(cr, ci, dst + smod, smod, Kp);
+  }
+}
+
+// One CTA converts 32 operand rows: first their norms, then the residues, 32 (re, im) or
+// (k, k + 1) pairs at a time, a lane per pair, so that every store of a warp is 128 contiguous bytes.
+// Rows that are contiguous in memory (s_row = 1) pass through a transpose in shared memory.
+template <int SRC>
+__global__ void __launch_bounds__(256) rns_convert_kernel(const ConvArgs a) {
+  __shared__ double2 tile[32][33];
+  __shared__ float sh_s[8][32];
+  __shared__ int sh_e[8][32], sh_bad[8][32], sh_scale[32];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int z = blockIdx.y, r0 = blockIdx.x * 32;
+  long long off = (long long)z * a.sbatch;
+  int K = a.K;
+  if (a.tab) {
+    const int4 t = a.tab[a.tab0 + z];
+    off = (a.sel ? (long long)t.y : (long long)t.x) * a.sbatch;
+    K = t.w;
+  }
+  const bool rowfast = a.s_row == 1;
+  const double2* src2 = reinterpret_cast<const double2*>(a.src) + off;
+  const double* src1 = a.src + off;
+
+  // norms
+  if (rowfast) {
+    RowNorm n{0.f, 0, 0};
+    if (r0 + lane < a.rows) {
+      for (int k = warp; k < K; k += 8) {
+        if constexpr (SRC == SRC_REAL) {
+          norm_add(n, src1[(r0 + lane) + (long long)k * a.s_k]);
+        } else {
+          const double2 v = src2[(r0 + lane) + (long long)k * a.s_k];
+          norm_add(n, v.x);
+          norm_add(n, v.y);
+        }
+      }
+    }
+    sh_s[warp][lane] = n.s;
+    sh_e[warp][lane] = n.e;
+    sh_bad[warp][lane] = n.bad;
+    __syncthreads();
+    if (warp == 0) {
+      for (int w = 1; w < 8; ++w) norm_merge(n, sh_s[w][lane], sh_e[w][lane], sh_bad[w][lane]);
+      sh_scale[lane] = norm_scale(n);
+    }
+  } else {
+    for (int i = 0; i < 4; ++i) {
+      const int r = r0 + warp * 4 + i;
+      RowNorm n{0.f, 0, 0};
+      if (r < a.rows) {
+        for (int k = lane; k < K; k += 32) {
+          if constexpr (SRC == SRC_REAL) {
+            norm_add(n, src1[(long long)r * a.s_row + (long long)k * a.s_k]);
+          } else {
+            const double2 v = src2[(long long)r * a.s_row + (long long)k * a.s_k];
+            norm_add(n, v.x);
+            norm_add(n, v.y);
+          }
+        }
+      }
+#pragma unroll
+      for (int o = 16; o; o >>= 1) {
+        const float s = __shfl_xor_sync(0xffffffffu, n.s, o);
+        const int e = __shfl_xor_sync(0xffffffffu, n.e, o), b = __shfl_xor_sync(0xffffffffu, n.bad, o);
+        norm_merge(n, s, e, b);
+      }
+      if (lane == 0) sh_scale[warp * 4 + i] = norm_scale(n);
+    }
+  }
+  __syncthreads();
+  if (warp == 0 && r0 + lane < a.rows) a.exps[(long long)z * a.rows + r0 + lane] = sh_scale[lane];
+
+  constexpr int RR = SRC == SRC_COMPLEX2 ? 2 : 1;
+  const int units = SRC == SRC_REAL ? (K + 1) / 2 : K, upad = a.Kp / 2;
+  for (int u0 = 0; u0 < upad; u0 += 32) {
+    if (rowfast) {
+      __syncthreads();
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int ul = warp * 4 + i, u = u0 + ul;
+        double2 v = make_double2(0.0, 0.0);
+        if (u < units && r0 + lane < a.rows) {
+          if constexpr (SRC == SRC_REAL) {
+            v.x = src1[(r0 + lane) + (long long)(2 * u) * a.s_k];
+            if (2 * u + 1 < K) v.y = src1[(r0 + lane) + (long long)(2 * u + 1) * a.s_k];
+          } else {
+            v = src2[(r0 + lane) + (long long)u * a.s_k];
+          }
+        }
+        tile[ul][lane] = v;
+      }
+      __syncthreads();
+    }
+    const int u = u0 + lane;
+    for (int i = 0; i < 4; ++i) {
+      const int rl = warp * 4 + i, r = r0 + rl;
+      if (r >= a.rows) break;
+      double2 v = make_double2(0.0, 0.0);
+      if (rowfast) {
+        v = tile[lane][rl];
+      } else if (u < units) {
+        if constexpr (SRC == SRC_REAL) {
+          v.x = src1[(long long)r * a.s_row + (long long)(2 * u) * a.s_k];
+          if (2 * u + 1 < K) v.y = src1[(long long)r * a.s_row + (long long)(2 * u + 1) * a.s_k];
+        } else {
+          v = src2[(long long)r * a.s_row + (long long)u * a.s_k];
+        }
+      }
+      const int s = sh_scale[rl];
+      long long ar = 0, ai = 0;
+      if (s != kPoison) {
+        ar = to_int(v.x, s);
+        ai = to_int(v.y, s);
+        if (SRC != SRC_REAL && a.conj) ai = -ai;
+      }
+      float cr[4], ci[4];
+      digits(ar, cr);
+      digits(ai, ci);
+      if (u < upad) {
+        __nv_bfloat16* dst = a.R + (((long long)z * a.rows + r) * RR) * a.Kp + 2 * u;
+        store_residues<SRC, 0>(cr, ci, dst, a.smod, a.Kp);
+      }
+    }
+  }
+}
+
+// ---------------- GEMM of residues ----------------
+
+constexpr int kTileM = 128;
+constexpr int kBK = 64;             // K elements per stage (128-byte rows)
+constexpr int kSegStages = 15;      // 960 K per segment: 960 * 128^2 + 128 < 2^24
+constexpr int kStages = 4;
+constexpr int kEpi = 8;             // epilogue warps
+constexpr int kGemmThreads = 32 * (4 + kEpi);
+constexpr int kABytes = kTileM * 128;
+constexpr int kBBytes = 256 * 128;
+constexpr int kStageBytes = kABytes + kBBytes;
+constexpr int kGemmSmem = 1024 + kStages * kStageBytes + 256;
+
+struct GemmArgs {
+  int nbatch, rows, cols;   // per batch entry
+  int rt, ct, bn;           // row tiles, column tiles, tile width (a multiple of 16, <= 256)
+  int tri, h0;              // tri: only tiles with a column <= the last row (square product, bn = 256); row 0 of
+                            // this launch is row 256 h0 of the product
+  int row0;                 // first row of the launch in the row operand
+  int tiles;                // per (modulus, batch)
+  int nkb;                  // K blocks
+  signed char* Y;           // [mod][batch][rows][ldy]
+  long long ymod;
+  int ldy;
+};
+
+struct Tile {
+  int mod, z, m0, n0;
+};
+
+// Tiles of the lower triangle: the row tiles 2 h and 2 h + 1 have h0 + h + 1 column tiles each.
+__host__ __device__ inline int tri_tiles_before(int mt, int h0) {
+  const int h = mt >> 1;
+  return h * h + (2 * h0 + 1) * h + (mt & 1) * (h0 + h + 1);
+}
+
+__device__ __forceinline__ Tile tile_of(const GemmArgs& g, int job) {
+  Tile t;
+  const int per = g.nbatch * g.tiles;
+  t.mod = job / per;
+  int r = job - t.mod * per;
+  t.z = r / g.tiles;
+  r -= t.z * g.tiles;
+  int mt, nt;
+  if (g.tri) {
+    int h = (int)((sqrtf((float)(2 * g.h0 + 1) * (float)(2 * g.h0 + 1) + 4.f * (float)r) - (float)(2 * g.h0 + 1)) * 0.5f);
+    while (tri_tiles_before(2 * h, g.h0) > r) --h;
+    while (tri_tiles_before(2 * h + 2, g.h0) <= r) ++h;
+    const int rem = r - tri_tiles_before(2 * h, g.h0), w = g.h0 + h + 1;
+    const int up = rem >= w;
+    mt = 2 * h + up;
+    nt = rem - up * w;
+  } else {
+    mt = r / g.ct;
+    nt = r - mt * g.ct;
+  }
+  t.m0 = mt * kTileM;
+  t.n0 = nt * g.bn;
+  return t;
+}
+
+// 16 accumulator columns to bytes: v (+ the running residue) modulo p.
+__device__ __forceinline__ uint4 reduce16(const uint32_t (&v)[16], bool add, uint4 prev, float p, float rp) {
+  uint32_t w[4];
+  const uint32_t pv[4] = {prev.x, prev.y, prev.z, prev.w};
+#pragma unroll
+  for (int g = 0; g < 4; ++g) {
+    uint32_t b[4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      float x = __uint_as_float(v[4 * g + c]);
+      if (add) x += (float)(int)(signed char)(pv[g] >> (8 * c));
+      b[c] = __float_as_uint(__fadd_rn(sym_mod(x, p, rp), kMagic));  // the low byte is the residue's
+    }
+    w[g] = __byte_perm(__byte_perm(b[0], b[1], 0x0040), __byte_perm(b[2], b[3], 0x0040), 0x5410);
+  }
+  return make_uint4(w[0], w[1], w[2], w[3]);
+}
+
+__global__ void __launch_bounds__(kGemmThreads, 1)
+    rns_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const GemmArgs g,
+                    int njobs, unsigned int* err, unsigned long long lim, int withhold) {
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+  uint64_t* bars = (uint64_t*)(smem + kStages * kStageBytes);
+  // bars: full[S], empty[S], accf[2], acce[2], done; then the TMEM address and a counter
+  volatile uint32_t* tmem_slot = (volatile uint32_t*)(bars + 2 * kStages + 5);
+  volatile int* consumed = (volatile int*)(bars + 2 * kStages + 5) + 1;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  auto full = [&](int s) { return smem_u32(bars + s); };
+  auto empty = [&](int s) { return smem_u32(bars + kStages + s); };
+  auto accf = [&](int b) { return smem_u32(bars + 2 * kStages + b); };
+  auto acce = [&](int b) { return smem_u32(bars + 2 * kStages + 2 + b); };
+  const uint32_t done_bar = smem_u32(bars + 2 * kStages + 4);
+  auto a_tile = [&](int s) { return smem_u32(smem + s * kStageBytes); };
+  auto b_tile = [&](int s) { return smem_u32(smem + s * kStageBytes + kABytes); };
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < kStages; ++s) {
+      mbar_init(full(s), 1);
+      mbar_init(empty(s), 1);
+    }
+    for (int b = 0; b < 2; ++b) {
+      mbar_init(accf(b), 1);
+      mbar_init(acce(b), kEpi);
+    }
+    mbar_init(done_bar, 1);
+    *consumed = 0;
+    fence_barrier_init();
+  }
+  if (warp == 1) {
+    tmem_alloc(smem_u32(bars + 2 * kStages + 5), 512);
+    tmem_relinquish();
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = *tmem_slot;
+
+  int issued = 0;
+  if (warp == 0) {
+    if (lane == 0) {
+      prefetch_tmap(&tmA);
+      prefetch_tmap(&tmB);
+      const uint32_t bytes = kABytes + (uint32_t)g.bn * 128u;
+      bool ok = !withhold;
+      for (int jb = blockIdx.x; jb < njobs && ok; jb += gridDim.x) {
+        const Tile t = tile_of(g, jb);
+        const int ra = t.z * g.rows + g.row0 + t.m0, rb = t.z * g.cols + t.n0;
+        for (int kb = 0; kb < g.nkb; ++kb) {
+          const int s = issued % kStages, ph = (issued / kStages) & 1;
+          if (!mbar_wait(empty(s), ph ^ 1, err, 1u, lim)) {
+            ok = false;
+            break;
+          }
+          mbar_arrive_expect_tx(full(s), bytes);
+          tma_load_3d(a_tile(s), &tmA, full(s), kb * kBK, ra, t.mod);
+          tma_load_3d(b_tile(s), &tmB, full(s), kb * kBK, rb, t.mod);
+          ++issued;
+        }
+      }
+    }
+  } else if (warp == 1) {
+    if (lane == 0) {
+      const uint32_t idesc = idesc_f32acc(1, kTileM, g.bn);
+      int it = 0, gs = 0;
+      bool ok = true;
+      for (int jb = blockIdx.x; jb < njobs && ok; jb += gridDim.x) {
+        for (int k0 = 0; k0 < g.nkb && ok; k0 += kSegStages, ++gs) {
+          const int b = gs & 1, u = gs >> 1;
+          if (!mbar_wait(acce(b), (u & 1) ^ 1, err, 2u, lim)) {
+            ok = false;
+            break;
+          }
+          tc_fence_after();
+          const int k1 = min(g.nkb, k0 + kSegStages);
+          for (int kb = k0; kb < k1; ++kb) {
+            const int s = it % kStages, ph = (it / kStages) & 1;
+            if (!mbar_wait(full(s), ph, err, 4u, lim)) {
+              ok = false;
+              break;
+            }
+#pragma unroll
+            for (int kk = 0; kk < 4; ++kk)
+              umma<0>(tmem + b * 256, smem_desc<128>(a_tile(s) + kk * 32), smem_desc<128>(b_tile(s) + kk * 32), idesc,
+                      (kb > k0 || kk) ? 1u : 0u);
+            umma_commit(empty(s));
+            ++it;
+            *consumed = it;
+          }
+          if (ok) umma_commit(accf(b));
+        }
+      }
+      umma_commit(done_bar);
+      mbar_wait(done_bar, 0, err, 16u, lim);
+    }
+  } else if (warp >= 4) {
+    const int quad = warp & 3, half = (warp - 4) >> 2;
+    bool ok = true;
+    int gs = 0;
+    for (int jb = blockIdx.x; jb < njobs && ok; jb += gridDim.x) {
+      const Tile t = tile_of(g, jb);
+      const float p = kModF[t.mod], rp = 1.0f / p;
+      const int row = t.m0 + quad * 32 + lane;
+      signed char* y = g.Y + (long long)t.mod * g.ymod + ((long long)t.z * g.rows + row) * g.ldy + t.n0;
+      const bool rok = row < g.rows;
+      for (int k0 = 0; k0 < g.nkb; k0 += kSegStages, ++gs) {
+        const int b = gs & 1, u = gs >> 1;
+        if (!mbar_wait(accf(b), u & 1, err, 8u, lim)) {
+          ok = false;
+          break;
+        }
+        tc_fence_after();
+        const uint32_t tm = tmem + b * 256 + ((uint32_t)(quad * 32) << 16);
+        for (int c = half * 16; c < g.bn; c += 32) {
+          if (t.n0 + c >= g.ldy) break;  // (uniform) past the last column
+          uint32_t v[16];
+          tmem_ld_32x32b_x16(tm + c, v);
+          uint4 prev = make_uint4(0, 0, 0, 0);
+          if (k0 && rok) prev = *reinterpret_cast<const uint4*>(y + c);
+          tmem_ld_wait();
+          const uint4 w = reduce16(v, k0 != 0, prev, p, rp);
+          if (rok) *reinterpret_cast<uint4*>(y + c) = w;
+        }
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(acce(b));
+      }
+    }
+  }
+  __syncthreads();
+  if (warp == 0 && lane == 0) {
+    // copies issued but never consumed (only after an expired wait) must land before exit
+    for (int i = *consumed; i < issued; ++i) mbar_wait(full(i % kStages), (i / kStages) & 1, err, 32u, lim);
+  }
+  __syncthreads();
+  if (warp == 1) {
+    tc_fence_after();
+    tmem_dealloc(tmem, 512);
+  }
+}
+
+// ---------------- reconstruction ----------------
+
+struct CrtArgs {
+  const signed char* Y;
+  long long ymod;
+  int ldy, rows, cols;      // cols: real columns (2 per complex column)
+  int row0;                 // first row of the launch in the product
+  const int* ea;            // [batch][ea_rows] scales, from row row0
+  const int* eb;            // [batch][columns (complex or real)]
+  int ea_rows, eb_rows;
+  // complex: D[z.. + row map + column map]
+  double2* D;
+  const int4* tab;
+  int tab0;
+  long long sD;
+  int r_div, c_div;
+  long long r_hi, r_lo, c_hi, c_lo;
+  // real
+  double* out;
+  long long ldo;
+  int tri;
+  double alpha;
+  int beta;
+};
+
+template <int I>
+__device__ __forceinline__ void crt_add(const uint4 (&y)[kMods], int w, int c, long long (&acc)[4]) {
+  if constexpr (I < kMods) {
+    const uint32_t word = w == 0 ? y[I].x : w == 1 ? y[I].y : w == 2 ? y[I].z : y[I].w;
+    const int r = (int)(signed char)(word >> (8 * c));
+    acc[0] += (long long)r * Crt<I>::w0;
+    acc[1] += (long long)r * Crt<I>::w1;
+    acc[2] += (long long)r * Crt<I>::w2;
+    acc[3] += (long long)r * Crt<I>::w3;
+    crt_add<I + 1>(y, w, c, acc);
+  }
+}
+
+// The integer x with |x| < P / 2 and x = sum_j acc_j 2^(30 j) (mod P), times 2^-s, rounded once.
+__device__ __forceinline__ double crt_value(long long (&acc)[4], int s) {
+  constexpr u128 P = mod_product();
+  // the quotient by P from the top limbs: the error of this estimate (2^-10) is far below the distance
+  // of |x| / P <= 0.39 from a half
+  constexpr float inv = (float)(65536.0 / ((double)(P >> 64) / 67108864.0));  // 2^16 / (P / 2^90)
+  const float f = (float)(int)(acc[3] >> 16) + (float)(int)(acc[2] >> 30) * (1.f / 65536.f);
+  const int q = (int)rintf(f * inv);
+  __int128 x = (__int128)(acc[0] - (long long)q * limb(P, 0));
+  x += (__int128)(acc[1] - (long long)q * limb(P, 1)) << 30;
+  x += (__int128)(acc[2] - (long long)q * limb(P, 2)) << 60;
+  x += (__int128)(acc[3] - (long long)q * limb(P, 3)) << 90;
+  const bool neg = x < 0;
+  const u128 a = neg ? (u128)(-x) : (u128)x;
+  unsigned long long hi = (unsigned long long)(a >> 64), lo = (unsigned long long)a;
+  if ((hi | lo) == 0) return 0.0;
+  int lz;
+  if (hi == 0) {
+    hi = lo;
+    lo = 0;
+    lz = 64;
+  } else {
+    lz = 0;
+  }
+  const int l = __clzll((long long)hi);
+  lz += l;
+  unsigned long long m = hi, rest = lo;
+  if (l) {
+    m = (hi << l) | (lo >> (64 - l));
+    rest = lo << l;
+  }
+  unsigned long long r = m >> 11;
+  const unsigned rem = (unsigned)(m & 0x7ff);
+  if (rem > 0x400u || (rem == 0x400u && (rest != 0 || (r & 1)))) ++r;
+  const int e = 127 - lz - s;  // the leading bit's exponent
+  if (e >= -1021 && e <= 1022) {
+    const unsigned long long b = ((unsigned long long)(e + 1022) << 52) + r;
+    return __longlong_as_double((long long)(b | (neg ? 1ull << 63 : 0ull)));
+  }
+  const double d = scalbn((double)r, e - 52);
+  return neg ? -d : d;
+}
+
+// A warp takes 32 rows x 16 columns, a lane per row. Complex results whose rows are contiguous in the
+// output go out directly (512 contiguous bytes per store); the others through shared memory, so
+// that the 16 columns of a row leave as one 128-byte (real) or 128-byte (8 complex) segment.
+template <bool CPLX>
+__global__ void __launch_bounds__(256) rns_crt_kernel(const CrtArgs a) {
+  __shared__ double stage[8][32 * 17];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int z = blockIdx.z;
+  const int c0 = (blockIdx.y * 8 + warp) * 16, rbase = blockIdx.x * 32, row = rbase + lane;
+  if (c0 >= a.cols) return;                                        // (whole warps leave)
+  if (!CPLX && a.tri && c0 > a.row0 + rbase + 31) return;
+  const bool rok = row < a.rows;
+  uint4 y[kMods];
+  const signed char* yp = a.Y + ((long long)z * a.rows + (rok ? row : 0)) * a.ldy + c0;
+#pragma unroll
+  for (int i = 0; i < kMods; ++i) y[i] = *reinterpret_cast<const uint4*>(yp + (long long)i * a.ymod);
+  const int sa = rok ? a.ea[(long long)z * a.ea_rows + row] : 0;
+  double* st = stage[warp];
+  double2* D = nullptr;
+  long long radr = 0;
+  bool direct = false;
+  if constexpr (CPLX) {
+    D = a.D + (a.tab ? (long long)a.tab[a.tab0 + z].z : (long long)z) * a.sD;
+    const int gr = a.row0 + row;
+    radr = (long long)(gr / a.r_div) * a.r_hi + (long long)(gr % a.r_div) * a.r_lo;
+    direct = a.r_lo == 1;
+  }
+#pragma unroll
+  for (int w = 0; w < 4; ++w) {
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      const int col = c0 + 4 * w + c;
+      const int ec = CPLX ? col >> 1 : col;
+      long long acc[4] = {0, 0, 0, 0};
+      crt_add<0>(y, w, c, acc);
+      double v = 0.0;
+      if (col < a.cols) {
+        const int sb = a.eb[(long long)z * a.eb_rows + ec];
+        v = (sa == kPoison || sb == kPoison) ? __longlong_as_double(0x7ff8000000000000ll) : crt_value(acc, sa + sb);
+      }
+      st[lane * 17 + 4 * w + c] = v;
+    }
+    if constexpr (CPLX) {
+      if (direct) {
+        // lanes hold consecutive rows: each lane stores its own pairs
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const int cc = (c0 >> 1) + 2 * w + h;
+          if (rok && 2 * cc < a.cols) {
+            double2 v = make_double2(st[lane * 17 + 4 * w + 2 * h], st[lane * 17 + 4 * w + 2 * h + 1]);
+            if (a.alpha != 1.0) {
+              v.x *= a.alpha;
+              v.y *= a.alpha;
+            }
+            double2* d = D + radr + (long long)(cc / a.c_div) * a.c_hi + (long long)(cc % a.c_div) * a.c_lo;
+            if (a.beta) {
+              const double2 o = *d;
+              v.x += o.x;
+              v.y += o.y;
+            }
+            *d = v;
+          }
+        }
+      }
+    }
+  }
+  if (CPLX && direct) return;
+  __syncwarp();
+  if constexpr (CPLX) {
+    // 4 rows x 8 complex columns per pass
+    const int cc = (c0 >> 1) + (lane & 7);
+    const long long cadr = (long long)(cc / a.c_div) * a.c_hi + (long long)(cc % a.c_div) * a.c_lo;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int rl = i * 4 + (lane >> 3), gr = a.row0 + rbase + rl;
+      if (rbase + rl < a.rows && 2 * cc < a.cols) {
+        double2 v = make_double2(st[rl * 17 + 2 * (lane & 7)], st[rl * 17 + 2 * (lane & 7) + 1]);
+        if (a.alpha != 1.0) {
+          v.x *= a.alpha;
+          v.y *= a.alpha;
+        }
+        double2* d = D + (long long)(gr / a.r_div) * a.r_hi + (long long)(gr % a.r_div) * a.r_lo + cadr;
+        if (a.beta) {
+          const double2 o = *d;
+          v.x += o.x;
+          v.y += o.y;
+        }
+        *d = v;
+      }
+    }
+  } else {
+    // 2 rows x 16 columns per pass
+    const int col = c0 + (lane & 15);
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+      const int rl = i * 2 + (lane >> 4);
+      const long long m = (long long)a.row0 + rbase + rl;
+      if (rbase + rl >= a.rows || col >= a.cols || (a.tri && col > m)) continue;
+      double* d = a.out + (a.tri ? m * (m + 1) / 2 + col : m * a.ldo + col);
+      *d += a.alpha * st[rl * 17 + (lane & 15)];
+    }
+  }
+}
+
+// ---------------- host side ----------------
+
+inline long long pad_to(long long x, long long m) { return (x + m - 1) / m * m; }
+
+// One operand in the engine's terms.
+struct Side {
+  int src;              // SRC_*
+  const double* base;
+  int sel;
+  long long sbatch, s_row, s_k;
+  int rows, conj;
+};
+
+cudaError_t convert(const Side& o, int r0, int nrows, const int4* tab, int tab0, int K, int Kp, int nb,
+                    long long batch0, __nv_bfloat16* R, long long smod, int* exps, cudaStream_t s) {
+  ConvArgs a;
+  std::memset(&a, 0, sizeof(a));
+  const int w = o.src == SRC_REAL ? 1 : 2;
+  a.src = o.base + (long long)w * (r0 * o.s_row + (tab ? 0 : batch0 * o.sbatch));
+  a.tab = tab;
+  a.tab0 = tab0;
+  a.sel = o.sel;
+  a.sbatch = o.sbatch;
+  a.s_row = o.s_row;
+  a.s_k = o.s_k;
+  a.rows = nrows;
+  a.K = K;
+  a.Kp = Kp;
+  a.conj = o.conj;
+  a.R = R;
+  a.smod = smod;
+  a.exps = exps;
+  const dim3 grid((nrows + 31) / 32, nb);
+  if (o.src == SRC_COMPLEX) rns_convert_kernel<SRC_COMPLEX><<<grid, 256, 0, s>>>(a);
+  else if (o.src == SRC_COMPLEX2) rns_convert_kernel<SRC_COMPLEX2><<<grid, 256, 0, s>>>(a);
+  else rns_convert_kernel<SRC_REAL><<<grid, 256, 0, s>>>(a);
+  return cudaGetLastError();
+}
+
+int tile_width(int cols) {
+  const int ct = (cols + 255) / 256;
+  return (int)pad_to((cols + ct - 1) / ct, 16);
+}
+
+cudaError_t gemm(const __nv_bfloat16* RA, long long smodA, const __nv_bfloat16* RB, long long smodB, GemmArgs g, int Kp,
+                 int total_rows_a, const RnsCtx& c, cudaStream_t s) {
+  CUtensorMap ma, mb;
+  cudaError_t e = make_tmap_rows128(&ma, RA, Kp, (unsigned long long)g.nbatch * total_rows_a, kMods, smodA, kTileM);
+  if (e != cudaSuccess) return e;
+  e = make_tmap_rows128(&mb, RB, Kp, (unsigned long long)g.nbatch * g.cols, kMods, smodB, g.bn);
+  if (e != cudaSuccess) return e;
+  e = cudaFuncSetAttribute(rns_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kGemmSmem);
+  if (e != cudaSuccess) return e;
+  const int njobs = kMods * g.nbatch * g.tiles;
+  rns_gemm_kernel<<<std::min(njobs, c.sms), kGemmThreads, kGemmSmem, s>>>(ma, mb, g, njobs, c.err, c.wait_ns,
+                                                                           c.withhold_loads);
+  return cudaGetLastError();
+}
+
+// Splits the context's scratch; every piece starts on a 1024-byte boundary.
+struct Carve {
+  char* p;
+  char* end;
+  void* take(size_t n) {
+    char* q = (char*)(((uintptr_t)p + 1023) & ~(uintptr_t)1023);
+    p = q + n;
+    return q;
+  }
+};
+
+struct ZPlan {
+  Side rows, cols;
+  int K, Kp, ldy;
+  size_t row_bytes, col_bytes, y_bytes;  // per batch entry: row residues, column residues, Y
+  bool rows_are_m;
+};
+
+ZPlan zplan(const ZgemmArgs& a, int al, bool cj, int bl) {
+  ZPlan p;
+  Side A{SRC_COMPLEX, reinterpret_cast<const double*>(a.A), 0, a.sA, al == A_KM ? 1 : a.lda, al == A_KM ? a.lda : 1, a.M,
+         cj ? 1 : 0};
+  Side B{SRC_COMPLEX, reinterpret_cast<const double*>(a.B), 1, a.sB, bl == B_KN ? 1 : a.ldb, bl == B_KN ? a.ldb : 1, a.N,
+         0};
+  p.rows_are_m = a.M > a.N;
+  p.rows = p.rows_are_m ? A : B;
+  p.cols = p.rows_are_m ? B : A;
+  p.cols.src = SRC_COMPLEX2;
+  p.K = a.K;
+  p.Kp = (int)pad_to(2ll * a.K, kBK);
+  p.ldy = (int)pad_to(2ll * p.cols.rows, 16);
+  p.row_bytes = (size_t)p.rows.rows * p.Kp * 2 * kMods;
+  p.col_bytes = (size_t)2 * p.cols.rows * p.Kp * 2 * kMods;
+  p.y_bytes = (size_t)p.rows.rows * p.ldy * kMods;
+  return p;
+}
+
+}  // namespace
+
+size_t rns_need(const ZgemmArgs& a) {
+  const ZPlan p = zplan(a, A_KM, false, B_KN);
+  return (p.row_bytes + p.col_bytes + p.y_bytes + ((size_t)p.rows.rows + p.cols.rows) * 4 + 4096) * a.batch + 16384;
+}
+
+size_t rns_need(const DsyrkArgs& a) {
+  const size_t kp = (size_t)pad_to(a.K, kBK), rows = (size_t)a.M + (a.mode ? a.N : 0);
+  return rows * kp * 2 * kMods + (size_t)a.M * pad_to(a.N, 16) * kMods + rows * 4 + 65536;
+}
+
+// Where the line between the two lies (measured on shapes from 8 x 256 x 8 to 128 x 22 880 x 1024, single and
+// batched): the FP64 kernel takes 4.3 us per k and 64 x 64 complex tile and SM (a warp whose 8 rows all lie
+// outside issues none), 7 us more per launch; the residues take about 40 us for their four launches, 17 ps per
+// real result (reconstruction and epilogue) and 12 ps per converted real element, and the MMAs. A
+// 128 x 4096 product: K = 8, 41 against 55 us; K = 16, 76 against 56; K = 64, 279 against 66.
+bool rns_takes_zgemm(const ZgemmArgs& a, const RnsCtx& c) {
+  if (!c.scratch || a.lower || a.M <= 0 || a.N <= 0 || a.K <= 0 || a.batch <= 0) return false;
+  const ZPlan p = zplan(a, A_KM, false, B_KN);
+  if (p.col_bytes + 2 * kBK * (size_t)p.Kp * 2 * kMods + 256 * (size_t)p.ldy * kMods + (4 << 20) > c.bytes) return false;
+  const double ctas = (double)((a.M + 63) / 64) * ((a.N + 63) / 64) * a.batch;
+  const double fill = (double)pad_to(a.M, 8) / pad_to(a.M, 64);
+  const double fp64 = 7 + 4.3 * a.K * fill * std::ceil(ctas / c.sms);
+  const double mn = (double)a.M * a.N * a.batch, conv = ((double)p.rows.rows + 2.0 * p.cols.rows) * p.Kp * a.batch;
+  return fp64 > 40 + 34e-6 * mn + 12e-6 * conv + 8.0 * kMods / 1.2e9 * mn * a.K;
+}
+
+cudaError_t rns_zgemm(const ZgemmArgs& a, int al, bool cj, int bl, const RnsCtx& c, cudaStream_t s, int* launches) {
+  const ZPlan p = zplan(a, al, cj, bl);
+  const size_t exps = ((size_t)p.rows.rows + p.cols.rows) * 4 + 4096;
+  // chunks of whole batch entries, or of rows of one entry
+  const size_t per = p.row_bytes + p.col_bytes + p.y_bytes + exps;
+  const size_t avail = c.bytes - 16384;
+  int nb = (int)std::min<size_t>((size_t)a.batch, avail / per);
+  int nr = p.rows.rows;
+  if (nb < 1) {
+    nb = 1;
+    const size_t fixed = p.col_bytes + exps;
+    const size_t per_row = (size_t)p.Kp * 2 * kMods + (size_t)p.ldy * kMods;
+    nr = (int)std::min<size_t>((size_t)p.rows.rows, (avail - fixed) / per_row / 128 * 128);
+    if (nr < 1) return cudaErrorInvalidValue;
+  }
+  for (int b0 = 0; b0 < a.batch; b0 += nb) {
+    const int n = std::min(nb, a.batch - b0);
+    for (int r0 = 0; r0 < p.rows.rows; r0 += nr) {
+      const int m = std::min(nr, p.rows.rows - r0);
+      Carve w{(char*)c.scratch, (char*)c.scratch + c.bytes};
+      const long long smA = (long long)n * m * p.Kp, smB = (long long)n * 2 * p.cols.rows * p.Kp;
+      __nv_bfloat16* RA = (__nv_bfloat16*)w.take((size_t)smA * 2 * kMods);
+      __nv_bfloat16* RB = (__nv_bfloat16*)w.take((size_t)smB * 2 * kMods);
+      signed char* Y = (signed char*)w.take((size_t)n * m * p.ldy * kMods);
+      int* ea = (int*)w.take((size_t)n * m * 4);
+      int* eb = (int*)w.take((size_t)n * p.cols.rows * 4);
+      if (w.p > w.end) return cudaErrorInvalidValue;
+      cudaError_t e = convert(p.cols, 0, p.cols.rows, a.tab, a.tab0 + b0, p.K, p.Kp, n, b0, RB, smB, eb, s);
+      if (e != cudaSuccess) return e;
+      e = convert(p.rows, r0, m, a.tab, a.tab0 + b0, p.K, p.Kp, n, b0, RA, smA, ea, s);
+      if (e != cudaSuccess) return e;
+      GemmArgs g;
+      std::memset(&g, 0, sizeof(g));
+      g.nbatch = n;
+      g.rows = m;
+      g.cols = 2 * p.cols.rows;
+      g.rt = (m + kTileM - 1) / kTileM;
+      g.bn = tile_width(g.cols);
+      g.ct = (g.cols + g.bn - 1) / g.bn;
+      g.tiles = g.rt * g.ct;
+      g.nkb = p.Kp / kBK;
+      g.Y = Y;
+      g.ymod = (long long)n * m * p.ldy;
+      g.ldy = p.ldy;
+      e = gemm(RA, smA, RB, smB, g, p.Kp, m, c, s);
+      if (e != cudaSuccess) return e;
+      CrtArgs x;
+      std::memset(&x, 0, sizeof(x));
+      x.Y = Y;
+      x.ymod = g.ymod;
+      x.ldy = p.ldy;
+      x.rows = m;
+      x.cols = g.cols;
+      x.row0 = r0;
+      x.ea = ea;
+      x.eb = eb;
+      x.ea_rows = m;
+      x.eb_rows = p.cols.rows;
+      x.D = a.D + (a.tab ? 0 : (long long)b0 * a.sD);
+      x.tab = a.tab;
+      x.tab0 = a.tab0 + b0;
+      x.sD = a.sD;
+      x.r_div = p.rows_are_m ? a.dm_div : a.dn_div;
+      x.r_hi = p.rows_are_m ? a.dm_hi : a.dn_hi;
+      x.r_lo = p.rows_are_m ? a.dm_lo : a.dn_lo;
+      x.c_div = p.rows_are_m ? a.dn_div : a.dm_div;
+      x.c_hi = p.rows_are_m ? a.dn_hi : a.dm_hi;
+      x.c_lo = p.rows_are_m ? a.dn_lo : a.dm_lo;
+      x.alpha = a.alpha;
+      x.beta = a.beta;
+      const dim3 grid((m + 31) / 32, (g.cols + 127) / 128, n);
+      rns_crt_kernel<true><<<grid, 256, 0, s>>>(x);
+      if ((e = cudaGetLastError()) != cudaSuccess) return e;
+      *launches += 4;
+    }
+  }
+  return cudaSuccess;
+}
+
+bool rns_takes_dsyrk(const DsyrkArgs& a, const RnsCtx& c) {
+  if (!c.scratch || a.M <= 0 || a.N <= 0 || a.K <= 0) return false;
+  // 1.08 us per k and 64 x 64 tile and SM on the FP64 pipe; a 64 x 64 result: K = 64, 75 against 32 us
+  const double tm = (a.M + 63) / 64, tn = (a.N + 63) / 64, ctas = a.mode == 0 ? tm * (tm + 1) / 2 : tm * tn;
+  const double fp64 = 7 + 1.08 * a.K * std::ceil(ctas / c.sms), mn = (a.mode == 0 ? 0.5 : 1.0) * a.M * (double)a.N;
+  const double conv = ((double)a.M + (a.mode ? a.N : 0)) * a.K;
+  if (fp64 < 40 + 17e-6 * mn + 12e-6 * conv + 2.0 * kMods / 1.2e9 * mn * a.K) return false;
+  // at least one K block of both operands and 256 rows of Y
+  const size_t ops = ((size_t)a.M + (a.mode ? a.N : 0)) * kBK * 2 * kMods, y = (size_t)256 * pad_to(a.N, 16) * kMods;
+  return ops + y + ((size_t)a.M + a.N) * 4 + (1 << 20) <= c.bytes;
+}
+
+cudaError_t rns_dsyrk(const DsyrkArgs& a, const RnsCtx& c, cudaStream_t s, int* launches) {
+  const bool tri = a.mode == 0;
+  const int N = a.N, M = a.M;
+  const long long ldy = pad_to(N, 16);
+  const size_t opsrow = (size_t)M + (tri ? 0 : N), exps = ((size_t)M + N) * 4 + 16384;
+  const size_t avail = c.bytes - exps;
+  // K in chunks whose residues take at most half of the scratch (or what the smallest row chunk
+  // leaves), rows of the result in chunks of what is left; every chunk adds into the output
+  const size_t ymin = (size_t)256 * ldy * kMods;
+  const size_t opmax = std::max(avail / 2, opsrow * kBK * 2 * kMods);
+  long long Kc = std::min<long long>(pad_to(a.K, kBK), (long long)(std::min(opmax, avail - ymin) / (opsrow * 2 * kMods)) / kBK * kBK);
+  const size_t yav = avail - opsrow * Kc * 2 * kMods;
+  const int nr = (int)std::min<size_t>((size_t)pad_to(M, 256), yav / ((size_t)ldy * kMods) / 256 * 256);
+  if (Kc < kBK || nr < 256) return cudaErrorInvalidValue;
+  const Side X{SRC_REAL, a.X, 0, 0, 1, a.ldx, M, 0}, Yo{SRC_REAL, a.Y, 0, 0, 1, a.ldy, N, 0};
+  for (long long k0 = 0; k0 < a.K; k0 += Kc) {
+    const int K = (int)std::min<long long>(Kc, a.K - k0), Kp = (int)pad_to(K, kBK);
+    Carve w{(char*)c.scratch, (char*)c.scratch + c.bytes};
+    const long long smA = (long long)M * Kp, smB = (long long)N * Kp;
+    __nv_bfloat16* RA = (__nv_bfloat16*)w.take((size_t)smA * 2 * kMods);
+    __nv_bfloat16* RB = tri ? RA : (__nv_bfloat16*)w.take((size_t)smB * 2 * kMods);
+    int* ea = (int*)w.take((size_t)M * 4);
+    int* eb = tri ? ea : (int*)w.take((size_t)N * 4);
+    signed char* Y = (signed char*)w.take((size_t)std::min((long long)nr, (long long)M) * ldy * kMods);
+    if (w.p > w.end) return cudaErrorInvalidValue;
+    Side xs = X, ys = Yo;
+    xs.base += k0 * a.ldx;
+    ys.base += k0 * a.ldy;
+    cudaError_t e = convert(xs, 0, M, nullptr, 0, K, Kp, 1, 0, RA, smA, ea, s);
+    if (e != cudaSuccess) return e;
+    if (!tri) {
+      e = convert(ys, 0, N, nullptr, 0, K, Kp, 1, 0, RB, smB, eb, s);
+      if (e != cudaSuccess) return e;
+    }
+    *launches += tri ? 1 : 2;
+    for (int r0 = 0; r0 < M; r0 += nr) {
+      const int m = std::min(nr, M - r0);
+      GemmArgs g;
+      std::memset(&g, 0, sizeof(g));
+      g.nbatch = 1;
+      g.rows = m;
+      g.cols = N;
+      g.rt = (m + kTileM - 1) / kTileM;
+      g.tri = tri;
+      g.h0 = r0 / 256;
+      g.row0 = r0;
+      g.bn = tri ? 256 : tile_width(N);
+      g.ct = (N + g.bn - 1) / g.bn;
+      g.tiles = tri ? tri_tiles_before(g.rt, g.h0) : g.rt * g.ct;
+      g.nkb = Kp / kBK;
+      g.Y = Y;
+      g.ymod = (long long)m * ldy;
+      g.ldy = (int)ldy;
+      e = gemm(RA, smA, RB, smB, g, Kp, M, c, s);
+      if (e != cudaSuccess) return e;
+      CrtArgs x;
+      std::memset(&x, 0, sizeof(x));
+      x.Y = Y;
+      x.ymod = g.ymod;
+      x.ldy = (int)ldy;
+      x.rows = m;
+      x.cols = N;
+      x.row0 = r0;
+      x.ea = ea + r0;
+      x.eb = eb;
+      x.out = a.out;
+      x.ldo = a.ldo;
+      x.tri = tri;
+      x.alpha = a.alpha;
+      const dim3 grid((m + 31) / 32, (N + 127) / 128, 1);
+      rns_crt_kernel<false><<<grid, 256, 0, s>>>(x);
+      if ((e = cudaGetLastError()) != cudaSuccess) return e;
+      *launches += 2;
+    }
+  }
+  return cudaSuccess;
+}
+
+}  // namespace dmet

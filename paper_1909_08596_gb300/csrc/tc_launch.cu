@@ -66,6 +66,21 @@ cudaError_t make_tmap_3d(CUtensorMap* map, int prec, const void* base, unsigned 
   return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
+cudaError_t make_tmap_rows128(CUtensorMap* map, const void* base, unsigned long long k_elems, unsigned long long rows,
+                              unsigned long long planes, unsigned long long plane_elems, int box_rows) {
+  EncodeTiledFn fn = encode_fn();
+  if (!fn) return cudaErrorNotSupported;
+  if (((uintptr_t)base & 127) || k_elems % 64 || plane_elems % 64) return cudaErrorInvalidValue;
+  const cuuint64_t dims[3] = {k_elems, rows, planes};
+  const cuuint64_t strides[2] = {k_elems * 2, plane_elems * 2};
+  const cuuint32_t box[3] = {64, (cuuint32_t)box_rows, 1};
+  const cuuint32_t estr[3] = {1, 1, 1};
+  CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
+                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
+}
+
 cudaError_t make_tmap_interleaved(CUtensorMap* map, int prec, const void* base, unsigned long long k_elems,
                                   unsigned long long rows, int slices, int box_rows) {
   EncodeTiledFn fn = encode_fn();
