@@ -20,8 +20,8 @@
 //   2. rns_gemm_kernel: tcgen05 (128 x up to 256 tiles, TMA-fed), one job per (modulus, batch, tile).
 //      After every kSegStages K blocks the FP32 sums, exact below 2^24, are reduced modulo p and the
 //      running residue is kept as one byte per element in Y [mod][batch][row][col].
-//   3. rns_crt_kernel: recovers the signed 117-bit integer, rounds it once to FP64, undoes the scales
-//      and writes the caller's layout.
+//   3. rns_crt_kernel: recovers the signed 117-bit integer as a 64-bit fraction of P, rounds it to FP64, undoes the
+//      scales and writes the caller's layout.
 //
 // A row with an infinity or a NaN gives NaN in every result it enters.
 
@@ -57,16 +57,31 @@ __host__ __device__ constexpr u128 mod_product() {
   for (int i = 0; i < kMods; ++i) p *= (u128)mod_of(i);
   return p;
 }
-// W_i = (P / p_i) * ((P / p_i)^-1 mod p_i): sum r_i W_i = x (mod P) for the residues r_i of x.
-__host__ __device__ constexpr u128 crt_weight(int i) {
-  const u128 m = mod_product() / (u128)mod_of(i);
-  const int p = mod_of(i), a = (int)(m % (u128)p);
+// x / P = sum r_i c_i (mod 1) for the residues r_i of x, with c_i = ((P / p_i)^-1 mod p_i) / p_i, as fixed-point
+// fractions of 72 bits in words of 32, 20 and 20 bits: a byte times a 20-bit word, kMods times, fits 32 bits, so
+// a residue adds with three 32-bit multiply-adds (the top word wraps: modulo 1).
+constexpr int kLimb = 20, kFrac = 32 + 2 * kLimb;
+static_assert(255 * kMods + 1 <= 1 << (32 - kLimb), "the 20-bit words' sums");
+__host__ __device__ constexpr int crt_inverse(int i) {
+  const int p = mod_of(i), a = (int)((mod_product() / (u128)p) % (u128)p);
   int inv = 1;
   while ((a * inv) % p != 1) ++inv;
-  return m * (u128)inv;
+  return inv;
 }
-// 30-bit limbs, so that a residue times a limb is a signed 32 x 32 -> 64-bit multiply-add
-__host__ __device__ constexpr int limb(u128 x, int j) { return (int)((x >> (30 * j)) & (u128)0x3fffffff); }
+__host__ __device__ constexpr u128 crt_fraction(int i) {
+  const u128 p = (u128)mod_of(i);
+  return (((u128)crt_inverse(i) << kFrac) + p / 2) / p;
+}
+// Minus the sum's offset for residues stored with 128 added (mod 1), plus half of the last bit that crt_fold keeps.
+__host__ __device__ constexpr u128 crt_offset() {
+  u128 t = 0;
+  for (int i = 0; i < kMods; ++i) t += 128 * crt_fraction(i);
+  t = ((u128)1 << (kFrac + 16)) - t + ((u128)1 << (kFrac - 65));
+  return t & (((u128)1 << kFrac) - 1);
+}
+__host__ __device__ constexpr unsigned frac_word(u128 x, int j) {
+  return j == 2 ? (unsigned)(x >> (2 * kLimb)) : (unsigned)(x >> (j * kLimb)) & ((1u << kLimb) - 1);
+}
 
 constexpr bool mods_ok() {
   for (int i = 0; i < kMods; ++i)
@@ -83,13 +98,7 @@ constexpr bool mods_ok() {
 }
 static_assert(mods_ok(), "the moduli must be pairwise coprime");
 static_assert((mod_product() >> (2 * kBeta + 1)) != 0, "P must exceed 2 * 2^(2 kBeta)");
-static_assert((mod_product() >> 120) == 0, "four 30-bit limbs must hold P");
-
-template <int I>
-struct Crt {
-  static constexpr u128 W = crt_weight(I);
-  static constexpr int w0 = limb(W, 0), w1 = limb(W, 1), w2 = limb(W, 2), w3 = limb(W, 3);
-};
+static_assert((mod_product() >> 117) == 1, "P in [2^117, 2^118)");
 
 // Symmetric residue of 2^(16 j) modulo p.
 __host__ __device__ constexpr int chunk_weight(int i, int j) {
@@ -99,7 +108,7 @@ __host__ __device__ constexpr int chunk_weight(int i, int j) {
   return r > p / 2 ? r - p : r;
 }
 
-constexpr int kPoison = INT_MIN;  // scale of a row that holds an infinity or a NaN
+constexpr int kPoison = -(1 << 28);  // scale of a row that holds an infinity or a NaN
 constexpr float kMagic = 12582912.f;  // 1.5 * 2^23: adding it rounds to an integer
 
 // v - p * rint(v / p) for an integer |v| <= 2^24: a residue with |r| <= (p + 1) / 2 (the rounding of v / p
@@ -220,16 +229,18 @@ __device__ __forceinline__ void store_residues(const float (&cr)[4], const float
   }
 }
 
-// One CTA converts 32 operand rows: first their norms, then the residues, 32 (re, im) or
-// (k, k + 1) pairs at a time, a lane per pair, so that every store of a warp is 128 contiguous bytes.
-// Rows that are contiguous in memory (s_row = 1) pass through a transpose in shared memory.
-template <int SRC>
+// One CTA converts RB operand rows (32, or 8 where that would leave SMs idle): first their norms, then the
+// residues, 32 (re, im) or (k, k + 1) pairs at a time, a lane per pair, so that every store of a warp is 128
+// contiguous bytes. Rows that are contiguous in memory (s_row = 1) pass through a transpose in shared memory.
+template <int SRC, int RB>
 __global__ void __launch_bounds__(256) rns_convert_kernel(const ConvArgs a) {
-  __shared__ double2 tile[32][33];
-  __shared__ float sh_s[8][32];
-  __shared__ int sh_e[8][32], sh_bad[8][32], sh_scale[32];
+  constexpr int KL = 256 / RB, RW = RB / 8;  // k lanes per row, rows per warp
+  __shared__ double2 tile[32][RB + 1];
+  __shared__ float sh_s[KL][RB];
+  __shared__ int sh_e[KL][RB], sh_bad[KL][RB], sh_scale[RB];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int z = blockIdx.y, r0 = blockIdx.x * 32;
+  const int trow = threadIdx.x % RB, tk = threadIdx.x / RB;
+  const int z = blockIdx.y, r0 = blockIdx.x * RB;
   long long off = (long long)z * a.sbatch;
   int K = a.K;
   if (a.tab) {
@@ -244,28 +255,28 @@ __global__ void __launch_bounds__(256) rns_convert_kernel(const ConvArgs a) {
   // norms
   if (rowfast) {
     RowNorm n{0.f, 0, 0};
-    if (r0 + lane < a.rows) {
-      for (int k = warp; k < K; k += 8) {
+    if (r0 + trow < a.rows) {
+      for (int k = tk; k < K; k += KL) {
         if constexpr (SRC == SRC_REAL) {
-          norm_add(n, src1[(r0 + lane) + (long long)k * a.s_k]);
+          norm_add(n, src1[(r0 + trow) + (long long)k * a.s_k]);
         } else {
-          const double2 v = src2[(r0 + lane) + (long long)k * a.s_k];
+          const double2 v = src2[(r0 + trow) + (long long)k * a.s_k];
           norm_add(n, v.x);
           norm_add(n, v.y);
         }
       }
     }
-    sh_s[warp][lane] = n.s;
-    sh_e[warp][lane] = n.e;
-    sh_bad[warp][lane] = n.bad;
+    sh_s[tk][trow] = n.s;
+    sh_e[tk][trow] = n.e;
+    sh_bad[tk][trow] = n.bad;
     __syncthreads();
-    if (warp == 0) {
-      for (int w = 1; w < 8; ++w) norm_merge(n, sh_s[w][lane], sh_e[w][lane], sh_bad[w][lane]);
-      sh_scale[lane] = norm_scale(n);
+    if (tk == 0) {
+      for (int w = 1; w < KL; ++w) norm_merge(n, sh_s[w][trow], sh_e[w][trow], sh_bad[w][trow]);
+      sh_scale[trow] = norm_scale(n);
     }
   } else {
-    for (int i = 0; i < 4; ++i) {
-      const int r = r0 + warp * 4 + i;
+    for (int i = 0; i < RW; ++i) {
+      const int r = r0 + warp * RW + i;
       RowNorm n{0.f, 0, 0};
       if (r < a.rows) {
         for (int k = lane; k < K; k += 32) {
@@ -278,17 +289,17 @@ __global__ void __launch_bounds__(256) rns_convert_kernel(const ConvArgs a) {
           }
         }
       }
+      const int e = __reduce_max_sync(0xffffffffu, n.e), d = n.e - e;
+      n.s = d > -60 ? n.s * pow2f(2 * d) : 0.f;
+      n.e = e;
+      n.bad = __any_sync(0xffffffffu, n.bad);
 #pragma unroll
-      for (int o = 16; o; o >>= 1) {
-        const float s = __shfl_xor_sync(0xffffffffu, n.s, o);
-        const int e = __shfl_xor_sync(0xffffffffu, n.e, o), b = __shfl_xor_sync(0xffffffffu, n.bad, o);
-        norm_merge(n, s, e, b);
-      }
-      if (lane == 0) sh_scale[warp * 4 + i] = norm_scale(n);
+      for (int o = 16; o; o >>= 1) n.s += __shfl_xor_sync(0xffffffffu, n.s, o);
+      if (lane == 0) sh_scale[warp * RW + i] = norm_scale(n);
     }
   }
   __syncthreads();
-  if (warp == 0 && r0 + lane < a.rows) a.exps[(long long)z * a.rows + r0 + lane] = sh_scale[lane];
+  if (threadIdx.x < RB && r0 + trow < a.rows) a.exps[(long long)z * a.rows + r0 + trow] = sh_scale[trow];
 
   constexpr int RR = SRC == SRC_COMPLEX2 ? 2 : 1;
   const int units = SRC == SRC_REAL ? (K + 1) / 2 : K, upad = a.Kp / 2;
@@ -296,24 +307,24 @@ __global__ void __launch_bounds__(256) rns_convert_kernel(const ConvArgs a) {
     if (rowfast) {
       __syncthreads();
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const int ul = warp * 4 + i, u = u0 + ul;
+      for (int ul = tk; ul < 32; ul += KL) {
+        const int u = u0 + ul;
         double2 v = make_double2(0.0, 0.0);
-        if (u < units && r0 + lane < a.rows) {
+        if (u < units && r0 + trow < a.rows) {
           if constexpr (SRC == SRC_REAL) {
-            v.x = src1[(r0 + lane) + (long long)(2 * u) * a.s_k];
-            if (2 * u + 1 < K) v.y = src1[(r0 + lane) + (long long)(2 * u + 1) * a.s_k];
+            v.x = src1[(r0 + trow) + (long long)(2 * u) * a.s_k];
+            if (2 * u + 1 < K) v.y = src1[(r0 + trow) + (long long)(2 * u + 1) * a.s_k];
           } else {
-            v = src2[(r0 + lane) + (long long)u * a.s_k];
+            v = src2[(r0 + trow) + (long long)u * a.s_k];
           }
         }
-        tile[ul][lane] = v;
+        tile[ul][trow] = v;
       }
       __syncthreads();
     }
     const int u = u0 + lane;
-    for (int i = 0; i < 4; ++i) {
-      const int rl = warp * 4 + i, r = r0 + rl;
+    for (int i = 0; i < RW; ++i) {
+      const int rl = warp * RW + i, r = r0 + rl;
       if (r >= a.rows) break;
       double2 v = make_double2(0.0, 0.0);
       if (rowfast) {
@@ -588,155 +599,159 @@ struct CrtArgs {
   long long ldo;
   int tri;
   double alpha;
+  int scaled;               // alpha != 1 (tested as an integer: the FP64 pipe is slow)
   int beta;
 };
 
+struct Frac {
+  unsigned w[3];  // low, middle, top word
+};
+__device__ __forceinline__ Frac frac_start() {
+  constexpr u128 off = crt_offset();
+  return Frac{{frac_word(off, 0), frac_word(off, 1), frac_word(off, 2)}};
+}
+// u = residue + 128
+__device__ __forceinline__ void frac_add(Frac& f, unsigned u, unsigned c0, unsigned c1, unsigned c2) {
+  f.w[0] += u * c0;
+  f.w[1] += u * c1;
+  f.w[2] += u * c2;
+}
+__device__ __forceinline__ unsigned long long frac_fold(const Frac& f) {
+  constexpr unsigned mask = (1u << kLimb) - 1;
+  const unsigned m = f.w[1] + (f.w[0] >> kLimb), t = f.w[2] + (m >> kLimb);
+  return ((unsigned long long)t << 32) | ((m & mask) << (32 - kLimb)) | ((f.w[0] & mask) >> (2 * kLimb - 32));
+}
+
 template <int I>
-__device__ __forceinline__ void crt_add(const uint4 (&y)[kMods], int w, int c, long long (&acc)[4]) {
+__device__ __forceinline__ void crt_add(const uint2 (&y)[kMods], int w, int c, Frac& f) {
   if constexpr (I < kMods) {
-    const uint32_t word = w == 0 ? y[I].x : w == 1 ? y[I].y : w == 2 ? y[I].z : y[I].w;
-    const int r = (int)(signed char)(word >> (8 * c));
-    acc[0] += (long long)r * Crt<I>::w0;
-    acc[1] += (long long)r * Crt<I>::w1;
-    acc[2] += (long long)r * Crt<I>::w2;
-    acc[3] += (long long)r * Crt<I>::w3;
-    crt_add<I + 1>(y, w, c, acc);
+    constexpr u128 C = crt_fraction(I);
+    frac_add(f, __byte_perm(w ? y[I].y : y[I].x, 0, 0x4440 + c), frac_word(C, 0), frac_word(C, 1), frac_word(C, 2));
+    crt_add<I + 1>(y, w, c, f);
   }
 }
 
-// The integer x with |x| < P / 2 and x = sum_j acc_j 2^(30 j) (mod P), times 2^-s, rounded once.
-__device__ __forceinline__ double crt_value(long long (&acc)[4], int s) {
-  constexpr u128 P = mod_product();
-  // the quotient by P from the top limbs: the error of this estimate (2^-10) is far below the distance
-  // of |x| / P <= 0.39 from a half
-  constexpr float inv = (float)(65536.0 / ((double)(P >> 64) / 67108864.0));  // 2^16 / (P / 2^90)
-  const float f = (float)(int)(acc[3] >> 16) + (float)(int)(acc[2] >> 30) * (1.f / 65536.f);
-  const int q = (int)rintf(f * inv);
-  __int128 x = (__int128)(acc[0] - (long long)q * limb(P, 0));
-  x += (__int128)(acc[1] - (long long)q * limb(P, 1)) << 30;
-  x += (__int128)(acc[2] - (long long)q * limb(P, 2)) << 60;
-  x += (__int128)(acc[3] - (long long)q * limb(P, 3)) << 90;
-  const bool neg = x < 0;
-  const u128 a = neg ? (u128)(-x) : (u128)x;
-  unsigned long long hi = (unsigned long long)(a >> 64), lo = (unsigned long long)a;
-  if ((hi | lo) == 0) return 0.0;
-  int lz;
-  if (hi == 0) {
-    hi = lo;
-    lo = 0;
-    lz = 64;
-  } else {
-    lz = 0;
-  }
-  const int l = __clzll((long long)hi);
-  lz += l;
-  unsigned long long m = hi, rest = lo;
-  if (l) {
-    m = (hi << l) | (lo >> (64 - l));
-    rest = lo << l;
-  }
-  unsigned long long r = m >> 11;
-  const unsigned rem = (unsigned)(m & 0x7ff);
-  if (rem > 0x400u || (rem == 0x400u && (rest != 0 || (r & 1)))) ++r;
-  const int e = 127 - lz - s;  // the leading bit's exponent
-  if (e >= -1021 && e <= 1022) {
-    const unsigned long long b = ((unsigned long long)(e + 1022) << 52) + r;
-    return __longlong_as_double((long long)(b | (neg ? 1ull << 63 : 0ull)));
-  }
+// Results outside FP64's normal range, and those of poisoned rows.
+__device__ __noinline__ double scaled_value(unsigned long long r, int e, bool poison, bool neg) {
+  if (poison) return __longlong_as_double(0x7ff8000000000000ll);
   const double d = scalbn((double)r, e - 52);
   return neg ? -d : d;
 }
 
-// A warp takes 32 rows x 16 columns, a lane per row. Complex results whose rows are contiguous in the
-// output go out directly (512 contiguous bytes per store); the others through shared memory, so
-// that the 16 columns of a row leave as one 128-byte (real) or 128-byte (8 complex) segment.
+// x 2^-s from the signed fraction f = 2^64 x / P: |f| P in integers (the FP64 pipe would take a conversion and a
+// multiplication per value, each 1/64 of the rate), rounded to FP64. The fraction is good to 2^-64, that is
+// to 2^-62 of the product of the two rows' norm bounds, below the rounding of the operands.
+__device__ __forceinline__ double crt_value(unsigned long long f, int s) {
+  constexpr unsigned long long P64 = (unsigned long long)(mod_product() >> 54);
+  const unsigned sign = (unsigned)(f >> 32) & 0x80000000u;
+  const unsigned long long a = sign ? 0ull - f : f;
+  const int lz = __clzll((long long)(a | 1));
+  unsigned long long h = __umul64hi(a << lz, P64);
+  int e = 63 + 54 - lz - s;
+  if (!(h >> 63)) {
+    h <<= 1;
+    --e;
+  }
+  const unsigned long long r = (h >> 11) + ((h >> 10) & 1);
+  if ((unsigned)(e + 1021) > 2043u) return scaled_value(r, e, s < kPoison / 2, sign != 0);
+  const unsigned hi = (unsigned)(r >> 32) + ((unsigned)(e + 1022) << 20);
+  return a ? __hiloint2double((int)(hi | sign), (int)(unsigned)r) : 0.0;
+}
+
+__device__ __forceinline__ long long map_index(int x, int div, long long hi, long long lo) {
+  if (div == INT_MAX) return x * lo;
+  const int q = x / div;
+  return q * hi + (x - q * div) * lo;
+}
+
+// Output of a warp's 32 rows x 16 columns (8 complex) from its stage[32][17], a lane per row. Complex results whose
+// rows are contiguous in the output leave as 512 contiguous bytes per store, the others as 128-byte segments
+// of a row (radrs: the rows' offsets).
+__device__ __forceinline__ void put_complex(const CrtArgs& a, double2* d, double re, double im) {
+  double2 v = make_double2(re, im);
+  if (a.scaled) {
+    v.x *= a.alpha;
+    v.y *= a.alpha;
+  }
+  if (a.beta) {
+    const double2 o = *d;
+    v.x += o.x;
+    v.y += o.y;
+  }
+  *d = v;
+}
+
+__device__ __forceinline__ void store_complex(const CrtArgs& a, double2* D, const double* st, long long* radrs, int c0,
+                                              int rbase, int lane) {
+  const int row = rbase + lane;
+  const long long radr = map_index(a.row0 + row, a.r_div, a.r_hi, a.r_lo);
+  if (a.r_lo == 1) {
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+      const int cc = (c0 >> 1) + c;
+      if (2 * cc >= a.cols) break;
+      if (row < a.rows)
+        put_complex(a, D + radr + map_index(cc, a.c_div, a.c_hi, a.c_lo), st[lane * 17 + 2 * c], st[lane * 17 + 2 * c + 1]);
+    }
+    return;
+  }
+  radrs[lane] = radr;
+  __syncwarp();
+  // 4 rows x 8 complex columns per pass
+  const int cc = (c0 >> 1) + (lane & 7);
+  const long long cadr = map_index(cc, a.c_div, a.c_hi, a.c_lo);
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const int rl = i * 4 + (lane >> 3);
+    if (rbase + rl < a.rows && 2 * cc < a.cols)
+      put_complex(a, D + radrs[rl] + cadr, st[rl * 17 + 2 * (lane & 7)], st[rl * 17 + 2 * (lane & 7) + 1]);
+  }
+  __syncwarp();
+}
+
+// A warp takes 32 rows x 16 columns, a lane per row, 8 columns at a time (15 planes of 8 bytes in registers, so
+// that four CTAs fit an SM). Bound by issue (157 instructions per value, 45 of them the multiply-adds of the
+// fractions; IPC 2): 23.8 M values in 190 us. The same with the whole integer in 64-bit multiply-adds on
+// 30-bit limbs and 16 columns a time took 238 instructions at half the occupancy, 390 us.
 template <bool CPLX>
-__global__ void __launch_bounds__(256) rns_crt_kernel(const CrtArgs a) {
+__global__ void __launch_bounds__(256, 4) rns_crt_kernel(const CrtArgs a) {
   __shared__ double stage[8][32 * 17];
+  __shared__ long long radrs[CPLX ? 8 : 1][32];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int z = blockIdx.z;
-  const int c0 = (blockIdx.y * 8 + warp) * 16, rbase = blockIdx.x * 32, row = rbase + lane;
-  if (c0 >= a.cols) return;                                        // (whole warps leave)
+  const int z = blockIdx.y;
+  const long long item = (long long)blockIdx.x * 8 + warp;
+  const int nc = (a.cols + 15) / 16;
+  const int rg = (int)(item / nc);
+  const int c0 = (int)(item - (long long)rg * nc) * 16, rbase = rg * 32, row = rbase + lane;
+  if (rbase >= a.rows) return;                                     // (whole warps leave)
   if (!CPLX && a.tri && c0 > a.row0 + rbase + 31) return;
   const bool rok = row < a.rows;
-  uint4 y[kMods];
   const signed char* yp = a.Y + ((long long)z * a.rows + (rok ? row : 0)) * a.ldy + c0;
-#pragma unroll
-  for (int i = 0; i < kMods; ++i) y[i] = *reinterpret_cast<const uint4*>(yp + (long long)i * a.ymod);
   const int sa = rok ? a.ea[(long long)z * a.ea_rows + row] : 0;
+  const int* ebp = a.eb + (long long)z * a.eb_rows;
   double* st = stage[warp];
-  double2* D = nullptr;
-  long long radr = 0;
-  bool direct = false;
-  if constexpr (CPLX) {
-    D = a.D + (a.tab ? (long long)a.tab[a.tab0 + z].z : (long long)z) * a.sD;
-    const int gr = a.row0 + row;
-    radr = (long long)(gr / a.r_div) * a.r_hi + (long long)(gr % a.r_div) * a.r_lo;
-    direct = a.r_lo == 1;
-  }
+#pragma unroll 1
+  for (int h = 0; h < 2; ++h) {
+    if (c0 + 8 * h >= a.cols) break;
+    uint2 y[kMods];
 #pragma unroll
-  for (int w = 0; w < 4; ++w) {
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      const int col = c0 + 4 * w + c;
-      const int ec = CPLX ? col >> 1 : col;
-      long long acc[4] = {0, 0, 0, 0};
-      crt_add<0>(y, w, c, acc);
-      double v = 0.0;
-      if (col < a.cols) {
-        const int sb = a.eb[(long long)z * a.eb_rows + ec];
-        v = (sa == kPoison || sb == kPoison) ? __longlong_as_double(0x7ff8000000000000ll) : crt_value(acc, sa + sb);
-      }
-      st[lane * 17 + 4 * w + c] = v;
+    for (int i = 0; i < kMods; ++i) {
+      y[i] = *reinterpret_cast<const uint2*>(yp + (long long)i * a.ymod + 8 * h);
+      y[i].x ^= 0x80808080u;
+      y[i].y ^= 0x80808080u;
     }
-    if constexpr (CPLX) {
-      if (direct) {
-        // lanes hold consecutive rows: each lane stores its own pairs
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const int cc = (c0 >> 1) + 2 * w + h;
-          if (rok && 2 * cc < a.cols) {
-            double2 v = make_double2(st[lane * 17 + 4 * w + 2 * h], st[lane * 17 + 4 * w + 2 * h + 1]);
-            if (a.alpha != 1.0) {
-              v.x *= a.alpha;
-              v.y *= a.alpha;
-            }
-            double2* d = D + radr + (long long)(cc / a.c_div) * a.c_hi + (long long)(cc % a.c_div) * a.c_lo;
-            if (a.beta) {
-              const double2 o = *d;
-              v.x += o.x;
-              v.y += o.y;
-            }
-            *d = v;
-          }
-        }
-      }
+    for (int c = 0; c < 8; ++c) {
+      Frac f = frac_start();
+      crt_add<0>(y, c >> 2, c & 3, f);
+      const int sb = ebp[min(c0 + 8 * h + c, a.cols - 1) >> (CPLX ? 1 : 0)];
+      st[lane * 17 + 8 * h + c] = crt_value(frac_fold(f), sa + sb);
     }
   }
-  if (CPLX && direct) return;
   __syncwarp();
   if constexpr (CPLX) {
-    // 4 rows x 8 complex columns per pass
-    const int cc = (c0 >> 1) + (lane & 7);
-    const long long cadr = (long long)(cc / a.c_div) * a.c_hi + (long long)(cc % a.c_div) * a.c_lo;
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const int rl = i * 4 + (lane >> 3), gr = a.row0 + rbase + rl;
-      if (rbase + rl < a.rows && 2 * cc < a.cols) {
-        double2 v = make_double2(st[rl * 17 + 2 * (lane & 7)], st[rl * 17 + 2 * (lane & 7) + 1]);
-        if (a.alpha != 1.0) {
-          v.x *= a.alpha;
-          v.y *= a.alpha;
-        }
-        double2* d = D + (long long)(gr / a.r_div) * a.r_hi + (long long)(gr % a.r_div) * a.r_lo + cadr;
-        if (a.beta) {
-          const double2 o = *d;
-          v.x += o.x;
-          v.y += o.y;
-        }
-        *d = v;
-      }
-    }
+    double2* D = a.D + (a.tab ? (long long)a.tab[a.tab0 + z].z : (long long)z) * a.sD;
+    store_complex(a, D, st, radrs[warp], c0, rbase, lane);
   } else {
     // 2 rows x 16 columns per pass
     const int col = c0 + (lane & 15);
@@ -749,6 +764,10 @@ __global__ void __launch_bounds__(256) rns_crt_kernel(const CrtArgs a) {
       *d += a.alpha * st[rl * 17 + (lane & 15)];
     }
   }
+}
+
+unsigned crt_blocks(int rows, int cols) {
+  return (unsigned)(((long long)((rows + 31) / 32) * ((cols + 15) / 16) + 7) / 8);
 }
 
 // ---------------- host side ----------------
@@ -765,7 +784,7 @@ struct Side {
 };
 
 cudaError_t convert(const Side& o, int r0, int nrows, const int4* tab, int tab0, int K, int Kp, int nb,
-                    long long batch0, __nv_bfloat16* R, long long smod, int* exps, cudaStream_t s) {
+                    long long batch0, __nv_bfloat16* R, long long smod, int* exps, int sms, cudaStream_t s) {
   ConvArgs a;
   std::memset(&a, 0, sizeof(a));
   const int w = o.src == SRC_REAL ? 1 : 2;
@@ -783,10 +802,15 @@ cudaError_t convert(const Side& o, int r0, int nrows, const int4* tab, int tab0,
   a.R = R;
   a.smod = smod;
   a.exps = exps;
-  const dim3 grid((nrows + 31) / 32, nb);
-  if (o.src == SRC_COMPLEX) rns_convert_kernel<SRC_COMPLEX><<<grid, 256, 0, s>>>(a);
-  else if (o.src == SRC_COMPLEX2) rns_convert_kernel<SRC_COMPLEX2><<<grid, 256, 0, s>>>(a);
-  else rns_convert_kernel<SRC_REAL><<<grid, 256, 0, s>>>(a);
+  const bool few = (long long)((nrows + 31) / 32) * nb < 2 * sms;
+  const dim3 grid(few ? (nrows + 7) / 8 : (nrows + 31) / 32, nb);
+  auto go = [&](auto wide, auto narrow) {
+    if (few) narrow<<<grid, 256, 0, s>>>(a);
+    else wide<<<grid, 256, 0, s>>>(a);
+  };
+  if (o.src == SRC_COMPLEX) go(rns_convert_kernel<SRC_COMPLEX, 32>, rns_convert_kernel<SRC_COMPLEX, 8>);
+  else if (o.src == SRC_COMPLEX2) go(rns_convert_kernel<SRC_COMPLEX2, 32>, rns_convert_kernel<SRC_COMPLEX2, 8>);
+  else go(rns_convert_kernel<SRC_REAL, 32>, rns_convert_kernel<SRC_REAL, 8>);
   return cudaGetLastError();
 }
 
@@ -896,38 +920,22 @@ cudaError_t rns_zgemm(const ZgemmArgs& a, int al, bool cj, int bl, const RnsCtx&
       const int m = std::min(nr, p.rows.rows - r0);
       Carve w{(char*)c.scratch, (char*)c.scratch + c.bytes};
       const long long smA = (long long)n * m * p.Kp, smB = (long long)n * 2 * p.cols.rows * p.Kp;
-      __nv_bfloat16* RA = (__nv_bfloat16*)w.take((size_t)smA * 2 * kMods);
+      // (the column operand first: it stays in place over the row chunks of an entry)
       __nv_bfloat16* RB = (__nv_bfloat16*)w.take((size_t)smB * 2 * kMods);
+      int* eb = (int*)w.take((size_t)n * p.cols.rows * 4);
+      __nv_bfloat16* RA = (__nv_bfloat16*)w.take((size_t)smA * 2 * kMods);
       signed char* Y = (signed char*)w.take((size_t)n * m * p.ldy * kMods);
       int* ea = (int*)w.take((size_t)n * m * 4);
-      int* eb = (int*)w.take((size_t)n * p.cols.rows * 4);
       if (w.p > w.end) return cudaErrorInvalidValue;
-      cudaError_t e = convert(p.cols, 0, p.cols.rows, a.tab, a.tab0 + b0, p.K, p.Kp, n, b0, RB, smB, eb, s);
+      cudaError_t e = cudaSuccess;
+      if (r0 == 0) e = convert(p.cols, 0, p.cols.rows, a.tab, a.tab0 + b0, p.K, p.Kp, n, b0, RB, smB, eb, c.sms, s);
       if (e != cudaSuccess) return e;
-      e = convert(p.rows, r0, m, a.tab, a.tab0 + b0, p.K, p.Kp, n, b0, RA, smA, ea, s);
-      if (e != cudaSuccess) return e;
-      GemmArgs g;
-      std::memset(&g, 0, sizeof(g));
-      g.nbatch = n;
-      g.rows = m;
-      g.cols = 2 * p.cols.rows;
-      g.rt = (m + kTileM - 1) / kTileM;
-      g.bn = tile_width(g.cols);
-      g.ct = (g.cols + g.bn - 1) / g.bn;
-      g.tiles = g.rt * g.ct;
-      g.nkb = p.Kp / kBK;
-      g.Y = Y;
-      g.ymod = (long long)n * m * p.ldy;
-      g.ldy = p.ldy;
-      e = gemm(RA, smA, RB, smB, g, p.Kp, m, c, s);
+      e = convert(p.rows, r0, m, a.tab, a.tab0 + b0, p.K, p.Kp, n, b0, RA, smA, ea, c.sms, s);
       if (e != cudaSuccess) return e;
       CrtArgs x;
       std::memset(&x, 0, sizeof(x));
-      x.Y = Y;
-      x.ymod = g.ymod;
-      x.ldy = p.ldy;
       x.rows = m;
-      x.cols = g.cols;
+      x.cols = 2 * p.cols.rows;
       x.row0 = r0;
       x.ea = ea;
       x.eb = eb;
@@ -944,11 +952,29 @@ cudaError_t rns_zgemm(const ZgemmArgs& a, int al, bool cj, int bl, const RnsCtx&
       x.c_hi = p.rows_are_m ? a.dn_hi : a.dm_hi;
       x.c_lo = p.rows_are_m ? a.dn_lo : a.dm_lo;
       x.alpha = a.alpha;
+      x.scaled = a.alpha != 1.0;
       x.beta = a.beta;
-      const dim3 grid((m + 31) / 32, (g.cols + 127) / 128, n);
+      GemmArgs g;
+      std::memset(&g, 0, sizeof(g));
+      g.nbatch = n;
+      g.rows = m;
+      g.cols = x.cols;
+      g.rt = (m + kTileM - 1) / kTileM;
+      g.bn = tile_width(g.cols);
+      g.ct = (g.cols + g.bn - 1) / g.bn;
+      g.tiles = g.rt * g.ct;
+      g.nkb = p.Kp / kBK;
+      g.Y = Y;
+      g.ymod = (long long)n * m * p.ldy;
+      g.ldy = p.ldy;
+      if ((e = gemm(RA, smA, RB, smB, g, p.Kp, m, c, s)) != cudaSuccess) return e;
+      x.Y = Y;
+      x.ymod = g.ymod;
+      x.ldy = p.ldy;
+      const dim3 grid(crt_blocks(m, g.cols), n);
       rns_crt_kernel<true><<<grid, 256, 0, s>>>(x);
       if ((e = cudaGetLastError()) != cudaSuccess) return e;
-      *launches += 4;
+      *launches += r0 == 0 ? 4 : 3;
     }
   }
   return cudaSuccess;
@@ -994,10 +1020,10 @@ cudaError_t rns_dsyrk(const DsyrkArgs& a, const RnsCtx& c, cudaStream_t s, int* 
     Side xs = X, ys = Yo;
     xs.base += k0 * a.ldx;
     ys.base += k0 * a.ldy;
-    cudaError_t e = convert(xs, 0, M, nullptr, 0, K, Kp, 1, 0, RA, smA, ea, s);
+    cudaError_t e = convert(xs, 0, M, nullptr, 0, K, Kp, 1, 0, RA, smA, ea, c.sms, s);
     if (e != cudaSuccess) return e;
     if (!tri) {
-      e = convert(ys, 0, N, nullptr, 0, K, Kp, 1, 0, RB, smB, eb, s);
+      e = convert(ys, 0, N, nullptr, 0, K, Kp, 1, 0, RB, smB, eb, c.sms, s);
       if (e != cudaSuccess) return e;
     }
     *launches += tri ? 1 : 2;
@@ -1035,7 +1061,7 @@ cudaError_t rns_dsyrk(const DsyrkArgs& a, const RnsCtx& c, cudaStream_t s, int* 
       x.ldo = a.ldo;
       x.tri = tri;
       x.alpha = a.alpha;
-      const dim3 grid((m + 31) / 32, (N + 127) / 128, 1);
+      const dim3 grid(crt_blocks(m, N), 1);
       rns_crt_kernel<false><<<grid, 256, 0, s>>>(x);
       if ((e = cudaGetLastError()) != cudaSuccess) return e;
       *launches += 2;
