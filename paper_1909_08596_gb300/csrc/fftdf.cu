@@ -103,15 +103,34 @@ __global__ void __launch_bounds__(256) dft_axis_kernel(const double2* __restrict
 }
 
 // out[i] += sum_p parts[p n + i]
-__global__ void sum_parts_kernel(const double2* __restrict__ parts, int np, long long n, double2* __restrict__ out) {
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    double2 a = out[i];
-    for (int p = 0; p < np; ++p) {
-      const double2 b = parts[(long long)p * n + i];
-      a.x += b.x;
-      a.y += b.y;
+// Eight threads share the parts of each element (32 elements per CTA), so that a small block with many parts (the
+// 104^2 exchange matrix from some 300 parts) still has a few hundred CTAs of loads in flight.
+__global__ void __launch_bounds__(256) sum_parts_kernel(const double2* __restrict__ parts, int np, long long n,
+                                                        double2* __restrict__ out) {
+  __shared__ double2 sh[8][33];
+  const int x = threadIdx.x & 31, g = threadIdx.x >> 5;
+  for (long long i0 = blockIdx.x * 32ll; i0 < n; i0 += gridDim.x * 32ll) {
+    double2 a = make_double2(0.0, 0.0);
+    if (i0 + x < n) {
+#pragma unroll 4
+      for (int p = g; p < np; p += 8) {
+        const double2 b = parts[(long long)p * n + i0 + x];
+        a.x += b.x;
+        a.y += b.y;
+      }
     }
-    out[i] = a;
+    sh[g][x] = a;
+    __syncthreads();
+    if (g == 0 && i0 + x < n) {
+      a = out[i0 + x];
+#pragma unroll
+      for (int h = 0; h < 8; ++h) {
+        a.x += sh[h][x].x;
+        a.y += sh[h][x].y;
+      }
+      out[i0 + x] = a;
+    }
+    __syncthreads();
   }
 }
 
@@ -127,7 +146,7 @@ cudaError_t launch_dft_axis_small(const double2* F, int g, long long outer, long
 }
 
 cudaError_t launch_sum_parts(const double2* parts, int np, long long n, double2* out, cudaStream_t st) {
-  sum_parts_kernel<<<grid_for(n, 256, 152 * 16), 256, 0, st>>>(parts, np, n, out);
+  sum_parts_kernel<<<grid_for(n, 32, 152 * 32), 256, 0, st>>>(parts, np, n, out);
   return cudaGetLastError();
 }
 

@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
+
 #include "internal.h"
 
 namespace dmet {
@@ -132,6 +134,64 @@ __global__ void __launch_bounds__(256) jk_trace_kernel(const double2* __restrict
   }
 }
 
+// gt[k][l] = gamma[l][k]
+__global__ void transpose_kernel(const double2* __restrict__ g, int n, double2* __restrict__ gt) {
+  for (int x = blockIdx.x * blockDim.x + threadIdx.x; x < n * n; x += gridDim.x * blockDim.x)
+    gt[x] = g[(x % n) * n + x / n];
+}
+
+// v[z] = sum_{k,l} Lq[m(z)][k][l] gt[k][l] for z = (q, P) from z0 on, m(z) = (neg[q], P). One CTA per z; bound by
+// reading the factors (the transposed density stays in L2).
+__global__ void __launch_bounds__(256) jk_trace_all_kernel(const double2* __restrict__ Lq, const int* __restrict__ neg,
+                                                           int naux, long long nn, const double2* __restrict__ gt,
+                                                           double2* __restrict__ v) {
+  const int q = blockIdx.y, P = blockIdx.x;
+  const double2* m = Lq + ((long long)neg[q] * naux + P) * nn;
+  double re = 0.0, im = 0.0;
+#pragma unroll 4
+  for (int x = threadIdx.x; x < (int)nn; x += 256) {
+    const double2 a = m[x], g = gt[x];
+    re = fma(a.x, g.x, fma(-a.y, g.y, re));
+    im = fma(a.x, g.y, fma(a.y, g.x, im));
+  }
+  __shared__ double sr[8], si[8];
+#pragma unroll
+  for (int o = 16; o; o >>= 1) {
+    re += __shfl_xor_sync(0xffffffffu, re, o);
+    im += __shfl_xor_sync(0xffffffffu, im, o);
+  }
+  if ((threadIdx.x & 31) == 0) {
+    sr[threadIdx.x >> 5] = re;
+    si[threadIdx.x >> 5] = im;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double a = 0.0, b = 0.0;
+    for (int w = 0; w < 8; ++w) {
+      a += sr[w];
+      b += si[w];
+    }
+    v[(long long)q * naux + P] = make_double2(a, b);
+  }
+}
+
+// part[y][x] = s sum_z v[z] Lq[z][x] over share y of the z.
+__global__ void __launch_bounds__(256) jk_weighted_kernel(const double2* __restrict__ Lq, const double2* __restrict__ v,
+                                                          long long nz, long long nn, double s,
+                                                          double2* __restrict__ part) {
+  const long long x = blockIdx.x * 256ll + threadIdx.x;
+  if (x >= nn) return;
+  const long long z0 = nz * blockIdx.y / gridDim.y, z1 = nz * (blockIdx.y + 1) / gridDim.y;
+  double jr = 0.0, ji = 0.0;
+#pragma unroll 4
+  for (long long z = z0; z < z1; ++z) {
+    const double2 a = Lq[z * nn + x], w = v[z];
+    jr = fma(a.x, w.x, fma(-a.y, w.y, jr));
+    ji = fma(a.x, w.y, fma(a.y, w.x, ji));
+  }
+  part[blockIdx.y * nn + x] = make_double2(s * jr, s * ji);
+}
+
 // J[x] += s sum_z v[z] Lq[tab[z].x][x] and K[x] += s sum_z Kb[z][x] over the nz entries of a chunk.
 __global__ void __launch_bounds__(256) jk_accumulate_kernel(const double2* __restrict__ Lq, const int4* __restrict__ tab,
                                                             const double2* __restrict__ v, const double2* __restrict__ Kb,
@@ -194,6 +254,21 @@ cudaError_t launch_jk_accumulate(const double2* Lq, const int4* tab, const doubl
   if (blocks > 152 * 8) blocks = 152 * 8;
   jk_accumulate_kernel<<<(unsigned)(blocks > 0 ? blocks : 1), 256, 0, st>>>(Lq, tab, v, Kb, nz, nn, s, J, K);
   return cudaGetLastError();
+}
+
+// J += s sum_{q,P} Lq[q][P] tr(Lq[-q][P] gamma): two passes over the factors (gt, v and part: scratch of n^2, nk naux
+// and jk_coulomb_parts() n^2 values).
+int jk_coulomb_parts(long long nn) { return (int)std::max(1LL, 8LL * 152 / std::max(1LL, (nn + 255) / 256)); }
+
+cudaError_t launch_jk_coulomb(const double2* Lq, const int* neg, int nk, int naux, int n, const double2* gamma, double s,
+                              double2* gt, double2* v, double2* part, double2* J, cudaStream_t st) {
+  const long long nn = (long long)n * n;
+  transpose_kernel<<<blocks_for(nn, 256, 152), 256, 0, st>>>(gamma, n, gt);
+  jk_trace_all_kernel<<<dim3(naux, nk), 256, 0, st>>>(Lq, neg, naux, nn, gt, v);
+  const int parts = jk_coulomb_parts(nn);
+  jk_weighted_kernel<<<dim3((unsigned)((nn + 255) / 256), parts), 256, 0, st>>>(Lq, v, (long long)nk * naux, nn, s, part);
+  cudaError_t e = cudaGetLastError();
+  return e == cudaSuccess ? launch_sum_parts(part, parts, nn, J, st) : e;
 }
 
 }  // namespace dmet

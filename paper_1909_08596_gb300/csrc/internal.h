@@ -101,6 +101,9 @@ cudaError_t launch_fftdf_phase_q(const double2* src, double2* dst, const int* qt
 // v[z] = tr(L^{-q}_P gamma); J += s sum_z v[z] L^q_P; K += s sum_z Kb[z] (Kb[z] = L^q_P gamma L^{-q}_P).
 cudaError_t launch_jk_trace(const double2* Lq, const int4* tab, int nz, int n, const double2* gamma, double2* v,
                             cudaStream_t st);
+int jk_coulomb_parts(long long nn);
+cudaError_t launch_jk_coulomb(const double2* Lq, const int* neg, int nk, int naux, int n, const double2* gamma, double s,
+                              double2* gt, double2* v, double2* part, double2* J, cudaStream_t st);
 cudaError_t launch_jk_accumulate(const double2* Lq, const int4* tab, const double2* v, const double2* Kb, int nz, int n,
                                  double s, double2* J, double2* K, cudaStream_t st);
 // Bath construction (bath.cu). The impurity columns that enter the SVD, by value.

@@ -597,9 +597,8 @@ ZgemmArgs zargs() {
 // tensor cores where that is faster (rns.cu), else on the FP64 pipe. `t` counts its launches.
 RnsCtx rns_ctx(dmet_emb_plan_s* P) {
   RnsCtx c;
-  if (!P->W || !P->W->rns) return c;
-  c.scratch = P->W->rns;
-  c.bytes = P->W->rns_b;
+  c.scratch = P->W ? P->W->rns : nullptr;
+  c.bytes = c.scratch ? P->W->rns_b : 0;
   c.sms = P->sms;
   c.err = P->derr;
   c.wait_ns = P->wait_ns;
@@ -2968,6 +2967,94 @@ dmet_status_t dmet_emb_bath(dmet_emb_plan_t P, int32_t problem, int32_t spin, co
   return DMET_OK;
 }
 
+// J and K of dmet_emb_jk_df through residue products, q by q in chunks: W = L^q_P gamma for every P, stored [P][l][i], then
+// K += (1/Nk) sum over (P, l) of W[(P, l)][i] L^{-q}[(P, l)][j] as one product of K = n_aux n per q, split into
+// parts of the aux functions that fill the GPU. *done = false: the products are too small for it (nothing queued).
+static dmet_status_t jk_residues(dmet_emb_plan_s* P, Prob& pr, int n, const double2* Lq, const double2* gamma,
+                                 double2* J, double2* K, bool* done) {
+  *done = false;
+  const int nk = pr.nk, naux = pr.naux;
+  const long long nn = (long long)n * n;
+  if ((long long)naux * n > INT_MAX / 4 || nk > 65535) return DMET_OK;
+  const size_t wq = (size_t)naux * nn * 16;  // W of one q
+  const int cq = (int)std::max<size_t>(1, std::min<size_t>(nk, ((size_t)256 << 20) / wq));
+  const long long tiles = ((n + 127) / 128) * (long long)((2 * n + 255) / 256);
+  const int want = (int)((4LL * P->sms + 15 * cq * tiles - 1) / (15 * cq * tiles));
+  const int pl = std::max(1, naux / std::min(naux, want)), parts = (naux + pl - 1) / pl;
+  if ((long long)cq * parts > 65535) return DMET_OK;
+  ZgemmArgs z1 = zargs(), z2 = zargs();
+  z1.A = gamma;  // opA(b, l) = gamma[l][b], opB(l, (P, a)) = L[(P, a)][l], stored at [P][b][a]
+  z1.M = n;
+  z1.K = n;
+  z1.lda = n;
+  z1.ldb = n;
+  z1.dm_lo = n;
+  z1.dn_div = n;
+  z1.dn_hi = nn;
+  z1.dn_lo = 1;
+  z1.N = (int)std::min<long long>((long long)cq * naux * n, INT_MAX / 4);
+  z2.M = n;      // opA((P, l), i) = W[P][l][i], opB((P, l), j) = L^{-q}[P][l][j]
+  z2.N = n;
+  z2.K = pl * n;
+  z2.lda = n;
+  z2.ldb = n;
+  z2.sA = nn;
+  z2.sB = nn;
+  z2.sD = nn;
+  z2.dm_lo = n;
+  z2.dn_lo = 1;
+  z2.alpha = 1.0 / nk;
+  z2.batch = cq * parts;
+  // scratch: W, the parts of K, the entry table, the Coulomb pass, the residues
+  const size_t oP = ((size_t)cq * wq + 255) / 256 * 256, oT = oP + (size_t)cq * parts * nn * 16;
+  const size_t oG = oT + (size_t)nk * parts * sizeof(int4), oV = oG + (size_t)nn * 16;
+  const size_t oJ = oV + (size_t)nk * naux * 16, oR = (oJ + (size_t)jk_coulomb_parts(nn) * nn * 16 + 1023) / 1024 * 1024;
+  const size_t rb = std::min<size_t>((size_t)704 << 20, std::max(rns_need(z1), rns_need(z2)));
+  RnsCtx c = rns_ctx(P);
+  c.scratch = (void*)16;  // (only tested for being there)
+  c.bytes = rb;
+  if (!rns_takes_zgemm(z1, c) || !rns_takes_zgemm(z2, c)) return DMET_OK;
+  TRY(ensure(&P->jk_ws, &P->jk_ws_b, oR + rb));
+  char* w = (char*)P->jk_ws;
+  double2* W = (double2*)w;
+  double2* part = (double2*)(w + oP);
+  int4* tab = (int4*)(w + oT);
+  c.scratch = w + oR;
+  std::vector<int4> t((size_t)nk * parts);
+  for (int q = 0; q < nk; ++q)
+    for (int h = 0; h < parts; ++h) {
+      const int p0 = h * pl, p1 = std::min(naux, p0 + pl);
+      t[(size_t)q * parts + h] = make_int4(q * naux + p0, pr.s.neg[q] * naux + p0, (q % cq) * parts + h, (p1 - p0) * n);
+    }
+  // flops: the two products and the two reductions of every (q, P)
+  Timed tm(P, KC_JK_DF, 8.0 * nk * naux * (2.0 * nn * n + 2.0 * nn), 16.0 * nk * naux * nn * 5, 4);
+  CK(cudaMemcpyAsync(tab, t.data(), t.size() * sizeof(int4), cudaMemcpyHostToDevice, P->cs));
+  CK(cudaMemsetAsync(J, 0, (size_t)nn * 16, P->cs));
+  CK(cudaMemsetAsync(K, 0, (size_t)nn * 16, P->cs));
+  int launches = 0;
+  CK(launch_jk_coulomb(Lq, pr.d_neg, nk, naux, n, gamma, 1.0 / nk, (double2*)(w + oG), (double2*)(w + oV),
+                       (double2*)(w + oJ), J, P->cs));
+  for (int q0 = 0; q0 < nk; q0 += cq) {
+    const int nq = std::min(cq, nk - q0);
+    z1.B = Lq + (long long)q0 * naux * nn;
+    z1.D = W;
+    z1.N = nq * naux * n;
+    CK(rns_zgemm(z1, A_KM, false, B_NK, c, P->cs, &launches));
+    z2.A = W - (long long)q0 * naux * nn;  // (the table holds absolute q)
+    z2.B = Lq;
+    z2.D = part;
+    z2.tab = tab;
+    z2.tab0 = q0 * parts;
+    z2.batch = nq * parts;
+    CK(rns_zgemm(z2, A_KM, false, B_KN, c, P->cs, &launches));
+    CK(launch_sum_parts(part, nq * parts, nn, K, P->cs));
+    ++launches;
+  }
+  tm.more(launches);
+  *done = true;
+  return DMET_OK;
+}
+
 dmet_status_t dmet_emb_jk_df(dmet_emb_plan_t P, int32_t problem, int32_t spin, const void* Lq, const void* gamma,
                              void* J, void* K) {
   clear_error();
@@ -2983,6 +3070,11 @@ dmet_status_t dmet_emb_jk_df(dmet_emb_plan_t P, int32_t problem, int32_t spin, c
   }
   const int nk = pr.nk, naux = pr.naux, n = pr.n[spin];
   const long long nn = (long long)n * n, nz_all = (long long)nk * naux;
+  P->cs = P->stream;
+  P->W = &P->ws[P->ws_of[problem]];
+  bool done = false;
+  TRY(jk_residues(P, pr, n, (const double2*)Lq, (const double2*)gamma, (double2*)J, (double2*)K, &done));
+  if (done) return DMET_OK;
   // batch entries z = (q, P) in chunks whose two n x n scratch matrices per entry stay within 1 GiB
   const long long per = 2 * nn * 16 + 16 + 2 * (long long)sizeof(int4);
   const int chunk = (int)std::max(1LL, std::min({nz_all, (1LL << 30) / per, 65535LL}));

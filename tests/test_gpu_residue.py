@@ -100,3 +100,30 @@ def test_non_finite_and_tiny(torch):
     bad[0, 0, 5, 3, 4] = np.nan
     (got,), _, _ = run_eri(torch, d, bad, [C])
     assert np.isnan(got).all()
+
+
+@pytest.mark.parametrize("mesh,n_aux,n,real", [((3, 2, 1), 91, 37, True), ((2, 2, 1), 130, 64, False), ((3, 1, 1), 53, 131, True)])
+def test_coulomb_exchange_from_factors(torch, mesh, n_aux, n, real):
+    """dmet_emb_jk_df in chunks of q with K split into ragged parts of the aux functions; factors without any
+    symmetry between q and -q."""
+    nk = int(np.prod(mesh))
+    rng = np.random.default_rng(6)
+    Lq = rng.standard_normal((nk, n_aux, n, n)) + 1j * rng.standard_normal((nk, n_aux, n, n))
+    gamma = synth.embedding_density(n, 9).astype(np.complex128)
+    if not real:
+        gamma = gamma + 0.1j * rng.standard_normal((n, n))
+    d = dm.make_desc(mesh, max(1, -(-n // nk)), n_aux, n, sym=B.DMET_SYM_NONE)
+    Ld, gd = torch.from_numpy(Lq).cuda(), torch.from_numpy(gamma).cuda()
+    J = torch.empty((n, n), dtype=torch.complex128, device="cuda")
+    K = torch.empty_like(J)
+    plan = dm.dmet_emb_plan(d, stream=torch.cuda.current_stream().cuda_stream)
+    try:
+        for _ in range(2):
+            dm.dmet_emb_jk_df(plan, Ld, gd, J, K)
+        st, _ = dm.dmet_emb_status(plan, 0)
+    finally:
+        dm.dmet_emb_destroy(plan)
+    assert st == B.DMET_OK
+    Jr, Kr = oracle.coulomb_exchange_df(Lq, gamma, mesh)
+    check(J.cpu().numpy().ravel(), Jr)
+    check(K.cpu().numpy().ravel(), Kr)
