@@ -88,6 +88,13 @@ cudaError_t launch_fftdf_kernel_mul(double2* buf, const double* v, long long ng,
 // A dense DFT along the middle axis of [outer][g][inner] for g <= 32 (fftdf_small_axis):
 // out[o][k][i] = sum_j F[k g + j] in[o][j][i].
 bool fftdf_small_axis(int g);
+// FFT along one axis of buf [q][grid][nx] for lengths with prime factors 2, 3, 5, 7 up to 32 (fftdf_fft_axis): columns
+// (o, i) of g points at o g inner + i, q = o / per_q. mode 0: times phase [q][g], forward (read from block qtab[q]
+// of `in` if qtab); mode 1: that, times v [o][g], inverse, times conj phase; mode 2: inverse, times conj phase.
+bool fftdf_fft_axis(int g);
+cudaError_t launch_fft_axis(int g, int mode, const double2* in, const int* qtab, double2* buf, const double2* F,
+                            const double2* phase, const double* v, long long outer, long long inner, long long per_q,
+                            cudaStream_t st);
 cudaError_t launch_dft_axis_small(const double2* F, int g, long long outer, long long inner, const double2* in,
                                   double2* out, cudaStream_t st);
 // out[i] += sum over the np parts of parts[p n + i] (the K parts of a split GEMM).

@@ -3254,6 +3254,21 @@ dmet_status_t dmet_emb_eri_fftdf(dmet_emb_plan_t P, int32_t problem, const void*
     qtab[qq] = pr.s.neg[qq];
     std::memcpy(vp.data() + (size_t)qq * ng, vq.data() + (size_t)qtab[qq] * ng, sizeof(double) * ng);
   }
+  // exp(-i q.r) = prod_d exp(-2 pi i j_d n_d / (N_d g_d)), tabulated per axis for q = -q', for the FFT passes
+  const bool ffts = fftdf_fft_axis(grid[0]) && fftdf_fft_axis(grid[1]) && fftdf_fft_axis(grid[2]);
+  std::vector<double2> ph;
+  size_t ph_off[3];
+  for (int d = 0; d < 3; ++d) {
+    ph_off[d] = ph.size();
+    for (int qq = 0; ffts && qq < nk; ++qq) {
+      const int* ms = pr.d.mesh;
+      const int n3[3] = {qtab[qq] / (ms[1] * ms[2]), (qtab[qq] / ms[2]) % ms[1], qtab[qq] % ms[2]};
+      for (int j = 0; j < grid[d]; ++j) {
+        const double x = 2.0 * M_PI * (double)((long long)j * n3[d]) / ((double)ms[d] * grid[d]);
+        ph.push_back(make_double2(std::cos(x), -std::sin(x)));
+      }
+    }
+  }
   // The contraction GEMM of a chunk is n^2 x n^2 with K = qc N_g: few output tiles over a long K, so
   // it is split in K into kparts batches (partial blocks, summed afterwards) that fill the GPU.
   const long long ktot = (long long)qc * ng, tiles_min = ((nx_max + 63) / 64) * ((nx_max + 63) / 64);
@@ -3264,7 +3279,8 @@ dmet_status_t dmet_emb_eri_fftdf(dmet_emb_plan_t P, int32_t problem, const void*
   // scratch: two [qc][grid][n^2] buffers, the DFT matrices, the kernels, the q table, the K parts
   const size_t bbuf = (size_t)qc * ng * nx_max * 16, oF = 2 * bbuf, oV = oF + (F.size() * 16 + 255) / 256 * 256;
   const size_t oQ = oV + (vp.size() * 8 + 255) / 256 * 256;
-  const size_t oP = oQ + (qtab.size() * sizeof(int) + 255) / 256 * 256;
+  const size_t oH = oQ + (qtab.size() * sizeof(int) + 255) / 256 * 256;
+  const size_t oP = oH + (ph.size() * 16 + 255) / 256 * 256;
   P->cs = P->stream;
   TRY(ensure(&P->fft_ws, &P->fft_ws_b, oP + (kparts > 1 ? (size_t)kparts * nx_max * nx_max * 16 : 0)));
   char* w = (char*)P->fft_ws;
@@ -3273,10 +3289,12 @@ dmet_status_t dmet_emb_eri_fftdf(dmet_emb_plan_t P, int32_t problem, const void*
   double2* dF = (double2*)(w + oF);
   double* dV = (double*)(w + oV);
   int* dQ = (int*)(w + oQ);
+  double2* dH = (double2*)(w + oH);
   double2* dPart = (double2*)(w + oP);
   CK(cudaMemcpyAsync(dF, F.data(), F.size() * 16, cudaMemcpyHostToDevice, P->cs));
   CK(cudaMemcpyAsync(dV, vp.data(), vp.size() * 8, cudaMemcpyHostToDevice, P->cs));
   CK(cudaMemcpyAsync(dQ, qtab.data(), qtab.size() * sizeof(int), cudaMemcpyHostToDevice, P->cs));
+  if (ffts) CK(cudaMemcpyAsync(dH, ph.data(), ph.size() * 16, cudaMemcpyHostToDevice, P->cs));
   // Step 1 of Algorithm 2 for every q and spin: (r|0i 0j) = s sum_k1 C^{k1+} rho^{k1,k1+q}(r) C^{k1+q}
   const double2* Cd[2] = {(const double2*)C[0], pr.nspin == 2 ? (const double2*)C[1] : nullptr};
   P->W = &P->ws[P->ws_of[problem]];
@@ -3289,7 +3307,22 @@ dmet_status_t dmet_emb_eri_fftdf(dmet_emb_plan_t P, int32_t problem, const void*
     const long long nx = (long long)pr.n[sa] * pr.n[sa];
     for (int c0 = 0; c0 < nk; c0 += qc) {
       const int nc = std::min(qc, nk - c0);
-      {
+      if (ffts) {
+        // 2. the same in five passes over the chunk, the phases and the kernel within them
+        Timed t(P, KC_FFTDF, 10.0 * ng * nx * std::log2((double)ng) * nc, 16.0 * ng * nx * 10 * nc, 5);
+        const double2* h[3];
+        for (int d = 0; d < 3; ++d) h[d] = dH + ph_off[d] + (size_t)c0 * grid[d];
+        auto pass = [&](int d, int mode, const double2* in) {
+          const long long per = d == 0 ? 1 : d == 1 ? g0 : g0 * g1, inner = d == 0 ? g1 * g2 * nx : d == 1 ? g2 * nx : nx;
+          return launch_fft_axis(grid[d], mode, in, in ? dQ + c0 : nullptr, buf1, dF + f_off[d][0], h[d],
+                                 dV + (size_t)c0 * ng, nc * per, inner, per, P->cs);
+        };
+        CK(pass(0, 0, lq[sa]));
+        CK(pass(1, 0, nullptr));
+        CK(pass(2, 1, nullptr));
+        CK(pass(1, 2, nullptr));
+        CK(pass(0, 2, nullptr));
+      } else {
         Timed t(P, KC_FFTDF, 8.0 * ng * nx * 2.0 * (g0 + g1 + g2) * nc, 16.0 * ng * nx * 14 * nc, 9);
         // 2. exp(-i q.r), forward DFT, 4 pi / |q + G|^2, inverse DFT, exp(+i q.r), for q = -q', q' in the chunk
         CK(launch_fftdf_phase_q(lq[sa], buf0, dQ + c0, nc, 1, grid, pr.d.mesh, -1.0, 1.0, nx, P->cs));
