@@ -2978,9 +2978,10 @@ static dmet_status_t jk_residues(dmet_emb_plan_s* P, Prob& pr, int n, const doub
   if ((long long)naux * n > INT_MAX / 4 || nk > 65535) return DMET_OK;
   const size_t wq = (size_t)naux * nn * 16;  // W of one q
   const int cq = (int)std::max<size_t>(1, std::min<size_t>(nk, ((size_t)256 << 20) / wq));
-  const long long tiles = ((n + 127) / 128) * (long long)((2 * n + 255) / 256);
-  const int want = (int)((4LL * P->sms + 15 * cq * tiles - 1) / (15 * cq * tiles));
-  const int pl = std::max(1, naux / std::min(naux, want)), parts = (naux + pl - 1) / pl;
+  // Parts of some 480 K (complex): as many parts then fit a chunk of the scratch as its conversions (one CTA per 32
+  // rows and part) need to fill the GPU twice. h-BN-shaped, 10 parts of K = 2912 a chunk: each conversion took
+  // 306 or 258 us at 130 CTAs, two thirds of the call.
+  const int pl = std::max(1, std::min(naux, 480 / n)), parts = (naux + pl - 1) / pl;
   if ((long long)cq * parts > 65535) return DMET_OK;
   ZgemmArgs z1 = zargs(), z2 = zargs();
   z1.A = gamma;  // opA(b, l) = gamma[l][b], opB(l, (P, a)) = L[(P, a)][l], stored at [P][b][a]
