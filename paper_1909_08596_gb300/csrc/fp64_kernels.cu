@@ -3,11 +3,10 @@
 // GB300 executes FP64 fused multiply-adds on the CUDA cores at a small fraction of its
 // FP32 rate, so the plain-FP64 path is bound by the DFMA pipe, not by memory: every
 // kernel here keeps its operands in shared memory and registers and spends its issue
-// slots on DFMAs. Tiles are 64x64 outputs per 256-thread CTA (4x4 outputs per thread);
-// a warp owns 8 consecutive rows of the tile and skips its FMAs when all of them lie
-// past the matrix edge, so small dimensions (n_emb) waste no DFMAs beyond a multiple of 8.
+// slots on DFMAs. (The large products run on the tensor cores instead: rns.cu.)
 
 #include <cuda_runtime.h>
+#include <limits.h>
 #include <math.h>
 #include <stdint.h>
 
@@ -17,22 +16,27 @@ namespace dmet {
 
 namespace {
 
-constexpr int TM = 64;   // tile rows
-constexpr int TN = 64;   // tile columns
-constexpr int ZBK = 8;   // complex k-step
-constexpr int DBK = 16;  // real k-step
+constexpr int TT = 16;  // tile rows and columns
+constexpr int TK = 16;  // complex k-step
+constexpr int DK = 64;  // real k-step
 
 __device__ __forceinline__ long long map2(int x, int div, long long hi, long long lo) {
   return (long long)(x / div) * hi + (long long)(x % div) * lo;
 }
 
+// The FP64 pipe takes 16 clocks of an SM per warp FMA, so a tile's loads and shared-memory reads hide behind it at
+// any tile size and the split of the work decides: 16 x 16 tiles, one output per thread, spread a small product
+// over all SMs (16 x 640 x 16 in four batches: 39 us with 64 x 64 tiles of 4 x 4 outputs per thread, 13 so; 64 x 256 x
+// 1024: 4134 and 283 us; 104 x 5720 x 26 in 20 batches, which fills the GPU either way: 2604 and 2124 us, less waste on
+// ragged edges; 104 x 22 880 x 520 in four: 33.1 and 33.8 ms); the next K step's values load while the current one is summed.
 template <int AL, bool CJ, int BL>
-__global__ void __launch_bounds__(256, 2) zgemm_fp64_kernel(const ZgemmArgs d) {
-  __shared__ __align__(16) double2 As[ZBK][TM];
-  __shared__ __align__(16) double2 Bs[ZBK][TN];
-  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-  const int m0 = blockIdx.y * TM, n0 = blockIdx.x * TN;
-  if (d.lower && n0 >= m0 + TM) return;  // the whole CTA leaves together
+__global__ void __launch_bounds__(256) zgemm_fp64_kernel(const ZgemmArgs d) {
+  __shared__ __align__(16) double2 As[2][TK][TT + 1];
+  __shared__ __align__(16) double2 Bs[2][TK][TT + 1];
+  const int tid = threadIdx.x, tx = tid & (TT - 1), ty = tid / TT;
+  const unsigned nt = (unsigned)(d.N + TT - 1) / TT;
+  const int m0 = (int)(blockIdx.x / nt) * TT, n0 = (int)(blockIdx.x % nt) * TT;
+  if (d.lower && n0 >= m0 + TT) return;  // the whole CTA leaves together
   const double2* A = d.A;
   const double2* B = d.B;
   double2* D = d.D;
@@ -48,152 +52,102 @@ __global__ void __launch_bounds__(256, 2) zgemm_fp64_kernel(const ZgemmArgs d) {
     B += (long long)blockIdx.z * d.sB;
     D += (long long)blockIdx.z * d.sD;
   }
-  const bool active = (m0 + (tid >> 5) * 8) < d.M;
-
-  double2 acc[4][4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = make_double2(0.0, 0.0);
-
-  for (int k0 = 0; k0 < K; k0 += ZBK) {
-#pragma unroll
-    for (int r = 0; r < 2; ++r) {
-      const int e = tid + r * 256;
-      int kk, mm, nn;
-      if (AL == A_KM) { kk = e >> 6; mm = e & 63; } else { mm = e >> 3; kk = e & 7; }
-      int gk = k0 + kk, gm = m0 + mm;
-      double2 v = make_double2(0.0, 0.0);
-      if (gk < K && gm < d.M) v = (AL == A_KM) ? A[gk * d.lda + gm] : A[gm * d.lda + gk];
-      if (CJ) v.y = -v.y;
-      As[kk][mm] = v;
-      if (BL == B_KN) { kk = e >> 6; nn = e & 63; } else { nn = e >> 3; kk = e & 7; }
-      gk = k0 + kk;
-      const int gn = n0 + nn;
-      double2 w = make_double2(0.0, 0.0);
-      if (gk < K && gn < d.N) w = (BL == B_KN) ? B[gk * d.ldb + gn] : B[gn * d.ldb + gk];
-      Bs[kk][nn] = w;
-    }
+  // thread (ty, tx) loads element (k = ty, m = tx) of a K-major operand, (k = tx, m = ty) of the other kind
+  const int ak = AL == A_KM ? ty : tx, am = AL == A_KM ? tx : ty, bk = BL == B_KN ? ty : tx, bn = BL == B_KN ? tx : ty;
+  const bool aok = m0 + am < d.M, bok = n0 + bn < d.N;
+  const double2* Ap = A + (AL == A_KM ? ak * d.lda + m0 + am : (m0 + am) * d.lda + ak);
+  const double2* Bp = B + (BL == B_KN ? bk * d.ldb + n0 + bn : (n0 + bn) * d.ldb + bk);
+  const long long as = AL == A_KM ? TK * d.lda : TK, bs = BL == B_KN ? TK * d.ldb : TK;
+  const double2 zero = make_double2(0.0, 0.0);
+  double2 av = aok && ak < K ? *Ap : zero, bv = bok && bk < K ? *Bp : zero;
+  const bool active = m0 + (tid >> 5) * (32 / TT) < d.M;
+  double re = 0.0, im = 0.0;
+  for (int k0 = 0, buf = 0; k0 < K; k0 += TK, buf ^= 1) {
+    if (CJ) av.y = -av.y;
+    As[buf][ak][am] = av;
+    Bs[buf][bk][bn] = bv;
     __syncthreads();
+    Ap += as;
+    Bp += bs;
+    av = aok && k0 + TK + ak < K ? *Ap : zero;
+    bv = bok && k0 + TK + bk < K ? *Bp : zero;
     if (active) {
-#pragma unroll
-      for (int kk = 0; kk < ZBK; ++kk) {
-        double2 a[4], b[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) a[i] = As[kk][ty * 4 + i];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) b[j] = Bs[kk][tx * 4 + j];
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            acc[i][j].x = fma(a[i].x, b[j].x, acc[i][j].x);
-            acc[i][j].x = fma(-a[i].y, b[j].y, acc[i][j].x);
-            acc[i][j].y = fma(a[i].x, b[j].y, acc[i][j].y);
-            acc[i][j].y = fma(a[i].y, b[j].x, acc[i][j].y);
-          }
+      const int kn = min(TK, K - k0);
+#pragma unroll 8
+      for (int kk = 0; kk < kn; ++kk) {
+        const double2 a = As[buf][kk][ty], b = Bs[buf][kk][tx];
+        re = fma(a.x, b.x, re);
+        im = fma(a.x, b.y, im);
+        re = fma(-a.y, b.y, re);
+        im = fma(a.y, b.x, im);
       }
     }
-    __syncthreads();
   }
-  if (!active) return;
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int m = m0 + ty * 4 + i;
-    if (m >= d.M) continue;
-    const long long rm = map2(m, d.dm_div, d.dm_hi, d.dm_lo);
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int n = n0 + tx * 4 + j;
-      if (n >= d.N) continue;
-      const long long addr = rm + map2(n, d.dn_div, d.dn_hi, d.dn_lo);
-      double2 v = make_double2(d.alpha * acc[i][j].x, d.alpha * acc[i][j].y);
-      if (d.beta) {
-        const double2 o = D[addr];
-        v.x += o.x;
-        v.y += o.y;
-      }
-      D[addr] = v;
-    }
+  const int m = m0 + ty, n = n0 + tx;
+  if (m >= d.M || n >= d.N) return;
+  const long long addr = map2(m, d.dm_div, d.dm_hi, d.dm_lo) + map2(n, d.dn_div, d.dn_hi, d.dn_lo);
+  double2 v = make_double2(d.alpha * re, d.alpha * im);
+  if (d.beta) {
+    const double2 o = D[addr];
+    v.x += o.x;
+    v.y += o.y;
   }
+  D[addr] = v;
 }
 
-__global__ void __launch_bounds__(256, 2) dsyrk_fp64_kernel(const DsyrkArgs d) {
-  __shared__ __align__(16) double Xs[DBK][TM];
-  __shared__ __align__(16) double Ys[DBK][TN];
-  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+__global__ void __launch_bounds__(256) dsyrk_fp64_kernel(const DsyrkArgs d) {
+  __shared__ double Xs[2][DK][TT + 1];
+  __shared__ double Ys[2][DK][TT + 1];
+  const int tid = threadIdx.x, tx = tid & (TT - 1), ty = tid / TT;
   int m0, n0;
   if (d.mode == 0) {
     const long long t = blockIdx.x;
     long long ti = (long long)((sqrt(8.0 * (double)t + 1.0) - 1.0) * 0.5);
     while (ti * (ti + 1) / 2 > t) --ti;
     while ((ti + 1) * (ti + 2) / 2 <= t) ++ti;
-    m0 = (int)ti * TM;
-    n0 = (int)(t - ti * (ti + 1) / 2) * TN;
+    m0 = (int)ti * TT;
+    n0 = (int)(t - ti * (ti + 1) / 2) * TT;
   } else {
-    m0 = blockIdx.y * TM;
-    n0 = blockIdx.x * TN;
+    const unsigned nt = (unsigned)(d.N + TT - 1) / TT;
+    m0 = (int)(blockIdx.x / nt) * TT;
+    n0 = (int)(blockIdx.x % nt) * TT;
   }
   const double* Y = d.mode == 0 ? d.X : d.Y;
   const long long ldy = d.mode == 0 ? d.ldx : d.ldy;
-  const int wrow = m0 + (tid >> 5) * 8;
-  // In the packed mode a warp whose 8 rows all lie above the tile's columns has no m >= n.
-  const bool active = wrow < d.M && (d.mode != 0 || wrow + 7 >= n0);
-
-  double acc[4][4];
+  const bool xok = m0 + tx < d.M, yok = n0 + tx < d.N;
+  const double* Xp = d.X + ty * d.ldx + m0 + tx;
+  const double* Yp = Y + ty * ldy + n0 + tx;
+  constexpr int R = DK / TT;
+  double xv[R], yv[R];
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+  for (int r = 0; r < R; ++r) {
+    const int k = ty + r * TT;
+    xv[r] = xok && k < d.K ? Xp[r * TT * d.ldx] : 0.0;
+    yv[r] = yok && k < d.K ? Yp[r * TT * ldy] : 0.0;
+  }
+  double acc = 0.0;
+  for (int k0 = 0, buf = 0; k0 < d.K; k0 += DK, buf ^= 1) {
 #pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = 0.0;
-
-  for (int k0 = 0; k0 < d.K; k0 += DBK) {
-#pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      const int e = tid + r * 256;
-      const int kk = e >> 6, mm = e & 63;
-      const int gk = k0 + kk;
-      double v = 0.0, w = 0.0;
-      if (gk < d.K && m0 + mm < d.M) v = d.X[gk * d.ldx + m0 + mm];
-      if (gk < d.K && n0 + mm < d.N) w = Y[gk * ldy + n0 + mm];
-      Xs[kk][mm] = v;
-      Ys[kk][mm] = w;
+    for (int r = 0; r < R; ++r) {
+      Xs[buf][ty + r * TT][tx] = xv[r];
+      Ys[buf][ty + r * TT][tx] = yv[r];
     }
     __syncthreads();
-    if (active) {
+    Xp += DK * d.ldx;
+    Yp += DK * ldy;
 #pragma unroll
-      for (int kk = 0; kk < DBK; ++kk) {
-        double a[4], b[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) a[i] = Xs[kk][ty * 4 + i];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) b[j] = Ys[kk][tx * 4 + j];
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-          for (int j = 0; j < 4; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
-      }
+    for (int r = 0; r < R; ++r) {
+      const int k = k0 + DK + ty + r * TT;
+      xv[r] = xok && k < d.K ? Xp[r * TT * d.ldx] : 0.0;
+      yv[r] = yok && k < d.K ? Yp[r * TT * ldy] : 0.0;
     }
-    __syncthreads();
+    const int kn = min(DK, d.K - k0);
+#pragma unroll 16
+    for (int kk = 0; kk < kn; ++kk) acc = fma(Xs[buf][kk][ty], Ys[buf][kk][tx], acc);
   }
-  if (!active) return;
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int m = m0 + ty * 4 + i;
-    if (m >= d.M) continue;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int n = n0 + tx * 4 + j;
-      if (n >= d.N) continue;
-      long long addr;
-      if (d.mode == 0) {
-        if (n > m) continue;
-        addr = (long long)m * (m + 1) / 2 + n;
-      } else {
-        addr = (long long)m * d.ldo + n;
-      }
-      d.out[addr] += d.alpha * acc[i][j];
-    }
-  }
+  const int m = m0 + ty, n = n0 + tx;
+  if (m >= d.M || n >= d.N || (d.mode == 0 && n > m)) return;
+  d.out[d.mode == 0 ? (long long)m * (m + 1) / 2 + n : (long long)m * d.ldo + n] += d.alpha * acc;
 }
 
 __global__ void gather_orbitals_kernel(const double2* __restrict__ C, double2* __restrict__ Crep,
@@ -430,7 +384,9 @@ __global__ void pack_s4_kernel(const double2* __restrict__ full, int na, int nb,
 
 cudaError_t launch_zgemm(const ZgemmArgs& a, int a_layout, bool conj_a, int b_layout, cudaStream_t s) {
   if (a.M <= 0 || a.N <= 0 || a.batch <= 0) return cudaSuccess;
-  const dim3 grid((a.N + TN - 1) / TN, (a.M + TM - 1) / TM, a.batch);
+  const long long tiles = (long long)((a.N + TT - 1) / TT) * ((a.M + TT - 1) / TT);
+  if (tiles > INT_MAX) return cudaErrorInvalidValue;
+  const dim3 grid((unsigned)tiles, 1, a.batch);
   if (a_layout == A_KM && conj_a && b_layout == B_KN)
     zgemm_fp64_kernel<A_KM, true, B_KN><<<grid, 256, 0, s>>>(a);
   else if (a_layout == A_KM && !conj_a && b_layout == B_KN)
@@ -444,14 +400,9 @@ cudaError_t launch_zgemm(const ZgemmArgs& a, int a_layout, bool conj_a, int b_la
 
 cudaError_t launch_dsyrk(const DsyrkArgs& a, cudaStream_t s) {
   if (a.M <= 0 || a.N <= 0) return cudaSuccess;
-  dim3 grid;
-  if (a.mode == 0) {
-    const long long nt = (a.M + TM - 1) / TM;
-    grid = dim3((unsigned)(nt * (nt + 1) / 2), 1, 1);
-  } else {
-    grid = dim3((a.N + TN - 1) / TN, (a.M + TM - 1) / TM, 1);
-  }
-  dsyrk_fp64_kernel<<<grid, 256, 0, s>>>(a);
+  const long long mt = (a.M + TT - 1) / TT, nt = (a.N + TT - 1) / TT, tiles = a.mode == 0 ? mt * (mt + 1) / 2 : mt * nt;
+  if (tiles > INT_MAX) return cudaErrorInvalidValue;
+  dsyrk_fp64_kernel<<<(unsigned)tiles, 256, 0, s>>>(a);
   return cudaGetLastError();
 }
 

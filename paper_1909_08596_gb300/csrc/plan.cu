@@ -2855,6 +2855,7 @@ dmet_status_t dmet_emb_fock(dmet_emb_plan_t P, int32_t problem, const void* F, c
   const size_t bW = (size_t)(nk * nao * n) * 16, bG = (size_t)(nk * n * n) * 16, bM = (size_t)(n * n) * 8;
   const size_t need = bW + bG + 3 * bM + 256;
   P->cs = P->stream;
+  P->W = &P->ws[P->ws_of[problem]];
   TRY(ensure(&P->fock_ws, &P->fock_ws_b, need));
   char* w = (char*)P->fock_ws;
   double2* W = (double2*)w;
@@ -2883,7 +2884,7 @@ dmet_status_t dmet_emb_fock(dmet_emb_plan_t P, int32_t problem, const void* F, c
     z.dm_lo = n;
     z.dn_lo = 1;
     z.batch = (int)nk;
-    CK(launch_zgemm(z, A_KM, true, B_KN, P->cs));
+    TRY(zgemm(P, t, z, A_KM, true, B_KN));
   }
   {
     // G[k] = C^k+ W[k]
@@ -2902,7 +2903,7 @@ dmet_status_t dmet_emb_fock(dmet_emb_plan_t P, int32_t problem, const void* F, c
     z.dm_lo = n;
     z.dn_lo = 1;
     z.batch = (int)nk;
-    CK(launch_zgemm(z, A_KM, true, B_KN, P->cs));
+    TRY(zgemm(P, t, z, A_KM, true, B_KN));
   }
   CK(launch_fock_reduce(G, (int)nk, (int)n, pr.ortho_scale, F0, P->cs));
   CK(cudaMemsetAsync(K, 0, bM, P->cs));

@@ -186,16 +186,16 @@ __device__ __forceinline__ int norm_scale(const RowNorm& n) {
   return kBeta - (n.e - 1023 + ((se + 2) >> 1));
 }
 
-// rint(x 2^s) as a two's-complement integer (round half away from zero), |result| <= 2^kBeta.
+// rint(x 2^s) as a two's-complement integer (round half away from zero), |result| <= 2^kBeta (so the binary point of
+// x's 53 bits moves left by at most 6).
 __device__ __forceinline__ long long to_int(double x, int s) {
-  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
-  const int e = (int)((b >> 52) & 0x7ff);
-  unsigned long long m = b & ((1ull << 52) - 1);
-  if (e) m |= 1ull << 52;
-  const int sh = (e ? e : 1) - 1075 + s;
-  if (sh >= 0) m <<= min(sh, 63);
-  else m = sh > -55 ? (m + (1ull << (-sh - 1))) >> -sh : 0ull;
-  return (long long)b < 0 ? -(long long)m : (long long)m;
+  const unsigned hi = (unsigned)__double2hiint(x);
+  const int e = (int)((hi >> 20) & 0x7ff);
+  const unsigned mh = (hi & 0xfffffu) | (e ? 0x100000u : 0u);
+  const unsigned long long m = (((unsigned long long)mh << 32) | (unsigned)__double2loint(x)) << 6;
+  const int r = min(max(1081 - s - (e ? e : 1), 0), 63);
+  const long long t = (long long)((m + ((1ull << r) >> 1)) >> r);
+  return (int)hi < 0 ? -t : t;
 }
 
 // Four signed 16-bit digits of a, as floats: a = sum c_j 2^(16 j).
@@ -217,15 +217,23 @@ __device__ __forceinline__ float residue(const float (&c)[4]) {
   return sym_mod(fmaf(c[3], w3, fmaf(c[2], w2, fmaf(c[1], w1, c[0]))), p, rp);
 }
 
-template <int SRC, int I>
-__device__ __forceinline__ void store_residues(const float (&cr)[4], const float (&ci)[4], __nv_bfloat16* dst,
-                                               long long smod, int Kp) {
+// The residues of one (re, im) or (k, k + 1) pair of each of RW rows, modulus by modulus (rows side by side: their
+// chains overlap and share the plane's address; off: byte offset of a row's pair in a plane, 2 KiB planes and up
+// to 4 GiB, or ~0 for a row that is not stored).
+template <int SRC, int RW, int I>
+__device__ __forceinline__ void store_residues(const float (&cr)[RW][4], const float (&ci)[RW][4],
+                                               const unsigned (&off)[RW], char* plane, long long smod, unsigned row2) {
   if constexpr (I < kMods) {
-    const float re = residue<I>(cr), im = residue<I>(ci);
-    const __nv_bfloat162 p = __floats2bfloat162_rn(re, SRC == SRC_COMPLEX2 ? -im : im);
-    *reinterpret_cast<__nv_bfloat162*>(dst) = p;
-    if constexpr (SRC == SRC_COMPLEX2) *reinterpret_cast<__nv_bfloat162*>(dst + Kp) = __floats2bfloat162_rn(im, re);
-    store_residues<SRC, I + 1>(cr, ci, dst + smod, smod, Kp);
+#pragma unroll
+    for (int i = 0; i < RW; ++i) {
+      const float re = residue<I>(cr[i]), im = residue<I>(ci[i]);
+      if (off[i] != ~0u) {
+        *reinterpret_cast<__nv_bfloat162*>(plane + off[i]) = __floats2bfloat162_rn(re, SRC == SRC_COMPLEX2 ? -im : im);
+        if constexpr (SRC == SRC_COMPLEX2)
+          *reinterpret_cast<__nv_bfloat162*>(plane + (off[i] + row2)) = __floats2bfloat162_rn(im, re);
+      }
+    }
+    store_residues<SRC, RW, I + 1>(cr, ci, off, plane + smod, smod, row2);
   }
 }
 
@@ -323,13 +331,15 @@ __global__ void __launch_bounds__(256) rns_convert_kernel(const ConvArgs a) {
       __syncthreads();
     }
     const int u = u0 + lane;
+    float cr[RW][4], ci[RW][4];
+    unsigned off[RW];
+#pragma unroll
     for (int i = 0; i < RW; ++i) {
       const int rl = warp * RW + i, r = r0 + rl;
-      if (r >= a.rows) break;
       double2 v = make_double2(0.0, 0.0);
       if (rowfast) {
         v = tile[lane][rl];
-      } else if (u < units) {
+      } else if (u < units && r < a.rows) {
         if constexpr (SRC == SRC_REAL) {
           v.x = src1[(long long)r * a.s_row + (long long)(2 * u) * a.s_k];
           if (2 * u + 1 < K) v.y = src1[(long long)r * a.s_row + (long long)(2 * u + 1) * a.s_k];
@@ -344,14 +354,11 @@ __global__ void __launch_bounds__(256) rns_convert_kernel(const ConvArgs a) {
         ai = to_int(v.y, s);
         if (SRC != SRC_REAL && a.conj) ai = -ai;
       }
-      float cr[4], ci[4];
-      digits(ar, cr);
-      digits(ai, ci);
-      if (u < upad) {
-        __nv_bfloat16* dst = a.R + (((long long)z * a.rows + r) * RR) * a.Kp + 2 * u;
-        store_residues<SRC, 0>(cr, ci, dst, a.smod, a.Kp);
-      }
+      digits(ar, cr[i]);
+      digits(ai, ci[i]);
+      off[i] = u < upad && r < a.rows ? (unsigned)((((long long)z * a.rows + r) * RR * a.Kp + 2 * u) * 2) : ~0u;
     }
+    store_residues<SRC, RW, 0>(cr, ci, off, reinterpret_cast<char*>(a.R), a.smod * 2, (unsigned)a.Kp * 2u);
   }
 }
 
@@ -883,20 +890,19 @@ size_t rns_need(const DsyrkArgs& a) {
   return rows * kp * 2 * kMods + (size_t)a.M * pad_to(a.N, 16) * kMods + rows * 4 + 65536;
 }
 
-// Where the line between the two lies (measured on shapes from 8 x 256 x 8 to 128 x 22 880 x 1024, single and
-// batched): the FP64 kernel takes 4.3 us per k and 64 x 64 complex tile and SM (a warp whose 8 rows all lie
-// outside issues none), 7 us more per launch; the residues take about 40 us for their four launches, 17 ps per
-// real result (reconstruction and epilogue) and 12 ps per converted real element, and the MMAs. A
-// 128 x 4096 product: K = 8, 41 against 55 us; K = 16, 76 against 56; K = 64, 279 against 66.
+// Where the line between the two lies (fitted to shapes from 8 x 256 x 8 to 128 x 22 880 x 1024, single and batched): the
+// FP64 kernel takes 0.27 us per k and 16 x 16 complex tile and SM (less where a tile has few rows); the residues
+// take 28 us for their four launches, 85 ns per k of a conversion that few CTAs share, 34 ps per complex
+// result (reconstruction and epilogue) and 12 ps per converted real element, and the MMAs. A 128 x 4096 product:
+// K = 8, 35 against 43 us; K = 16, 64 against 44; K = 64, 238 against 48.
 bool rns_takes_zgemm(const ZgemmArgs& a, const RnsCtx& c) {
   if (!c.scratch || a.lower || a.M <= 0 || a.N <= 0 || a.K <= 0 || a.batch <= 0) return false;
   const ZPlan p = zplan(a, A_KM, false, B_KN);
   if (p.col_bytes + 2 * kBK * (size_t)p.Kp * 2 * kMods + 256 * (size_t)p.ldy * kMods + (4 << 20) > c.bytes) return false;
-  const double ctas = (double)((a.M + 63) / 64) * ((a.N + 63) / 64) * a.batch;
-  const double fill = (double)pad_to(a.M, 8) / pad_to(a.M, 64);
-  const double fp64 = 7 + 4.3 * a.K * fill * std::ceil(ctas / c.sms);
+  const double ctas = std::ceil((double)((a.M + 15) / 16) * ((a.N + 15) / 16) * a.batch / c.sms);
+  const double fp64 = 5 + 0.27 * a.K * ctas * std::min(16, (a.M + 1) / 2 * 2) / 16.0;
   const double mn = (double)a.M * a.N * a.batch, conv = ((double)p.rows.rows + 2.0 * p.cols.rows) * p.Kp * a.batch;
-  return fp64 > 40 + 34e-6 * mn + 12e-6 * conv + 8.0 * kMods / 1.2e9 * mn * a.K;
+  return fp64 > 28 + 0.085 * a.K + 34e-6 * mn + 12e-6 * conv + 8.0 * kMods / 1.2e9 * mn * a.K;
 }
 
 cudaError_t rns_zgemm(const ZgemmArgs& a, int al, bool cj, int bl, const RnsCtx& c, cudaStream_t s, int* launches) {
@@ -982,11 +988,13 @@ cudaError_t rns_zgemm(const ZgemmArgs& a, int al, bool cj, int bl, const RnsCtx&
 
 bool rns_takes_dsyrk(const DsyrkArgs& a, const RnsCtx& c) {
   if (!c.scratch || a.M <= 0 || a.N <= 0 || a.K <= 0) return false;
-  // 1.08 us per k and 64 x 64 tile and SM on the FP64 pipe; a 64 x 64 result: K = 64, 75 against 32 us
-  const double tm = (a.M + 63) / 64, tn = (a.N + 63) / 64, ctas = a.mode == 0 ? tm * (tm + 1) / 2 : tm * tn;
-  const double fp64 = 7 + 1.08 * a.K * std::ceil(ctas / c.sms), mn = (a.mode == 0 ? 0.5 : 1.0) * a.M * (double)a.N;
+  // 68 ns per k and 16 x 16 tile and SM on the FP64 pipe, against launches, conversions and results as above: a
+  // 64 x 64 result, K = 256: 23 against 32 us, K = 1024: 75 against 50
+  const double tm = (a.M + 15) / 16, tn = (a.N + 15) / 16, ctas = a.mode == 0 ? tm * (tm + 1) / 2 : tm * tn;
+  const double fp64 = 5 + 0.068 * a.K * std::ceil(ctas / c.sms), mn = (a.mode == 0 ? 0.5 : 1.0) * a.M * (double)a.N;
   const double conv = ((double)a.M + (a.mode ? a.N : 0)) * a.K;
-  if (fp64 < 40 + 17e-6 * mn + 12e-6 * conv + 2.0 * kMods / 1.2e9 * mn * a.K) return false;
+  if (fp64 < 26 + (a.mode ? 8 : 0) + 0.024 * a.K + 17e-6 * mn + 12e-6 * conv + 2.0 * kMods / 1.2e9 * mn * a.K)
+    return false;
   // at least one K block of both operands and 256 rows of Y
   const size_t ops = ((size_t)a.M + (a.mode ? a.N : 0)) * kBK * 2 * kMods, y = (size_t)256 * pad_to(a.N, 16) * kMods;
   return ops + y + ((size_t)a.M + a.N) * 4 + (1 << 20) <= c.bytes;
