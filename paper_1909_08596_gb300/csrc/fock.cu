@@ -23,76 +23,124 @@ __global__ void fock_reduce_kernel(const double2* __restrict__ G, int nk, int n,
   }
 }
 
-// One block per pair row A = {i, k}, i >= k: the block stages the row of the packed ERI in shared
-// memory, V[B] = (ik|B) for every pair B (the element at max(A,B)(max+1)/2 + min), and then
-//   thread j:  K_ij += sum_l (ik|lj) gamma_kl   and, for i != k,   K_kj += sum_l (ki|lj) gamma_il,
-//   all:       J_ik  = J_ki = sum_{l,j} (ik|lj) gamma_jl = sum_B V[B] gamma_B (2 - delta_B),
-// with V[{l, j}] = (ik|lj) = (ki|lj) (real orbitals). Each row is read once; the exchange rows are
-// added to K (which starts at zero) with one atomic add per element and block.
-__global__ void __launch_bounds__(256) coulomb_exchange_kernel(const double* __restrict__ eri,
-                                                               const double* __restrict__ gamma, int n,
-                                                               double* __restrict__ J, double* __restrict__ K) {
-  extern __shared__ double sm[];
-  const long long npair = (long long)n * (n + 1) / 2;
-  double* row = sm;             // [npair]
-  double* gi = sm + npair;      // gamma row i [n]
-  double* gk = gi + n;          // gamma row k [n]
-  __shared__ double red[8];
-  for (long long A = blockIdx.x; A < npair; A += gridDim.x) {
-    // (i, k) of A: i = floor((sqrt(8A + 1) - 1) / 2), made exact
-    long long il = (long long)((sqrt(8.0 * (double)A + 1.0) - 1.0) * 0.5);
-    while (il * (il + 1) / 2 > A) --il;
-    while ((il + 1) * (il + 2) / 2 <= A) ++il;
-    const int i = (int)il, k = (int)(A - il * (il + 1) / 2);
-    const long long rowA = A * (A + 1) / 2;
-    __syncthreads();  // the previous row's readers are done
-    for (long long B = threadIdx.x; B < npair; B += blockDim.x)
-      row[B] = B <= A ? eri[rowA + B] : eri[B * (B + 1) / 2 + A];
-    for (int t = threadIdx.x; t < n; t += blockDim.x) {
-      gi[t] = gamma[(long long)i * n + t];
-      gk[t] = gamma[(long long)k * n + t];
-    }
-    __syncthreads();
-    // The exchange rows: nsplit groups of n threads each take a share of l for every j (so that a
-    // block of 256 threads keeps busy when n is below 256); their partial sums meet in the atomic adds.
-    // (Pair indices fit 32 bits: n <= 2047.)
-    const int nsplit = n < (int)blockDim.x ? (int)blockDim.x / n : 1;
-    for (int t = threadIdx.x; t < nsplit * n; t += blockDim.x) {
-      const int j = t % n, h = t / n;
-      const int l0 = h * n / nsplit, l1 = (h + 1) * n / nsplit;
-      double si = 0.0, sk = 0.0;
-      const int jj = j * (j + 1) / 2;
-      for (int l = l0; l < l1; ++l) {
-        const double v = row[l >= j ? l * (l + 1) / 2 + j : jj + l];
-        si = fma(v, gk[l], si);
-        sk = fma(v, gi[l], sk);
-      }
-      atomicAdd(&K[(long long)i * n + j], si);
-      if (i != k) atomicAdd(&K[(long long)k * n + j], sk);
-    }
-    double js = 0.0;
-    for (int l = threadIdx.x >> 5; l < n; l += blockDim.x >> 5) {
-      const long long base = (long long)l * (l + 1) / 2;
-      for (int j = threadIdx.x & 31; j <= l; j += 32)
-        js = fma(row[base + j], (l == j ? 1.0 : 2.0) * gamma[(long long)l * n + j], js);
-    }
-    for (int o = 16; o; o >>= 1) js += __shfl_xor_sync(0xffffffffu, js, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = js;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      double t = 0.0;
-      for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[w];
-      J[(long long)i * n + k] = t;
-      J[(long long)k * n + i] = t;
-    }
+// The FP64 pipe bounds both sums over the packed ERI (an FMA of a warp takes 16 clocks of an SM), so each stored
+// element is used along its row together with its electron-exchange mirror: K = K' + K'^T, where K' takes
+// the elements (A, B) with B < A and half of A = B, A = {i, k} giving the index of K' and B = {l, j} the other;
+// and J_A = sum_{B <= A} V_AB w_B along the rows, plus sum_{A' > A} V_A'A w_A' down the columns, w_B = gamma_B (2 -
+// delta_B). n = 104, staging whole rows (their second halves read down the columns): 562 us for both; so 250 for the rows and 71 for the columns.
+
+__global__ void pair_weights_kernel(const double* __restrict__ gamma, int n, double* __restrict__ w) {
+  for (int x = blockIdx.x * blockDim.x + threadIdx.x; x < n * n; x += gridDim.x * blockDim.x) {
+    const int l = x / n, j = x - l * n;
+    if (j <= l) w[l * (l + 1) / 2 + j] = (l == j ? 1.0 : 2.0) * gamma[x];
   }
 }
 
-// out = F0 - (J - K / 2)
+// part[y][B] = sum of V_AB w_A over share y of the rows A > B: a thread per column, rows in order (a warp reads 256
+// contiguous bytes of each), four running sums.
+constexpr int kColShares = 16;
+__global__ void __launch_bounds__(256) coulomb_columns_kernel(const double* __restrict__ eri, const double* __restrict__ w,
+                                                              int npair, double* __restrict__ part) {
+  const int B = blockIdx.x * 256 + threadIdx.x, first = blockIdx.x * 256 + 1, span = npair - first;
+  const int a0 = first + (int)((long long)span * blockIdx.y / kColShares);
+  const int a1 = first + (int)((long long)span * (blockIdx.y + 1) / kColShares);
+  double s[4] = {0.0, 0.0, 0.0, 0.0};
+  const double* p = eri + (long long)a0 * (a0 + 1) / 2 + B;
+  int A = a0;
+  for (; A + 4 <= a1; A += 4) {
+    double v[4];
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      v[r] = B < A + r ? *p : 0.0;
+      p += A + r + 1;
+    }
+#pragma unroll
+    for (int r = 0; r < 4; ++r) s[r] = fma(v[r], w[A + r], s[r]);
+  }
+  for (; A < a1; ++A) {
+    if (B < A) s[0] = fma(*p, w[A], s[0]);
+    p += A + 1;
+  }
+  if (B < npair) part[(long long)blockIdx.y * npair + B] = (s[0] + s[1]) + (s[2] + s[3]);
+}
+
+// One CTA per pair row A = {i, k}, i >= k, long rows first: the row's elements B <= A in shared memory (the last one
+// halved, the rest of the pairs {i, j} zero), then thread (h, j), j <= i, over its share h of l <= i:
+//   K'_ij += sum_l (ik|lj) gamma_kl   and, for i != k,   K'_kj += sum_l (ki|lj) gamma_il,
+// and the row's share of J_A. The rows' sums meet in eight copies of K' (a long chain of additions into one
+// rounds sqrt(8) times as much).
+constexpr int kExchangeCopies = 8;
+__global__ void __launch_bounds__(256) exchange_kernel(const double* __restrict__ eri, const double* __restrict__ gamma,
+                                                       const double* __restrict__ w, int n, double* __restrict__ J,
+                                                       double* __restrict__ K) {
+  extern __shared__ double sm[];
+  __shared__ double red[8];
+  const int npair = n * (n + 1) / 2, A = npair - 1 - (int)blockIdx.x;
+  int i = (int)((sqrtf(8.f * (float)A + 1.f) - 1.f) * 0.5f);
+  while (i * (i + 1) / 2 > A) --i;
+  while ((i + 1) * (i + 2) / 2 <= A) ++i;
+  const int k = A - i * (i + 1) / 2, m = i + 1, len = m * (m + 1) / 2;
+  double* row = sm;
+  double* gi = sm + len;
+  double* gk = gi + m;
+  const double* src = eri + (long long)A * (A + 1) / 2;
+  double js = 0.0;
+  for (int B = threadIdx.x; B < len; B += 256) {
+    const double v = B <= A ? src[B] : 0.0;
+    row[B] = B == A ? 0.5 * v : v;
+    if (B <= A) js = fma(v, w[B], js);
+  }
+  for (int t = threadIdx.x; t < m; t += 256) {
+    gi[t] = gamma[i * n + t];
+    gk[t] = gamma[k * n + t];
+  }
+  __syncthreads();
+  const int nsplit = m < 256 ? 256 / m : 1;
+  double* Kc = K + (long long)(A % kExchangeCopies) * n * n;
+  for (int t = threadIdx.x; t < nsplit * m; t += 256) {
+    const int h = t / m, j = t - h * m;
+    const int l0 = h * m / nsplit, l1 = (h + 1) * m / nsplit, lm = min(max(j, l0), l1);
+    double si = 0.0, sk = 0.0;
+    const double* p = row + j * (j + 1) / 2;
+#pragma unroll 4
+    for (int l = l0; l < lm; ++l) {
+      si = fma(p[l], gk[l], si);
+      sk = fma(p[l], gi[l], sk);
+    }
+    const double* q = row + lm * (lm + 1) / 2 + j;
+#pragma unroll 4
+    for (int l = lm; l < l1; ++l) {
+      si = fma(*q, gk[l], si);
+      sk = fma(*q, gi[l], sk);
+      q += l + 1;
+    }
+    atomicAdd(&Kc[i * n + j], si);
+    if (i != k) atomicAdd(&Kc[k * n + j], sk);
+  }
+#pragma unroll
+  for (int o = 16; o; o >>= 1) js += __shfl_xor_sync(0xffffffffu, js, o);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = js;
+  __syncthreads();
+  if (threadIdx.x == 0)
+    J[A] = ((red[0] + red[1]) + (red[2] + red[3])) + ((red[4] + red[5]) + (red[6] + red[7]));
+}
+
+// out = F0 - (J - K / 2), J = the rows' shares plus the columns', K = sum of the copies of K' + K'^T
 __global__ void fock_combine_kernel(const double* __restrict__ F0, const double* __restrict__ J,
-                                    const double* __restrict__ K, int nn, double* __restrict__ out) {
-  for (int x = blockIdx.x * blockDim.x + threadIdx.x; x < nn; x += gridDim.x * blockDim.x)
-    out[x] = F0[x] - (J[x] - 0.5 * K[x]);
+                                    const double* __restrict__ part, const double* __restrict__ K, int n,
+                                    double* __restrict__ out) {
+  const int npair = n * (n + 1) / 2;
+  for (int x = blockIdx.x * blockDim.x + threadIdx.x; x < n * n; x += gridDim.x * blockDim.x) {
+    const int a = x / n, b = x - a * n, i = max(a, b), j = min(a, b), B = i * (i + 1) / 2 + j;
+    double c[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll
+    for (int y = 0; y < kColShares; ++y) c[y & 3] += part[(long long)y * npair + B];
+    double e[kExchangeCopies];
+#pragma unroll
+    for (int h = 0; h < kExchangeCopies; ++h) e[h] = K[h * n * n + x] + K[h * n * n + b * n + a];
+    const double ex = ((e[0] + e[1]) + (e[2] + e[3])) + ((e[4] + e[5]) + (e[6] + e[7]));
+    out[x] = F0[x] - ((J[B] + ((c[0] + c[1]) + (c[2] + c[3]))) - 0.5 * ex);
+  }
 }
 
 inline int blocks_for(long long total, int threads, int cap) {
@@ -218,25 +266,31 @@ cudaError_t launch_fock_reduce(const double2* G, int nk, int n, double s, double
   return cudaGetLastError();
 }
 
-cudaError_t launch_coulomb_exchange(const double* eri, const double* gamma, int n, double* J, double* K,
+int exchange_copies() { return kExchangeCopies; }
+
+size_t coulomb_scratch(int n) { return (size_t)(kColShares + 1) * ((size_t)n * (n + 1) / 2) * sizeof(double); }
+
+cudaError_t launch_coulomb_exchange(const double* eri, const double* gamma, int n, double* J, double* K, double* scratch,
                                     cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
   if (n > 1024) return cudaErrorInvalidValue;
   const long long npair = (long long)n * (n + 1) / 2;
   const size_t smem = (size_t)(npair + 2 * n) * sizeof(double);
-  if (smem > 227 * 1024) return cudaErrorInvalidValue;  // the caller checks the size first
-  if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(coulomb_exchange_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (smem > 227 * 1024 - 64) return cudaErrorInvalidValue;  // the caller checks the size first
+  if (smem > 48 * 1024 - 64) {
+    cudaError_t e = cudaFuncSetAttribute(exchange_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
   }
-  const int grid = (int)(npair < 152 * 16 ? npair : 152 * 16);
-  coulomb_exchange_kernel<<<grid, 256, smem, st>>>(eri, gamma, n, J, K);
+  double* w = scratch + kColShares * npair;
+  pair_weights_kernel<<<blocks_for((long long)n * n, 256, 152), 256, 0, st>>>(gamma, n, w);
+  coulomb_columns_kernel<<<dim3((unsigned)((npair + 255) / 256), kColShares), 256, 0, st>>>(eri, w, (int)npair, scratch);
+  exchange_kernel<<<(unsigned)npair, 256, smem, st>>>(eri, gamma, w, n, J, K);
   return cudaGetLastError();
 }
 
-cudaError_t launch_fock_combine(const double* F0, const double* J, const double* K, int n, double* out,
-                                cudaStream_t st) {
-  fock_combine_kernel<<<blocks_for((long long)n * n, 256, 152 * 8), 256, 0, st>>>(F0, J, K, n * n, out);
+cudaError_t launch_fock_combine(const double* F0, const double* J, const double* scratch, const double* K, int n,
+                                double* out, cudaStream_t st) {
+  fock_combine_kernel<<<blocks_for((long long)n * n, 256, 152 * 8), 256, 0, st>>>(F0, J, scratch, K, n, out);
   return cudaGetLastError();
 }
 

@@ -74,12 +74,15 @@ cudaError_t launch_symmetrize(const double2* Z, double2* Lq, int nq, int naux, i
 // [2] |C|, [3] Hermiticity of L, [4] time reversal of L, [5] |L| (the last three component-wise).
 // The orthonormality reduction sums ng split-K partial products S_g = C_g^+ C_g first.
 // Embedding Fock matrix (fock.cu): F0 = s sum_k Re G[k]; J and K of gamma from the 8-fold packed
-// ERI (K must start at zero; n(n+1)/2 + n doubles of shared memory, so n <= 232); out = F0 - J + K/2.
+// ERI (J by rows, packed, with the columns' shares in the scratch; copies of K' with K = sum of K' + K'^T, which must
+// start at zero; n(n+1)/2 + 2 n doubles of shared memory, so n <= 232); out = F0 - J + K/2.
 cudaError_t launch_fock_reduce(const double2* G, int nk, int n, double s, double* F0, cudaStream_t st);
-cudaError_t launch_coulomb_exchange(const double* eri, const double* gamma, int n, double* J, double* K,
+size_t coulomb_scratch(int n);
+int exchange_copies();  // K' is [copies][n][n]
+cudaError_t launch_coulomb_exchange(const double* eri, const double* gamma, int n, double* J, double* K, double* scratch,
                                     cudaStream_t st);
-cudaError_t launch_fock_combine(const double* F0, const double* J, const double* K, int n, double* out,
-                                cudaStream_t st);
+cudaError_t launch_fock_combine(const double* F0, const double* J, const double* scratch, const double* K, int n,
+                                double* out, cudaStream_t st);
 // FFTDF (fftdf.cu): dst = s exp(sign i q.r) src over the cell grid ([r][x], x < nx), q the mesh point of
 // triple nq; buf[G][x] *= v[G].
 cudaError_t launch_fftdf_phase(const double2* src, double2* dst, const int grid[3], const int nq[3], const int mesh[3],

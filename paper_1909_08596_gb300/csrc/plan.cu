@@ -2853,7 +2853,8 @@ dmet_status_t dmet_emb_fock(dmet_emb_plan_t P, int32_t problem, const void* F, c
   const long long nk = pr.nk, nao = pr.nao, n = pr.n[0], npair = n * (n + 1) / 2;
   // scratch: W = F^k C^k [k][mu][j], G = C^k+ W [k][i][j], F0, J, K [n][n]
   const size_t bW = (size_t)(nk * nao * n) * 16, bG = (size_t)(nk * n * n) * 16, bM = (size_t)(n * n) * 8;
-  const size_t need = bW + bG + 3 * bM + 256;
+  const size_t bK = (size_t)exchange_copies() * bM;
+  const size_t need = bW + bG + 2 * bM + bK + coulomb_scratch((int)n) + 256;
   P->cs = P->stream;
   P->W = &P->ws[P->ws_of[problem]];
   TRY(ensure(&P->fock_ws, &P->fock_ws_b, need));
@@ -2863,10 +2864,10 @@ dmet_status_t dmet_emb_fock(dmet_emb_plan_t P, int32_t problem, const void* F, c
   double* F0 = (double*)(w + bW + bG);
   double* J = F0 + n * n;
   double* K = J + n * n;
-  // flops executed: the two complex GEMMs; per pair row {i, k}: 2 n^2 exchange and n(n+1)/2 Coulomb
-  // multiply-adds
-  Timed t(P, KC_FOCK, 8.0 * nk * (nao * nao * n + nao * n * n) + 2.0 * npair * (2.0 * n * n + npair),
-          16.0 * nk * (nao * nao + nao * n) + 8.0 * npair * (npair + 1) / 2 + 8.0 * n * n * 2, 5);
+  double* cols = K + exchange_copies() * n * n;
+  // flops executed: the two complex GEMMs; per stored ERI element four exchange and two Coulomb multiply-adds
+  Timed t(P, KC_FOCK, 8.0 * nk * (nao * nao * n + nao * n * n) + 6.0 * npair * (npair + 1.0),
+          16.0 * nk * (nao * nao + nao * n) + 8.0 * npair * (npair + 1) / 2 + 8.0 * n * n * 2, 7);
   {
     // W[k] = F^k C^k: opA(mu, nu) = conj(F[k][nu][mu]) = F[k][mu][nu] (F^k is Hermitian)
     ZgemmArgs z = zargs();
@@ -2906,9 +2907,9 @@ dmet_status_t dmet_emb_fock(dmet_emb_plan_t P, int32_t problem, const void* F, c
     TRY(zgemm(P, t, z, A_KM, true, B_KN));
   }
   CK(launch_fock_reduce(G, (int)nk, (int)n, pr.ortho_scale, F0, P->cs));
-  CK(cudaMemsetAsync(K, 0, bM, P->cs));
-  CK(launch_coulomb_exchange(eri, gamma, (int)n, J, K, P->cs));
-  CK(launch_fock_combine(F0, J, K, (int)n, fock_out, P->cs));
+  CK(cudaMemsetAsync(K, 0, bK, P->cs));
+  CK(launch_coulomb_exchange(eri, gamma, (int)n, J, K, cols, P->cs));
+  CK(launch_fock_combine(F0, J, cols, K, (int)n, fock_out, P->cs));
   return DMET_OK;
 }
 
