@@ -112,30 +112,38 @@ __device__ __forceinline__ double warp_sum(double v) {
 }
 
 // One-sided Jacobi SVD (Hestenes 1958; the rotation angle as in Rutishauser's symmetric Jacobi
-// method) of the m x n_val block A (column-major), on one cluster of kBathCluster CTAs: CTA rank
-// r owns the rows [r mc, (r + 1) mc) of every column (mc = ceil(m / kBathCluster)), in shared
+// method) of the m x n_val block A (column-major), on one cluster of CS CTAs: CTA rank
+// r owns the rows [r mc, (r + 1) mc) of every column (mc = ceil(m / CS)), in shared
 // memory when they fit, else in place in global memory. A sweep visits every column pair in
 // n_pad - 1 rounds of the round-robin ordering (n_pad = n_val rounded up to even; the pad column
-// never rotates), one warp per pair of a round (the FP64 pipe of a sub-partition is charged per
-// warp instruction, idle lanes included, so the pairs go to different warps and the warps of a
-// round to different sub-partitions). Per round each CTA forms
-// the pair's three dot products over its rows, the cluster barrier publishes them, and every CTA
-// adds the partials in the same fixed order (the same numbers in the same order, so every CTA
-// takes the same rotation and the same convergence decision, and all pass the same barriers),
-// then rotates its own rows. The partials alternate between two buffers, so one barrier per
-// round suffices. The rotation angle is taken in FP32 and the rotation then made orthogonal in
-// FP64 (an angle off by 1e-7 relative leaves a cosine 1e-7 times the old one, which the next
-// sweep removes; the rotation itself never loses orthogonality). After convergence
+// never rotates), lp lanes per pair. Per round each CTA forms the pair's dot product over its rows, the cluster
+// barrier publishes it, and every CTA adds the partials in the same fixed order (the same numbers in the
+// same order, so every CTA takes the same rotation and the same convergence decision, and all pass the
+// same barriers), then rotates its own rows. The partials alternate between two buffers, so one
+// barrier per round suffices. The squared column norms are summed at the start of a sweep and updated by each
+// rotation (a_p loses t a_p.a_q, a_q gains it), so a round needs one dot product and not three; the
+// last sweep, which rotates nothing, decides with fresh ones. The rotation angle is taken in FP32 and the
+// rotation then made orthogonal in FP64 (an angle off by 1e-7 relative leaves a cosine 1e-7 times the old one,
+// which the next sweep removes; the rotation itself never loses orthogonality). After convergence
 // column c is sigma_c u_c. The columns are written in decreasing sigma, each scaled by
 // sign / sigma with the sign that makes its largest-magnitude entry (the first of equal ones)
 // positive: B[r][rank] = u. A zero singular value leaves a zero column. stats[2] = sweeps,
 // stats[3] = largest pair cosine |a_p.a_q| / (||a_p|| ||a_q||) of the last sweep,
 // stats[4] = sigma_min / sigma_max.
-__global__ void __cluster_dims__(kBathCluster, 1, 1) __launch_bounds__(kJacobiThreads)
-    bath_jacobi_kernel(double* __restrict__ Ag, int m, int n_val, int in_smem, double* __restrict__ B,
+//
+// What bounds it: the FP64 pipe is charged 64 clocks of a sub-partition per warp instruction, idle lanes included, so a
+// round costs a sub-partition its pairs' instructions: per pair 5 per lp rows, log2(lp) per sum and some 14 for
+// the angle. Several pairs per warp (lp = 8 or 16) and 16 CTAs (the non-portable cluster size, where the
+// device schedules it) cut them; launch_bath_jacobi picks lp by that count. 910 x 24: 1551 us with a warp per
+// pair, three dot products a round and 8 CTAs; 712 so (4.1 us a round, half of it latency: the cluster barrier, the
+// remote reads, the dependent FP64 chain of the angle).
+template <int CS>
+__global__ void __launch_bounds__(kJacobiThreads)
+    bath_jacobi_kernel(double* __restrict__ Ag, int m, int n_val, int in_smem, int lp, double* __restrict__ B,
                        double* __restrict__ sigma_out, double* __restrict__ stats) {
   extern __shared__ double sm[];
-  __shared__ double part[2][kMaxBathCols / 2][3];
+  __shared__ double part[2][kMaxBathCols / 2];
+  __shared__ double s_nrm[kMaxBathCols];     // squared norms of the whole columns
   __shared__ double s_norm2[kMaxBathCols];   // this CTA's share of ||a_c||^2
   __shared__ double s_big[kMaxBathCols];     // this CTA's largest |a_c| entry, signed
   __shared__ int s_big_row[kMaxBathCols];    // and its global row (m if the CTA has no rows)
@@ -147,7 +155,7 @@ __global__ void __cluster_dims__(kBathCluster, 1, 1) __launch_bounds__(kJacobiTh
   cg::cluster_group cl = cg::this_cluster();
   const int crank = (int)cl.block_rank();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int mc = (m + kBathCluster - 1) / kBathCluster;
+  const int mc = (m + CS - 1) / CS;
   const int r0 = min(m, crank * mc), ml = min(m, r0 + mc) - r0;
   double* A = Ag + r0;
   long long ld = m;
@@ -162,57 +170,63 @@ __global__ void __cluster_dims__(kBathCluster, 1, 1) __launch_bounds__(kJacobiTh
   __syncthreads();
   const int n_pad = n_val + (n_val & 1);
   const int half = n_pad / 2;
+  const unsigned gmask = lp == 32 ? 0xffffffffu : ((1u << lp) - 1u) << (lane & ~(lp - 1));
+  const int l = threadIdx.x & (lp - 1), grp = threadIdx.x / lp, ngrp = kJacobiThreads / lp;
+  // sums over the lp lanes of a group (every lane of the warp takes part)
+  auto group_sum = [&](double v) {
+    for (int o = lp / 2; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+  };
   int sweeps = 0, buf = 0;
   double off = 0.0;
   for (int sweep = 0; sweep < kMaxSweeps && n_val > 1; ++sweep) {
     if (threadIdx.x == 0) s_rot = 0;
     double woff = 0.0;
+    for (int c0 = 0; c0 < n_val; c0 += ngrp) {
+      const int c = c0 + grp;
+      double ss = 0.0;
+      if (c < n_val)
+        for (int r = l; r < ml; r += lp) ss = fma(A[c * ld + r], A[c * ld + r], ss);
+      ss = group_sum(ss);
+      if (l == 0 && c < n_val) s_norm2[c] = ss;
+    }
+    cl.sync();
+    if ((int)threadIdx.x < n_val) {
+      double ss = 0.0;
+      for (int r = 0; r < CS; ++r) ss += *cl.map_shared_rank(&s_norm2[threadIdx.x], r);
+      s_nrm[threadIdx.x] = ss;
+    }
     __syncthreads();
     for (int round = 0; round < n_pad - 1; ++round) {
-      // dot products of this CTA's rows, one warp per pair slot j (j = warp, warp + 16, ...)
-      for (int j = warp; j < half; j += kJacobiWarps) {
-        int p, q;
-        pair_of(round, j, n_pad, p, q);
-        if (p >= n_val || q >= n_val) continue;
-        const double* ap = A + p * ld;
-        const double* aq = A + q * ld;
-        double al = 0.0, be = 0.0, ga = 0.0;
-        for (int r = lane; r < ml; r += 32) {
-          const double x = ap[r], y = aq[r];
-          al = fma(x, x, al);
-          be = fma(y, y, be);
-          ga = fma(x, y, ga);
+      // dot products of this CTA's rows, lp lanes per pair slot j (the trip count is the same for a warp's groups)
+      for (int j0 = 0; j0 < half; j0 += ngrp) {
+        const int j = j0 + grp;
+        int p = n_val, q = n_val;
+        if (j < half) pair_of(round, j, n_pad, p, q);
+        const bool ok = p < n_val && q < n_val;
+        double ga = 0.0;
+        if (ok) {
+          const double* ap = A + p * ld;
+          const double* aq = A + q * ld;
+          for (int r = l; r < ml; r += lp) ga = fma(ap[r], aq[r], ga);
         }
-        al = warp_sum(al);
-        be = warp_sum(be);
-        ga = warp_sum(ga);
-        if (lane == 0) {
-          part[buf][j][0] = al;
-          part[buf][j][1] = be;
-          part[buf][j][2] = ga;
-        }
+        ga = group_sum(ga);
+        if (l == 0 && ok) part[buf][j] = ga;
       }
       cl.sync();
-      for (int j = warp; j < half; j += kJacobiWarps) {
-        int p, q;
-        pair_of(round, j, n_pad, p, q);
-        if (p >= n_val || q >= n_val) continue;
-        // lane g < 8 reads CTA g's three partials; a fixed shuffle tree adds them
-        double al = 0.0, be = 0.0, ga = 0.0;
-        if (lane < kBathCluster) {
-          const double* rp = cl.map_shared_rank(&part[buf][j][0], lane);
-          al = rp[0];
-          be = rp[1];
-          ga = rp[2];
-        }
-        for (int o = kBathCluster / 2; o; o >>= 1) {
-          al += __shfl_xor_sync(0xffffffffu, al, o);
-          be += __shfl_xor_sync(0xffffffffu, be, o);
-          ga += __shfl_xor_sync(0xffffffffu, ga, o);
-        }
-        al = __shfl_sync(0xffffffffu, al, 0);
-        be = __shfl_sync(0xffffffffu, be, 0);
-        ga = __shfl_sync(0xffffffffu, ga, 0);
+      for (int j0 = 0; j0 < half; j0 += ngrp) {
+        const int j = j0 + grp;
+        int p = n_val, q = n_val;
+        if (j < half) pair_of(round, j, n_pad, p, q);
+        const bool ok = p < n_val && q < n_val;
+        // lane l adds the partials of CTAs l, l + lp, ...; a fixed shuffle tree adds the lanes (all end with the
+        // same bits)
+        double ga = 0.0;
+        if (ok)
+          for (int r = l; r < CS; r += lp) ga += *cl.map_shared_rank(&part[buf][j], r);
+        ga = group_sum(ga);
+        if (!ok) continue;
+        const double al = s_nrm[p], be = s_nrm[q];
         // The angle in FP32 (its error only slows convergence a little), the rotation made
         // orthogonal to FP64 rounding: (c, s) scaled by 1/sqrt(c^2 + s^2) = 1 - d/2 + 3d^2/8,
         // d = c^2 + s^2 - 1 = O(1e-7). A zero column gives a NaN cosine and never rotates.
@@ -232,12 +246,17 @@ __global__ void __cluster_dims__(kBathCluster, 1, 1) __launch_bounds__(kJacobiTh
         const double c = cd * nr, sn = sd * nr;
         double* ap = A + p * ld;
         double* aq = A + q * ld;
-        for (int r = lane; r < ml; r += 32) {
+        for (int r = l; r < ml; r += lp) {
           const double x = ap[r], y = aq[r];
           ap[r] = fma(c, x, -sn * y);
           aq[r] = fma(sn, x, c * y);
         }
-        if (lane == 0) s_rot = 1;
+        __syncwarp(gmask);  // (a group's lanes take the same branches: the same ga, al and be)
+        if (l == 0) {
+          s_nrm[p] = fmax(fma(-(double)t, ga, al), 0.0);
+          s_nrm[q] = fmax(fma((double)t, ga, be), 0.0);
+          s_rot = 1;
+        }
       }
       buf ^= 1;
       __syncthreads();
@@ -287,11 +306,11 @@ __global__ void __cluster_dims__(kBathCluster, 1, 1) __launch_bounds__(kJacobiTh
   if (threadIdx.x < n_val) {
     const int c = threadIdx.x;
     double n2 = 0.0;
-    for (int r = 0; r < kBathCluster; ++r) n2 += *cl.map_shared_rank(&s_norm2[c], r);
+    for (int r = 0; r < CS; ++r) n2 += *cl.map_shared_rank(&s_norm2[c], r);
     s_sigma[c] = sqrt(n2);
     double best = -1.0, val = 0.0;
     int at = m;
-    for (int r = 0; r < kBathCluster; ++r) {
+    for (int r = 0; r < CS; ++r) {
       const double v = *cl.map_shared_rank(&s_big[c], r);
       const int a = *cl.map_shared_rank(&s_big_row[c], r);
       if (fabs(v) > best || (fabs(v) == best && a < at)) {
@@ -416,22 +435,65 @@ cudaError_t launch_bath_offdiag(const double2* gk, const double2* tw, const int 
   return cudaGetLastError();
 }
 
-size_t bath_jacobi_smem(int m, int n_val) {
-  return (size_t)((m + kBathCluster - 1) / kBathCluster) * n_val * sizeof(double);
+size_t bath_jacobi_smem(int m, int n_val, int cs) {
+  return (size_t)((m + cs - 1) / cs) * n_val * sizeof(double);
 }
+
+namespace {
+
+// Lanes per pair: the FP64 warp instructions a round charges the busiest sub-partition (see the kernel).
+int lanes_per_pair(int m, int n_val, int cs) {
+  const int mc = (m + cs - 1) / cs, half = (n_val + 1) / 2;
+  int best = 32;
+  double cost = 1e30;
+  for (int lp = 32, lg = 5; lp >= 8; lp /= 2, --lg) {
+    const int warps = (half * lp + 31) / 32, turns = (warps + 3) / 4;
+    const double c = turns * (5.0 * ((mc + lp - 1) / lp) + 2 * lg + 14 + (cs + lp - 1) / lp);
+    if (c < cost) cost = c, best = lp;
+  }
+  return best;
+}
+
+template <int CS>
+cudaError_t jacobi(double* A, int m, int n_val, double* B, double* sigma, double* stats, cudaStream_t st, bool* ran) {
+  *ran = false;
+  const size_t need = bath_jacobi_smem(m, n_val, CS);
+  const bool in_smem = need <= kBathJacobiSmem;
+  auto kernel = bath_jacobi_kernel<CS>;
+  cudaError_t e = cudaSuccess;
+  if (in_smem) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBathJacobiSmem);
+  if (e == cudaSuccess && CS > 8) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(CS);
+  cfg.blockDim = dim3(kJacobiThreads);
+  cfg.dynamicSmemBytes = in_smem ? need : 0;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = CS;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  if (CS > 8) {
+    int fit = 0;
+    if (cudaOccupancyMaxActiveClusters(&fit, kernel, &cfg) != cudaSuccess || fit < 1) {
+      cudaGetLastError();
+      return cudaSuccess;
+    }
+  }
+  *ran = true;
+  return cudaLaunchKernelEx(&cfg, kernel, A, m, n_val, in_smem ? 1 : 0, lanes_per_pair(m, n_val, CS), B, sigma, stats);
+}
+
+}  // namespace
 
 cudaError_t launch_bath_jacobi(double* A, int m, int n_val, double* B, double* sigma, double* stats,
                                cudaStream_t st) {
-  const size_t need = bath_jacobi_smem(m, n_val);
-  const bool in_smem = need <= kBathJacobiSmem;
-  if (in_smem) {
-    cudaError_t e = cudaFuncSetAttribute(bath_jacobi_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)kBathJacobiSmem);
-    if (e != cudaSuccess) return e;
-  }
-  bath_jacobi_kernel<<<kBathCluster, kJacobiThreads, in_smem ? need : 0, st>>>(A, m, n_val, in_smem ? 1 : 0, B, sigma,
-                                                                                stats);
-  return cudaGetLastError();
+  bool ran = false;
+  cudaError_t e = jacobi<16>(A, m, n_val, B, sigma, stats, st, &ran);
+  if (e != cudaSuccess || ran) return e;
+  return jacobi<8>(A, m, n_val, B, sigma, stats, st, &ran);
 }
 
 cudaError_t launch_bath_bloch(const double* B, const double2* Clo, const double2* tw, const int mesh[3], int n_lo,

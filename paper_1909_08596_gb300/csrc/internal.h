@@ -123,11 +123,9 @@ struct BathCols {
   int v[kMaxBathCols];
 };
 constexpr size_t kBathJacobiSmem = 200 * 1024;  // each CTA's rows stay in shared memory up to this size
-constexpr int kBathCluster = 8;                  // CTAs (SMs) of the Jacobi SVD's cluster
 cudaError_t launch_bath_twiddle(int nk, double2* tw, cudaStream_t st);
 cudaError_t launch_bath_offdiag(const double2* gk, const double2* tw, const int mesh[3], int n_lo, const BathCols& val,
                                 double* A, double* stats, cudaStream_t st);
-size_t bath_jacobi_smem(int m, int n_val);
 cudaError_t launch_bath_jacobi(double* A, int m, int n_val, double* B, double* sigma, double* stats,
                                cudaStream_t st);
 cudaError_t launch_bath_product(const double2* Clo, const double2* Cb, int nk, int n_lo, int n_val, double2* Cout,
