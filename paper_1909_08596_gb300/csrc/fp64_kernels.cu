@@ -232,23 +232,36 @@ __device__ __forceinline__ void block_max_commit(double v, double* out) {
 }
 
 // S = s * sum_g S_g (ng split-K partial products of C^+ C); stat = max |S_ij - delta_ij| over
-// the lower triangle j <= i (S is Hermitian, and only those tiles of S_g are computed).
-__global__ void orth_reduce_kernel(const double2* __restrict__ Sg, int ng, int n, double s, double* stat) {
+// the lower triangle j <= i (S is Hermitian, and only those tiles of S_g are computed). Eight threads share the
+// partials of an element.
+__global__ void __launch_bounds__(256) orth_reduce_kernel(const double2* __restrict__ Sg, int ng, int n, double s,
+                                                          double* stat) {
+  __shared__ double2 sh[8][33];
+  const int e = threadIdx.x & 31, gl = threadIdx.x >> 5;
   double v = 0.0;
   const long long nn = (long long)n * n;
-  for (long long x = blockIdx.x * (long long)blockDim.x + threadIdx.x; x < nn;
-       x += (long long)gridDim.x * blockDim.x) {
-    const int i = (int)(x / n), j = (int)(x % n);
-    if (j > i) continue;
-    double re = 0.0, im = 0.0;
-    for (int g = 0; g < ng; ++g) {
-      const double2 e = Sg[g * nn + x];
-      re += e.x;
-      im += e.y;
+  for (long long x0 = blockIdx.x * 32ll; x0 < nn; x0 += gridDim.x * 32ll) {
+    const long long x = x0 + e;
+    const int i = (int)(x / n), j = (int)(x - (long long)i * n);
+    const bool ok = x < nn && j <= i;
+    double2 a = make_double2(0.0, 0.0);
+    if (ok)
+      for (int g = gl; g < ng; g += 8) {
+        const double2 b = Sg[g * nn + x];
+        a.x += b.x;
+        a.y += b.y;
+      }
+    sh[gl][e] = a;
+    __syncthreads();
+    if (gl == 0 && ok) {
+      for (int g = 1; g < 8; ++g) {
+        a.x += sh[g][e].x;
+        a.y += sh[g][e].y;
+      }
+      const double re = s * a.x - (i == j ? 1.0 : 0.0), im = s * a.y;
+      v = wmax(v, sqrt(re * re + im * im));
     }
-    re = s * re - (i == j ? 1.0 : 0.0);
-    im = s * im;
-    v = wmax(v, sqrt(re * re + im * im));
+    __syncthreads();
   }
   block_max_commit(v, stat);
 }
@@ -429,7 +442,7 @@ cudaError_t launch_symmetrize(const double2* Z, double2* Lq, int nq, int naux, i
 }
 
 cudaError_t launch_orth_reduce(const double2* Sg, int ng, int n, double sc, double* stat, cudaStream_t s) {
-  orth_reduce_kernel<<<grid_for((long long)n * n, 256, 152), 256, 0, s>>>(Sg, ng, n, sc, stat);
+  orth_reduce_kernel<<<grid_for((long long)n * n, 32, 152 * 8), 256, 0, s>>>(Sg, ng, n, sc, stat);
   return cudaGetLastError();
 }
 

@@ -321,6 +321,8 @@ struct dmet_emb_plan_s {
   std::vector<cudaEvent_t> join;
   Workspace* W = nullptr;          // workspace of the problem being enqueued
   cudaStream_t cs = nullptr;       // stream of the problem being enqueued
+  cudaStream_t chk = nullptr;      // the orbital checks' stream (fork_checks)
+  cudaEvent_t chk_fork = nullptr, chk_join = nullptr;
   double* dstats = nullptr;        // [n_problems][8]
   unsigned int* derr = nullptr;
   // staging of host buffers
@@ -568,16 +570,17 @@ struct Timed {
 };
 
 // Split-K groups of the orthonormality product C^+ C (K = Nk n_AO rows of C): a divisor of K
-// whose chunks hold >= 8 rows (one k-step of the FP64 kernel), as many as make about four
-// CTAs per SM over the lower-triangle tiles, with the partial products kept under 256 MB.
+// whose chunks hold >= 16 rows (one k-step of the FP64 kernel), as many as make about two
+// CTAs per SM over the lower-triangle tiles of 16 x 16 and at most 32 (the reduction reads them all), with the
+// partial products kept under 256 MB.
 int orth_groups_for(int nk, int nao, int n) {
   const long long K = (long long)nk * nao;
-  const long long tiles = (n + 63) / 64, lower = tiles * (tiles + 1) / 2;
-  const long long want = std::max(1LL, 4 * 152 / lower);
+  const long long tiles = (n + 15) / 16, lower = tiles * (tiles + 1) / 2;
+  const long long want = std::min(32LL, std::max(1LL, 2 * 152 / lower));
   const long long cap = std::max(1LL, (256LL << 20) / std::max(1LL, (long long)n * n * 16));
   int best = 1;
-  for (long long g = 1; g <= K; ++g) {
-    if (K % g || K / g < 8 || g > want || g > cap) continue;
+  for (long long g = 1; g <= K && g <= want; ++g) {
+    if (K % g || K / g < 16 || g > cap) continue;
     best = (int)g;
   }
   return best;
@@ -655,8 +658,8 @@ dmet_status_t run_orbital_checks(dmet_emb_plan_s* P, Prob& pr, int p, const doub
     {
       // split-K over groups of k-points so that the small n x n product fills the GPU
       const int ng = pr.orth_groups;
-      const int tiles = (n + 63) / 64;
-      Timed t(P, KC_CHECK_C, 8.0 * 64 * 64 * (tiles * (tiles + 1) / 2) * (double)pr.nk * pr.nao,
+      const int tiles = (n + 15) / 16;
+      Timed t(P, KC_CHECK_C, 8.0 * 16 * 16 * (tiles * (tiles + 1) / 2) * (double)pr.nk * pr.nao,
               16.0 * pr.nk * pr.nao * n, 2);
       ZgemmArgs z = zargs();
       z.A = C[s];
@@ -682,6 +685,29 @@ dmet_status_t run_orbital_checks(dmet_emb_plan_s* P, Prob& pr, int p, const doub
       CK(launch_c_real_check(C[s], pr.d_neg, pr.nk, pr.nao, n, st, P->cs));
     }
   }
+  return DMET_OK;
+}
+
+// The orbital checks read only C and write only the problem's statistics, so they run beside the transforms on a
+// stream of their own (135 us of an h-BN-shaped call, on the FP64 pipe, under operand splitting that is bound by
+// memory): forked from the problem's stream here, joined back by join_checks before the call's work ends. Problems
+// on side streams of their own keep them there: they already overlap, and one stream for the checks of a batch is
+// slower (24 problems in grouped launches: 5.49 against 5.32 ms).
+dmet_status_t fork_checks(dmet_emb_plan_s* P, Prob& pr, int p, const double2* const* C, bool beside) {
+  if (!beside) return run_orbital_checks(P, pr, p, C);
+  CK(cudaEventRecord(P->chk_fork, P->cs));
+  CK(cudaStreamWaitEvent(P->chk, P->chk_fork, 0));
+  const cudaStream_t cs = P->cs;
+  P->cs = P->chk;
+  const dmet_status_t st = run_orbital_checks(P, pr, p, C);
+  P->cs = cs;
+  // (recorded on a failure too: a captured fork has to be joined)
+  CK(cudaEventRecord(P->chk_join, P->chk));
+  return st;
+}
+
+dmet_status_t join_checks(dmet_emb_plan_s* P, cudaStream_t s) {
+  CK(cudaStreamWaitEvent(s, P->chk_join, 0));
   return DMET_OK;
 }
 
@@ -995,6 +1021,7 @@ void destroy_plan(dmet_emb_plan_s* P) {
   if (P->stream) cudaStreamSynchronize(P->stream);
   else cudaDeviceSynchronize();
   for (cudaStream_t st : P->side) cudaStreamSynchronize(st);
+  if (P->chk) cudaStreamSynchronize(P->chk);
   for (auto& pr : P->probs) {
     free_tables(pr.nat);
     free_tables(pr.con);
@@ -1016,6 +1043,9 @@ void destroy_plan(dmet_emb_plan_s* P) {
   if (P->gexec) cudaGraphExecDestroy(P->gexec);
   for (cudaStream_t st : P->side) cudaStreamDestroy(st);
   if (P->cap) cudaStreamDestroy(P->cap);
+  if (P->chk) cudaStreamDestroy(P->chk);
+  if (P->chk_fork) cudaEventDestroy(P->chk_fork);
+  if (P->chk_join) cudaEventDestroy(P->chk_join);
   if (P->fork) cudaEventDestroy(P->fork);
   for (auto e : P->join) cudaEventDestroy(e);
   for (auto& e : P->pev) {
@@ -2010,6 +2040,10 @@ dmet_status_t dmet_emb_plan(const dmet_emb_desc_t* descs, int32_t n_problems, vo
     if (st == DMET_OK && cudaEventCreateWithFlags(&P->fork, cudaEventDisableTiming) != cudaSuccess)
       st = fail(DMET_ERR_CUDA, "event creation failed");
   }
+  if (st == DMET_OK && (cudaStreamCreateWithFlags(&P->chk, cudaStreamNonBlocking) != cudaSuccess ||
+                        cudaEventCreateWithFlags(&P->chk_fork, cudaEventDisableTiming) != cudaSuccess ||
+                        cudaEventCreateWithFlags(&P->chk_join, cudaEventDisableTiming) != cudaSuccess))
+    st = fail(DMET_ERR_CUDA, "check stream creation failed");
   if (st == DMET_OK && cudaMalloc(&P->derr, sizeof(unsigned int)) != cudaSuccess) {
     cudaGetLastError();
     st = fail(DMET_ERR_OOM, "error word allocation failed");
@@ -2155,7 +2189,7 @@ dmet_status_t dmet_emb_transform_3idx(dmet_emb_plan_t P, int32_t problem, const 
   const double2* Cd[2] = {nullptr, nullptr};
   TRY(stage_inputs(P, pr, L, C, &Ld, Cd));
   CK(cudaMemsetAsync(P->dstats + 8 * problem, 0, 8 * sizeof(double), P->cs));
-  TRY(run_orbital_checks(P, pr, problem, Cd));
+  TRY(fork_checks(P, pr, problem, Cd, true));
   TRY(run_l_check(P, pr, problem, Ld));
   double2* out[2] = {nullptr, nullptr};
   size_t ob[2] = {0, 0}, need = 0;
@@ -2194,6 +2228,7 @@ dmet_status_t dmet_emb_transform_3idx(dmet_emb_plan_t P, int32_t problem, const 
   } else {
     TRY(transform_range(P, pr, Ld, Cd, q_begin, q_end, out, pr.bq));
   }
+  TRY(join_checks(P, P->cs));
   if (need) {
     for (int s = 0; s < pr.nspin; ++s)
       if (ohost[s]) {
@@ -2220,7 +2255,8 @@ static dmet_status_t enqueue_problem(dmet_emb_plan_s* P, int p, const void* L, c
   const double2* Cd[2] = {nullptr, nullptr};
   TRY(stage_inputs(P, pr, L, C, &Ld, Cd, /*subset=*/true));
   CK(cudaMemsetAsync(P->dstats + 8 * p, 0, 8 * sizeof(double), P->cs));
-  TRY(run_orbital_checks(P, pr, p, Cd));
+  const bool beside = P->side.empty();
+  TRY(fork_checks(P, pr, p, Cd, beside));
   TRY(run_l_check(P, pr, p, Ld));
   const int nblk = pr.nspin == 1 ? 1 : 3;
   void* out[3] = {nullptr, nullptr, nullptr};
@@ -2247,6 +2283,7 @@ static dmet_status_t enqueue_problem(dmet_emb_plan_s* P, int p, const void* L, c
   else if (pr.pack == DMET_PACK_S8) st = eri_s8(P, pr, Ld, Cd, out);
   else st = eri_full(P, pr, Ld, Cd, out);
   P->xpending = false;
+  if (beside) TRY(join_checks(P, P->cs));
   TRY(st);
   if (need) {
     for (int b = 0; b < nblk; ++b)
@@ -3302,7 +3339,7 @@ dmet_status_t dmet_emb_eri_fftdf(dmet_emb_plan_t P, int32_t problem, const void*
   const double2* Cd[2] = {(const double2*)C[0], pr.nspin == 2 ? (const double2*)C[1] : nullptr};
   P->W = &P->ws[P->ws_of[problem]];
   CK(cudaMemsetAsync(P->dstats + 8 * problem, 0, 8 * sizeof(double), P->cs));
-  TRY(run_orbital_checks(P, pr, problem, Cd));
+  TRY(fork_checks(P, pr, problem, Cd, true));
   double2* lq[2] = {P->W->lq_all[0], P->W->lq_all[1]};
   TRY(transform_range(P, pr, (const double2*)rho, Cd, 0, nk, lq, pr.bq));
   for (int b = 0; b < nblk; ++b) CK(cudaMemsetAsync(eri_out[b], 0, eri_bytes_of(pr.d, b), P->cs));
@@ -3369,6 +3406,7 @@ dmet_status_t dmet_emb_eri_fftdf(dmet_emb_plan_t P, int32_t problem, const void*
       }
     }
   }
+  TRY(join_checks(P, P->cs));
   CK(cudaGetLastError());
   return DMET_OK;
 }
