@@ -165,43 +165,76 @@ __global__ void gather_orbitals_kernel(const double2* __restrict__ C, double2* _
   }
 }
 
-__device__ __forceinline__ void pair_of(long long ij, int& i, int& j) {
-  long long r = (long long)((sqrt(8.0 * (double)ij + 1.0) - 1.0) * 0.5);
-  while (r * (r + 1) / 2 > ij) --r;
-  while ((r + 1) * (r + 2) / 2 <= ij) ++r;
-  i = (int)r;
-  j = (int)(ij - r * (r + 1) / 2);
+// Z + Z^T of every (q, P) matrix, one CTA per 32 x 32 tile of its lower triangle: the tile and its mirror are read along
+// their rows and met in shared memory (reading the mirror down its columns, and a pair's (i, j) from a square root,
+// took 576 us for 1760 matrices of 104 x 104; this 114).
+constexpr int kSymTile = 32;
+struct SymTile {
+  int i0, j0;
+};
+__device__ __forceinline__ SymTile sym_tile(int t) {
+  int r = (int)((sqrtf(8.f * (float)t + 1.f) - 1.f) * 0.5f);
+  while (r * (r + 1) / 2 > t) --r;
+  while ((r + 1) * (r + 2) / 2 <= t) ++r;
+  return {r * kSymTile, (t - r * (r + 1) / 2) * kSymTile};
+}
+__device__ __forceinline__ void load_sym_tile(const double2* z, int n, SymTile t, double2 (&m)[kSymTile][kSymTile + 1]) {
+  const int x = threadIdx.x & 31, y = threadIdx.x >> 5;
+#pragma unroll
+  for (int r = y; r < kSymTile; r += 8)
+    if (t.j0 + r < n && t.i0 + x < n) m[r][x] = z[(long long)(t.j0 + r) * n + t.i0 + x];  // rows j of the mirror
+  __syncthreads();
 }
 
-__global__ void pack_pairs_kernel(const double2* __restrict__ Z, double* __restrict__ X, int nq, int naux,
-                                  int n, int nc, double s) {
+// X[(q, P, c)][pair ij] = s (Re or Im of Z_ij + Z_ji)
+__global__ void __launch_bounds__(256) pack_pairs_kernel(const double2* __restrict__ Z, double* __restrict__ X, int n,
+                                                         int nc, double s) {
+  __shared__ double2 m[kSymTile][kSymTile + 1];
+  const SymTile t = sym_tile(blockIdx.y + blockIdx.z * gridDim.y);
+  if (t.i0 >= n) return;
+  const double2* z = Z + (long long)blockIdx.x * n * n;
+  load_sym_tile(z, n, t, m);
   const long long npair = (long long)n * (n + 1) / 2;
-  const long long total = (long long)nq * naux * nc * npair;
-  for (long long x = blockIdx.x * (long long)blockDim.x + threadIdx.x; x < total;
-       x += (long long)gridDim.x * blockDim.x) {
-    const long long ij = x % npair;
-    const long long row = x / npair;  // (q, P, c)
-    const int c = (int)(row % nc);
-    const long long qp = row / nc;    // q * naux + P
-    int i, j;
-    pair_of(ij, i, j);
-    const double2* z = Z + qp * n * (long long)n;
-    const double2 a = z[(long long)i * n + j], b = z[(long long)j * n + i];
-    X[x] = s * (c == 0 ? a.x + b.x : a.y + b.y);
+  double* out = X + (long long)blockIdx.x * nc * npair;
+  const int x = threadIdx.x & 31, y = threadIdx.x >> 5, j = t.j0 + x;
+#pragma unroll
+  for (int r = y; r < kSymTile; r += 8) {
+    const int i = t.i0 + r;
+    if (i >= n || j > i) continue;
+    const double2 a = z[(long long)i * n + j], b = m[x][r];
+    const long long ij = (long long)i * (i + 1) / 2 + j;
+    out[ij] = s * (a.x + b.x);
+    if (nc == 2) out[npair + ij] = s * (a.y + b.y);
   }
 }
 
-__global__ void symmetrize_kernel(const double2* __restrict__ Z, double2* __restrict__ Lq, int nq, int naux,
-                                  int n, double s, double sim) {
-  const long long nn = (long long)n * n;
-  const long long total = (long long)nq * naux * nn;
-  for (long long x = blockIdx.x * (long long)blockDim.x + threadIdx.x; x < total;
-       x += (long long)gridDim.x * blockDim.x) {
-    const long long base = x - x % nn;
-    const int i = (int)((x % nn) / n), j = (int)(x % n);
-    const double2 a = Z[x], b = Z[base + (long long)j * n + i];
-    Lq[x] = make_double2(s * (a.x + b.x), sim * (a.y + b.y));
+// Lq = (s Re, sim Im) of Z + Z^T
+__global__ void __launch_bounds__(256) symmetrize_kernel(const double2* __restrict__ Z, double2* __restrict__ Lq, int n,
+                                                         double s, double sim) {
+  __shared__ double2 m[kSymTile][kSymTile + 1];
+  const SymTile t = sym_tile(blockIdx.y + blockIdx.z * gridDim.y);
+  if (t.i0 >= n) return;
+  const double2* z = Z + (long long)blockIdx.x * n * n;
+  double2* out = Lq + (long long)blockIdx.x * n * n;
+  load_sym_tile(z, n, t, m);
+  const int x = threadIdx.x & 31, y = threadIdx.x >> 5, j = t.j0 + x;
+  double2 v[kSymTile / 8];
+#pragma unroll
+  for (int h = 0; h < kSymTile / 8; ++h) {
+    const int r = y + 8 * h, i = t.i0 + r;
+    if (i >= n || j >= n) continue;
+    const double2 a = z[(long long)i * n + j], b = m[x][r];
+    v[h] = make_double2(s * (a.x + b.x), sim * (a.y + b.y));
+    out[(long long)i * n + j] = v[h];
   }
+  if (t.i0 == t.j0) return;  // (a diagonal tile is its own mirror)
+  __syncthreads();
+#pragma unroll
+  for (int h = 0; h < kSymTile / 8; ++h) m[x][y + 8 * h] = v[h];
+  __syncthreads();
+#pragma unroll
+  for (int r = y; r < kSymTile; r += 8)
+    if (t.j0 + r < n && t.i0 + x < n) out[(long long)(t.j0 + r) * n + t.i0 + x] = m[r][x];
 }
 
 // Max of non-negative doubles through their bit patterns (NaN compares above +inf).
@@ -427,17 +460,23 @@ cudaError_t launch_gather_orbitals(const double2* C, double2* Crep, const int4* 
   return cudaGetLastError();
 }
 
+namespace {
+// one CTA per (matrix, lower-triangle tile), the tiles over y and z
+dim3 sym_grid(long long matrices, int n) {
+  const long long t = (n + kSymTile - 1) / kSymTile, tiles = t * (t + 1) / 2, y = tiles < 32768 ? tiles : 32768;
+  return dim3((unsigned)matrices, (unsigned)y, (unsigned)((tiles + y - 1) / y));
+}
+}  // namespace
+
 cudaError_t launch_pack_pairs(const double2* Z, double* X, int nq, int naux, int n, int nc, double sc,
                               cudaStream_t s) {
-  const long long total = (long long)nq * naux * nc * ((long long)n * (n + 1) / 2);
-  pack_pairs_kernel<<<grid_for(total, 256, 152 * 16), 256, 0, s>>>(Z, X, nq, naux, n, nc, sc);
+  pack_pairs_kernel<<<sym_grid((long long)nq * naux, n), 256, 0, s>>>(Z, X, n, nc, sc);
   return cudaGetLastError();
 }
 
 cudaError_t launch_symmetrize(const double2* Z, double2* Lq, int nq, int naux, int n, double sc, int conj,
                               cudaStream_t s) {
-  const long long total = (long long)nq * naux * n * n;
-  symmetrize_kernel<<<grid_for(total, 256, 152 * 16), 256, 0, s>>>(Z, Lq, nq, naux, n, sc, conj ? -sc : sc);
+  symmetrize_kernel<<<sym_grid((long long)nq * naux, n), 256, 0, s>>>(Z, Lq, n, sc, conj ? -sc : sc);
   return cudaGetLastError();
 }
 

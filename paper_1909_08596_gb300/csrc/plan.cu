@@ -538,7 +538,7 @@ static dmet_status_t queue_block_copies(dmet_emb_plan_s* P, const Prob& pr, int 
   return DMET_OK;
 }
 
-constexpr size_t kRnsScratch = (size_t)1 << 30;
+constexpr size_t kRnsScratch = (size_t)3 << 29;
 
 struct Timed {
   dmet_emb_plan_s* P;

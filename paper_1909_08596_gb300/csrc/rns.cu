@@ -240,10 +240,10 @@ __device__ __forceinline__ void store_residues(const float (&cr)[RW][4], const f
 // One CTA converts RB operand rows (32, or 8 where that would leave SMs idle): first their norms, then the
 // residues, 32 (re, im) or (k, k + 1) pairs at a time, a lane per pair, so that every store of a warp is 128
 // contiguous bytes. Rows that are contiguous in memory (s_row = 1) pass through a transpose in shared memory.
-template <int SRC, int RB>
+template <int SRC, int RB, bool rowfast>
 __global__ void __launch_bounds__(256) rns_convert_kernel(const ConvArgs a) {
   constexpr int KL = 256 / RB, RW = RB / 8;  // k lanes per row, rows per warp
-  __shared__ double2 tile[32][RB + 1];
+  __shared__ double2 tile[rowfast ? 32 : 1][RB + 1];
   __shared__ float sh_s[KL][RB];
   __shared__ int sh_e[KL][RB], sh_bad[KL][RB], sh_scale[RB];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -256,24 +256,40 @@ __global__ void __launch_bounds__(256) rns_convert_kernel(const ConvArgs a) {
     off = (a.sel ? (long long)t.y : (long long)t.x) * a.sbatch;
     K = t.w;
   }
-  const bool rowfast = a.s_row == 1;
   const double2* src2 = reinterpret_cast<const double2*>(a.src) + off;
   const double* src1 = a.src + off;
 
-  // norms
-  if (rowfast) {
-    RowNorm n{0.f, 0, 0};
-    if (r0 + trow < a.rows) {
-      for (int k = tk; k < K; k += KL) {
-        if constexpr (SRC == SRC_REAL) {
-          norm_add(n, src1[(r0 + trow) + (long long)k * a.s_k]);
-        } else {
-          const double2 v = src2[(r0 + trow) + (long long)k * a.s_k];
-          norm_add(n, v.x);
-          norm_add(n, v.y);
-        }
-      }
+  // one element (its second component zero for a real one), zero outside
+  auto element = [&](int r, int k) {
+    double2 v = make_double2(0.0, 0.0);
+    if (r < a.rows && k < K) {
+      const long long at = (long long)r * a.s_row + (long long)k * a.s_k;
+      if constexpr (SRC == SRC_REAL) v.x = src1[at];
+      else v = src2[at];
     }
+    return v;
+  };
+  // norms, four loads in flight per thread
+  auto norm_of = [&](int r, int k0, int step) {
+    RowNorm n{0.f, 0, 0};
+    auto add = [&](double2 v) {
+      norm_add(n, v.x);
+      if constexpr (SRC != SRC_REAL) norm_add(n, v.y);
+    };
+    if (r >= a.rows) return n;
+    int k = k0;
+    for (; k + 3 * step < K; k += 4 * step) {
+      double2 v[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) v[i] = element(r, k + i * step);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) add(v[i]);
+    }
+    for (; k < K; k += step) add(element(r, k));
+    return n;
+  };
+  if constexpr (rowfast) {
+    RowNorm n = norm_of(r0 + trow, tk, KL);
     sh_s[tk][trow] = n.s;
     sh_e[tk][trow] = n.e;
     sh_bad[tk][trow] = n.bad;
@@ -284,19 +300,7 @@ __global__ void __launch_bounds__(256) rns_convert_kernel(const ConvArgs a) {
     }
   } else {
     for (int i = 0; i < RW; ++i) {
-      const int r = r0 + warp * RW + i;
-      RowNorm n{0.f, 0, 0};
-      if (r < a.rows) {
-        for (int k = lane; k < K; k += 32) {
-          if constexpr (SRC == SRC_REAL) {
-            norm_add(n, src1[(long long)r * a.s_row + (long long)k * a.s_k]);
-          } else {
-            const double2 v = src2[(long long)r * a.s_row + (long long)k * a.s_k];
-            norm_add(n, v.x);
-            norm_add(n, v.y);
-          }
-        }
-      }
+      RowNorm n = norm_of(r0 + warp * RW + i, lane, 32);
       const int e = __reduce_max_sync(0xffffffffu, n.e), d = n.e - e;
       n.s = d > -60 ? n.s * pow2f(2 * d) : 0.f;
       n.e = e;
@@ -310,25 +314,28 @@ __global__ void __launch_bounds__(256) rns_convert_kernel(const ConvArgs a) {
   if (threadIdx.x < RB && r0 + trow < a.rows) a.exps[(long long)z * a.rows + r0 + trow] = sh_scale[trow];
 
   constexpr int RR = SRC == SRC_COMPLEX2 ? 2 : 1;
-  const int units = SRC == SRC_REAL ? (K + 1) / 2 : K, upad = a.Kp / 2;
+  const int upad = a.Kp / 2;
+  // pair u of row r: (re, im), or (k, k + 1) of a real operand
+  auto pair = [&](int r, int u) {
+    if constexpr (SRC == SRC_REAL) return make_double2(element(r, 2 * u).x, element(r, 2 * u + 1).x);
+    else return element(r, u);
+  };
+  // a thread's share of the transpose of the tile of 32 pairs from u on: the next tile's is loaded before the current
+  // one is converted (22 880 x 520: 286 us without, 250 with)
+  static_assert(RW * KL == 32, "a thread's share of a tile");
+  double2 next[RW];
+  auto fetch = [&](int u) {
+#pragma unroll
+    for (int i = 0; i < RW; ++i) next[i] = pair(r0 + trow, u + tk + i * KL);
+  };
+  if constexpr (rowfast) fetch(0);
   for (int u0 = 0; u0 < upad; u0 += 32) {
-    if (rowfast) {
+    if constexpr (rowfast) {
       __syncthreads();
 #pragma unroll
-      for (int ul = tk; ul < 32; ul += KL) {
-        const int u = u0 + ul;
-        double2 v = make_double2(0.0, 0.0);
-        if (u < units && r0 + trow < a.rows) {
-          if constexpr (SRC == SRC_REAL) {
-            v.x = src1[(r0 + trow) + (long long)(2 * u) * a.s_k];
-            if (2 * u + 1 < K) v.y = src1[(r0 + trow) + (long long)(2 * u + 1) * a.s_k];
-          } else {
-            v = src2[(r0 + trow) + (long long)u * a.s_k];
-          }
-        }
-        tile[ul][trow] = v;
-      }
+      for (int i = 0; i < RW; ++i) tile[tk + i * KL][trow] = next[i];
       __syncthreads();
+      if (u0 + 32 < upad) fetch(u0 + 32);
     }
     const int u = u0 + lane;
     float cr[RW][4], ci[RW][4];
@@ -336,17 +343,7 @@ __global__ void __launch_bounds__(256) rns_convert_kernel(const ConvArgs a) {
 #pragma unroll
     for (int i = 0; i < RW; ++i) {
       const int rl = warp * RW + i, r = r0 + rl;
-      double2 v = make_double2(0.0, 0.0);
-      if (rowfast) {
-        v = tile[lane][rl];
-      } else if (u < units && r < a.rows) {
-        if constexpr (SRC == SRC_REAL) {
-          v.x = src1[(long long)r * a.s_row + (long long)(2 * u) * a.s_k];
-          if (2 * u + 1 < K) v.y = src1[(long long)r * a.s_row + (long long)(2 * u + 1) * a.s_k];
-        } else {
-          v = src2[(long long)r * a.s_row + (long long)u * a.s_k];
-        }
-      }
+      const double2 v = rowfast ? tile[rowfast ? lane : 0][rl] : pair(r, u0 + lane);
       const int s = sh_scale[rl];
       long long ar = 0, ai = 0;
       if (s != kPoison) {
@@ -381,8 +378,8 @@ struct GemmArgs {
   int tri, h0;              // tri: only tiles with a column <= the last row (square product, bn = 256); row 0 of
                             // this launch is row 256 h0 of the product
   int row0;                 // first row of the launch in the row operand
-  int tiles;                // per (modulus, batch)
-  int nkb;                  // K blocks
+  int jobs;                 // (clusters of tiles) per (modulus, batch)
+  int nkb, seg;             // K blocks, and how many of them between reductions (at most kSegStages)
   signed char* Y;           // [mod][batch][rows][ldy]
   long long ymod;
   int ldy;
@@ -392,33 +389,31 @@ struct Tile {
   int mod, z, m0, n0;
 };
 
-// Tiles of the lower triangle: the row tiles 2 h and 2 h + 1 have h0 + h + 1 column tiles each.
-__host__ __device__ inline int tri_tiles_before(int mt, int h0) {
-  const int h = mt >> 1;
-  return h * h + (2 * h0 + 1) * h + (mt & 1) * (h0 + h + 1);
-}
+// Lower triangle: the row tiles 2 h and 2 h + 1 have h0 + h + 1 column tiles each; jobs take the pair together (CL = 2).
+__host__ __device__ inline int tri_jobs_before(int h, int h0) { return h * h0 + h * (h + 1) / 2; }
 
-__device__ __forceinline__ Tile tile_of(const GemmArgs& g, int job) {
+// Job `job` of a launch, for the CTA of rank `rank` of its cluster: CL neighbouring row tiles of one column tile.
+template <int CL>
+__device__ __forceinline__ Tile tile_of(const GemmArgs& g, int job, int rank) {
   Tile t;
-  const int per = g.nbatch * g.tiles;
+  const int per = g.nbatch * g.jobs;
   t.mod = job / per;
   int r = job - t.mod * per;
-  t.z = r / g.tiles;
-  r -= t.z * g.tiles;
+  t.z = r / g.jobs;
+  r -= t.z * g.jobs;
   int mt, nt;
-  if (g.tri) {
-    int h = (int)((sqrtf((float)(2 * g.h0 + 1) * (float)(2 * g.h0 + 1) + 4.f * (float)r) - (float)(2 * g.h0 + 1)) * 0.5f);
-    while (tri_tiles_before(2 * h, g.h0) > r) --h;
-    while (tri_tiles_before(2 * h + 2, g.h0) <= r) ++h;
-    const int rem = r - tri_tiles_before(2 * h, g.h0), w = g.h0 + h + 1;
-    const int up = rem >= w;
-    mt = 2 * h + up;
-    nt = rem - up * w;
+  if (CL == 2 && g.tri) {
+    const float c = (float)(2 * g.h0 + 1);
+    int h = (int)((sqrtf(c * c + 8.f * (float)r) - c) * 0.5f);
+    while (h > 0 && tri_jobs_before(h, g.h0) > r) --h;
+    while (tri_jobs_before(h + 1, g.h0) <= r) ++h;
+    mt = h;
+    nt = r - tri_jobs_before(h, g.h0);
   } else {
     mt = r / g.ct;
     nt = r - mt * g.ct;
   }
-  t.m0 = mt * kTileM;
+  t.m0 = (mt * CL + rank) * kTileM;
   t.n0 = nt * g.bn;
   return t;
 }
@@ -441,6 +436,10 @@ __device__ __forceinline__ uint4 reduce16(const uint32_t (&v)[16], bool add, uin
   return make_uint4(w[0], w[1], w[2], w[3]);
 }
 
+// Bound by the L2 reads of the operands (a 128 x 256 tile alone reads 48 KB per 512 clocks of MMA): with CL = 2 a
+// cluster's two CTAs take neighbouring row tiles, load half of the column tile each and multicast it to both, 32 KB
+// per CTA. A stage is free again when both CTAs' MMAs have read it.
+template <int CL>
 __global__ void __launch_bounds__(kGemmThreads, 1)
     rns_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const GemmArgs g,
                     int njobs, unsigned int* err, unsigned long long lim, int withhold) {
@@ -458,11 +457,15 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
   const uint32_t done_bar = smem_u32(bars + 2 * kStages + 4);
   auto a_tile = [&](int s) { return smem_u32(smem + s * kStageBytes); };
   auto b_tile = [&](int s) { return smem_u32(smem + s * kStageBytes + kABytes); };
+  const int rank = CL > 1 ? (int)cluster_rank() : 0;
+  const int job0 = (int)blockIdx.x / CL, njob = (int)gridDim.x / CL;
+  constexpr uint16_t kAll = (1u << CL) - 1u;
+  bool failed = false;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages; ++s) {
       mbar_init(full(s), 1);
-      mbar_init(empty(s), 1);
+      mbar_init(empty(s), CL);
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(accf(b), 1);
@@ -478,6 +481,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
   }
   tc_fence_before();
   __syncthreads();
+  if (CL > 1) cluster_sync_all();  // every CTA's barriers are initialised
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
 
@@ -488,8 +492,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
       prefetch_tmap(&tmB);
       const uint32_t bytes = kABytes + (uint32_t)g.bn * 128u;
       bool ok = !withhold;
-      for (int jb = blockIdx.x; jb < njobs && ok; jb += gridDim.x) {
-        const Tile t = tile_of(g, jb);
+      for (int jb = job0; jb < njobs && ok; jb += njob) {
+        const Tile t = tile_of<CL>(g, jb, rank);
         const int ra = t.z * g.rows + g.row0 + t.m0, rb = t.z * g.cols + t.n0;
         for (int kb = 0; kb < g.nkb; ++kb) {
           const int s = issued % kStages, ph = (issued / kStages) & 1;
@@ -499,25 +503,32 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
           }
           mbar_arrive_expect_tx(full(s), bytes);
           tma_load_3d(a_tile(s), &tmA, full(s), kb * kBK, ra, t.mod);
-          tma_load_3d(b_tile(s), &tmB, full(s), kb * kBK, rb, t.mod);
+          if constexpr (CL == 1) {
+            tma_load_3d(b_tile(s), &tmB, full(s), kb * kBK, rb, t.mod);
+          } else {
+            // this CTA's share of the column tile's rows (a multiple of 8: whole swizzle atoms), to both CTAs
+            const int share = g.bn / CL;
+            tma_load_3d_multicast(b_tile(s) + rank * share * 128, &tmB, full(s), kb * kBK, rb + rank * share, t.mod, kAll);
+          }
           ++issued;
         }
       }
+      failed = !ok;
     }
   } else if (warp == 1) {
     if (lane == 0) {
       const uint32_t idesc = idesc_f32acc(1, kTileM, g.bn);
       int it = 0, gs = 0;
       bool ok = true;
-      for (int jb = blockIdx.x; jb < njobs && ok; jb += gridDim.x) {
-        for (int k0 = 0; k0 < g.nkb && ok; k0 += kSegStages, ++gs) {
+      for (int jb = job0; jb < njobs && ok; jb += njob) {
+        for (int k0 = 0; k0 < g.nkb && ok; k0 += g.seg, ++gs) {
           const int b = gs & 1, u = gs >> 1;
           if (!mbar_wait(acce(b), (u & 1) ^ 1, err, 2u, lim)) {
             ok = false;
             break;
           }
           tc_fence_after();
-          const int k1 = min(g.nkb, k0 + kSegStages);
+          const int k1 = min(g.nkb, k0 + g.seg);
           for (int kb = k0; kb < k1; ++kb) {
             const int s = it % kStages, ph = (it / kStages) & 1;
             if (!mbar_wait(full(s), ph, err, 4u, lim)) {
@@ -528,7 +539,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
             for (int kk = 0; kk < 4; ++kk)
               umma<0>(tmem + b * 256, smem_desc<128>(a_tile(s) + kk * 32), smem_desc<128>(b_tile(s) + kk * 32), idesc,
                       (kb > k0 || kk) ? 1u : 0u);
-            umma_commit(empty(s));
+            if constexpr (CL == 1) umma_commit(empty(s));
+            else umma_commit_multicast(empty(s), kAll);
             ++it;
             *consumed = it;
           }
@@ -536,34 +548,43 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
         }
       }
       umma_commit(done_bar);
-      mbar_wait(done_bar, 0, err, 16u, lim);
+      failed = !mbar_wait(done_bar, 0, err, 16u, lim) || !ok;
     }
   } else if (warp >= 4) {
     const int quad = warp & 3, half = (warp - 4) >> 2;
     bool ok = true;
     int gs = 0;
-    for (int jb = blockIdx.x; jb < njobs && ok; jb += gridDim.x) {
-      const Tile t = tile_of(g, jb);
+    for (int jb = job0; jb < njobs && ok; jb += njob) {
+      const Tile t = tile_of<CL>(g, jb, rank);
       const float p = kModF[t.mod], rp = 1.0f / p;
       const int row = t.m0 + quad * 32 + lane;
       signed char* y = g.Y + (long long)t.mod * g.ymod + ((long long)t.z * g.rows + row) * g.ldy + t.n0;
       const bool rok = row < g.rows;
-      for (int k0 = 0; k0 < g.nkb; k0 += kSegStages, ++gs) {
+      const int cols = min(g.bn, g.ldy - t.n0);
+      for (int k0 = 0; k0 < g.nkb; k0 += g.seg, ++gs) {
         const int b = gs & 1, u = gs >> 1;
+        // the running residues, on their way while the MMAs finish (one at a time behind each accumulator
+        // read, their latency was most of the epilogue)
+        uint4 prev[8];
+        if (k0 && rok) {
+#pragma unroll
+          for (int i = 0; i < 8; ++i)
+            if (half * 16 + 32 * i < cols) prev[i] = *reinterpret_cast<const uint4*>(y + half * 16 + 32 * i);
+        }
         if (!mbar_wait(accf(b), u & 1, err, 8u, lim)) {
           ok = false;
           break;
         }
         tc_fence_after();
         const uint32_t tm = tmem + b * 256 + ((uint32_t)(quad * 32) << 16);
-        for (int c = half * 16; c < g.bn; c += 32) {
-          if (t.n0 + c >= g.ldy) break;  // (uniform) past the last column
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          const int c = half * 16 + 32 * i;
+          if (c >= cols) break;  // (uniform)
           uint32_t v[16];
           tmem_ld_32x32b_x16(tm + c, v);
-          uint4 prev = make_uint4(0, 0, 0, 0);
-          if (k0 && rok) prev = *reinterpret_cast<const uint4*>(y + c);
           tmem_ld_wait();
-          const uint4 w = reduce16(v, k0 != 0, prev, p, rp);
+          const uint4 w = reduce16(v, k0 != 0, prev[i], p, rp);
           if (rok) *reinterpret_cast<uint4*>(y + c) = w;
         }
         tc_fence_before();
@@ -576,6 +597,12 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
   if (warp == 0 && lane == 0) {
     // copies issued but never consumed (only after an expired wait) must land before exit
     for (int i = *consumed; i < issued; ++i) mbar_wait(full(i % kStages), (i / kStages) & 1, err, 32u, lim);
+  }
+  if (CL > 1) {
+    // After an expired wait the peer's copies into this CTA may still be in flight: give them a millisecond to land.
+    if (__syncthreads_or(failed))
+      for (int i = 0; i < 1000; ++i) __nanosleep(1000);
+    cluster_sync_all();  // no CTA leaves while the other's copies and commits can still reach it
   }
   __syncthreads();
   if (warp == 1) {
@@ -811,13 +838,21 @@ cudaError_t convert(const Side& o, int r0, int nrows, const int4* tab, int tab0,
   a.exps = exps;
   const bool few = (long long)((nrows + 31) / 32) * nb < 2 * sms;
   const dim3 grid(few ? (nrows + 7) / 8 : (nrows + 31) / 32, nb);
-  auto go = [&](auto wide, auto narrow) {
-    if (few) narrow<<<grid, 256, 0, s>>>(a);
-    else wide<<<grid, 256, 0, s>>>(a);
+  const bool rf = o.s_row == 1;
+  auto go = [&](auto wide_rows, auto wide_k, auto narrow_rows, auto narrow_k) {
+    if (few && rf) narrow_rows<<<grid, 256, 0, s>>>(a);
+    else if (few) narrow_k<<<grid, 256, 0, s>>>(a);
+    else if (rf) wide_rows<<<grid, 256, 0, s>>>(a);
+    else wide_k<<<grid, 256, 0, s>>>(a);
   };
-  if (o.src == SRC_COMPLEX) go(rns_convert_kernel<SRC_COMPLEX, 32>, rns_convert_kernel<SRC_COMPLEX, 8>);
-  else if (o.src == SRC_COMPLEX2) go(rns_convert_kernel<SRC_COMPLEX2, 32>, rns_convert_kernel<SRC_COMPLEX2, 8>);
-  else go(rns_convert_kernel<SRC_REAL, 32>, rns_convert_kernel<SRC_REAL, 8>);
+#define DMET_RNS_CONVERT(S)                                                              \
+  go(rns_convert_kernel<S, 32, true>, rns_convert_kernel<S, 32, false>, rns_convert_kernel<S, 8, true>, \
+     rns_convert_kernel<S, 8, false>)
+  if (o.src == SRC_COMPLEX) DMET_RNS_CONVERT(SRC_COMPLEX);
+  else if (o.src == SRC_COMPLEX2) DMET_RNS_CONVERT(SRC_COMPLEX2);
+  else go(rns_convert_kernel<SRC_REAL, 32, true>, rns_convert_kernel<SRC_REAL, 32, true>,
+          rns_convert_kernel<SRC_REAL, 8, true>, rns_convert_kernel<SRC_REAL, 8, true>);  // (real rows are contiguous)
+#undef DMET_RNS_CONVERT
   return cudaGetLastError();
 }
 
@@ -826,19 +861,57 @@ int tile_width(int cols) {
   return (int)pad_to((cols + ct - 1) / ct, 16);
 }
 
+// Row tiles in pairs where the operands' reads bound the GEMM and pairing wastes little: not for a lone row tile nor
+// an odd few, and not for a K of a few blocks, which the epilogue bounds (5720 x 208 x 52 in 36 batches: 266 us
+// alone, 299 in pairs; 5460^2 x 3264, lower triangle: 1.28 PFLOP/s in pairs; the L2 gives some 10 TB/s).
+int cluster_of(int rt, bool tri, int nkb) {
+  return tri || (nkb > 4 && (rt >= 8 || (rt >= 2 && rt % 2 == 0))) ? 2 : 1;
+}
+
+template <int CL>
+cudaError_t launch_gemm(const CUtensorMap& ma, const CUtensorMap& mb, const GemmArgs& g, int njobs, const RnsCtx& c,
+                        cudaStream_t s) {
+  auto kernel = rns_gemm_kernel<CL>;
+  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kGemmSmem);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)CL);
+  cfg.blockDim = dim3(kGemmThreads);
+  cfg.dynamicSmemBytes = kGemmSmem;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  if (CL > 1) {
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = CL;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+  }
+  // as many clusters as run at once (the jobs are dealt out statically)
+  int fit = c.sms / CL;
+  if (CL > 1) {
+    e = cudaOccupancyMaxActiveClusters(&fit, kernel, &cfg);
+    if (e != cudaSuccess) return e;
+    fit = std::max(1, std::min(fit, c.sms / CL));
+  }
+  cfg.gridDim = dim3((unsigned)(std::min(njobs, fit) * CL));
+  return cudaLaunchKernelEx(&cfg, kernel, ma, mb, g, njobs, c.err, c.wait_ns, c.withhold_loads);
+}
+
 cudaError_t gemm(const __nv_bfloat16* RA, long long smodA, const __nv_bfloat16* RB, long long smodB, GemmArgs g, int Kp,
                  int total_rows_a, const RnsCtx& c, cudaStream_t s) {
   CUtensorMap ma, mb;
   cudaError_t e = make_tmap_rows128(&ma, RA, Kp, (unsigned long long)g.nbatch * total_rows_a, kMods, smodA, kTileM);
   if (e != cudaSuccess) return e;
-  e = make_tmap_rows128(&mb, RB, Kp, (unsigned long long)g.nbatch * g.cols, kMods, smodB, g.bn);
+  const int cl = cluster_of(g.rt, g.tri, g.nkb);
+  const int pairs = (g.rt + cl - 1) / cl;
+  g.jobs = g.tri ? tri_jobs_before(pairs, g.h0) : pairs * g.ct;
+  e = make_tmap_rows128(&mb, RB, Kp, (unsigned long long)g.nbatch * g.cols, kMods, smodB, g.bn / cl);
   if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(rns_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kGemmSmem);
-  if (e != cudaSuccess) return e;
-  const int njobs = kMods * g.nbatch * g.tiles;
-  rns_gemm_kernel<<<std::min(njobs, c.sms), kGemmThreads, kGemmSmem, s>>>(ma, mb, g, njobs, c.err, c.wait_ns,
-                                                                           c.withhold_loads);
-  return cudaGetLastError();
+  const int segs = (g.nkb + kSegStages - 1) / kSegStages;
+  g.seg = (g.nkb + segs - 1) / segs;
+  const int njobs = kMods * g.nbatch * g.jobs;
+  return cl == 2 ? launch_gemm<2>(ma, mb, g, njobs, c, s) : launch_gemm<1>(ma, mb, g, njobs, c, s);
 }
 
 // Splits the context's scratch; every piece starts on a 1024-byte boundary.
@@ -968,7 +1041,6 @@ cudaError_t rns_zgemm(const ZgemmArgs& a, int al, bool cj, int bl, const RnsCtx&
       g.rt = (m + kTileM - 1) / kTileM;
       g.bn = tile_width(g.cols);
       g.ct = (g.cols + g.bn - 1) / g.bn;
-      g.tiles = g.rt * g.ct;
       g.nkb = p.Kp / kBK;
       g.Y = Y;
       g.ymod = (long long)n * m * p.ldy;
@@ -1048,7 +1120,6 @@ cudaError_t rns_dsyrk(const DsyrkArgs& a, const RnsCtx& c, cudaStream_t s, int* 
       g.row0 = r0;
       g.bn = tri ? 256 : tile_width(N);
       g.ct = (N + g.bn - 1) / g.bn;
-      g.tiles = tri ? tri_tiles_before(g.rt, g.h0) : g.rt * g.ct;
       g.nkb = Kp / kBK;
       g.Y = Y;
       g.ymod = (long long)m * ldy;

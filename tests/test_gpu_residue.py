@@ -127,3 +127,27 @@ def test_coulomb_exchange_from_factors(torch, mesh, n_aux, n, real):
     Jr, Kr = oracle.coulomb_exchange_df(Lq, gamma, mesh)
     check(J.cpu().numpy().ravel(), Jr)
     check(K.cpu().numpy().ravel(), Kr)
+
+
+@pytest.mark.parametrize("n_aux", [60, 700])
+def test_expired_waits(torch, n_aux):
+    """The residue GEMM's bounded waits, alone and with its CTAs in clusters (the longer products): with the copies
+    withheld they give up after 2 ms, the status says so once, and the same plan then runs normally."""
+    spec = synth.LatticeSpec((3, 2, 1), 24, n_aux, 48, 1, 0.6, 0.0, 76, "r")
+    L, (C,), _ = synth.make_problem(spec)
+    d = B.make_desc(spec.mesh, 24, n_aux, 48)
+    Ld, Cd = torch.from_numpy(L).cuda(), torch.from_numpy(C).cuda()
+    outs = out_buffers(torch, d)
+    plan = dm.dmet_emb_plan(d, stream=torch.cuda.current_stream().cuda_stream)
+    try:
+        dm.dmet_emb_wait_limit(plan, 2_000_000, test_withhold_loads=True)
+        dm.dmet_emb_eri(plan, [Ld], [[Cd]], [outs])
+        st, _ = dm.dmet_emb_status(plan, 0)
+        assert st == B.DMET_ERR_TIMEOUT
+        dm.dmet_emb_wait_limit(plan, 0)
+        dm.dmet_emb_eri(plan, [Ld], [[Cd]], [outs])
+        st, _ = dm.dmet_emb_status(plan, 0)
+        assert st == B.DMET_OK
+    finally:
+        dm.dmet_emb_destroy(plan)
+    check(outs[0].cpu().numpy(), oracle.pack_s8(oracle.embedded_eri(L, C, spec.mesh).real))
