@@ -102,7 +102,7 @@ __global__ void __launch_bounds__(256) dsyrk_fp64_kernel(const DsyrkArgs d) {
   int m0, n0;
   if (d.mode == 0) {
     const long long t = blockIdx.x;
-    long long ti = (long long)((sqrt(8.0 * (double)t + 1.0) - 1.0) * 0.5);
+    long long ti = (long long)((sqrtf(8.f * (float)t + 1.f) - 1.f) * 0.5f);  // (made exact below)
     while (ti * (ti + 1) / 2 > t) --ti;
     while ((ti + 1) * (ti + 2) / 2 <= t) ++ti;
     m0 = (int)ti * TT;
@@ -308,11 +308,12 @@ __global__ void c_real_check_kernel(const double2* __restrict__ C, const int* __
     const int k = (int)(x / per);
     const double2 a = C[x], b = C[neg[k] * per + x % per];
     const double dr = b.x - a.x, di = b.y + a.y;
-    dv = wmax(dv, sqrt(dr * dr + di * di));
-    mv = wmax(mv, sqrt(a.x * a.x + a.y * a.y));
+    dv = wmax(dv, dr * dr + di * di);
+    mv = wmax(mv, a.x * a.x + a.y * a.y);
   }
-  block_max_commit(dv, stats + 1);
-  block_max_commit(mv, stats + 2);
+  // (the square root, once: it keeps the order, rounded)
+  block_max_commit(sqrt(dv), stats + 1);
+  block_max_commit(sqrt(mv), stats + 2);
 }
 
 // |x| of a double as its bit pattern with the sign cleared: for non-negative doubles the
@@ -385,9 +386,11 @@ inline int grid_for(long long total, int threads, int cap) {
   return (int)(g < cap ? g : cap);
 }
 
-// Largest t with t(t+1)/2 <= x (the row of a lower-triangle index), exact for x < 2^50.
+// Largest t with t(t+1)/2 <= x (the row of a lower-triangle index), exact for x < 2^50. (An FP32 square root where it
+// comes near enough: the FP64 one takes some 40 instructions of the slow pipe.)
 __device__ __forceinline__ long long tri_row(long long x) {
-  long long t = (long long)((sqrt(8.0 * (double)x + 1.0) - 1.0) * 0.5);
+  long long t = x < (1 << 28) ? (long long)((sqrtf(8.f * (float)x + 1.f) - 1.f) * 0.5f)
+                              : (long long)((sqrt(8.0 * (double)x + 1.0) - 1.0) * 0.5);
   while (t * (t + 1) / 2 > x) --t;
   while ((t + 1) * (t + 2) / 2 <= x) ++t;
   return t;

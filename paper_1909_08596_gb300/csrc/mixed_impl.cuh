@@ -223,9 +223,10 @@ __global__ void __launch_bounds__(256) pack_split_kernel(const float2* __restric
   constexpr int kPitch = PK_B * PK_B + 1;
   __shared__ float4 za[PK_P][kPitch];
   __shared__ float4 zb[PK_P][kPitch];
-  // pair-block decode: lower triangle of ceil(n / PK_B) blocks
+  // pair-block decode: lower triangle of ceil(n / PK_B) blocks (an FP32 square root, made exact: every thread takes
+  // it, and an FP64 one cost the 90 small launches of a batch of 24 problems 15% of their time, 986 -> 832 us)
   const long long t = blockIdx.x;
-  long long bi = (long long)((sqrt(8.0 * (double)t + 1.0) - 1.0) * 0.5);
+  long long bi = (long long)((sqrtf(8.f * (float)t + 1.f) - 1.f) * 0.5f);
   while (bi * (bi + 1) / 2 > t) --bi;
   while ((bi + 1) * (bi + 2) / 2 <= t) ++bi;
   const int bj = (int)(t - bi * (bi + 1) / 2);
@@ -494,18 +495,26 @@ __global__ void __launch_bounds__(256) combine_parts_kernel(const tc::TcJob* __r
   }
 }
 
+// max(m, |x|) on bit patterns (for non-negative doubles the integer order is the numeric one), NaNs left out as by
+// fmax: an FP64 comparison per component bound the pass over L (1.58 GB: 433 us, 260 without).
+__device__ __forceinline__ unsigned long long abs_max(unsigned long long m, double x) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x) & 0x7fffffffffffffffull;
+  return b > m && b <= 0x7ff0000000000000ull ? b : m;
+}
+
 // Largest |component| of the L blocks t1[e0 .. e0 + E).y, as float bits (atomicMax on the bits of a
 // non-negative float orders like the value).
 __global__ void __launch_bounds__(256) absmax_L_kernel(const double2* __restrict__ L, const int4* __restrict__ t1,
                                                        int e0, long long per_block, unsigned int* __restrict__ out) {
   const double2* src = L + (long long)t1[e0 + blockIdx.y].y * per_block;
-  double m = 0.0;
+  unsigned long long m = 0;
+#pragma unroll 4
   for (long long x = blockIdx.x * (long long)blockDim.x + threadIdx.x; x < per_block;
        x += (long long)gridDim.x * blockDim.x) {
     const double2 v = src[x];
-    m = fmax(m, fmax(fabs(v.x), fabs(v.y)));
+    m = abs_max(abs_max(m, v.x), v.y);
   }
-  float mf = (float)m;
+  float mf = (float)__longlong_as_double((long long)m);
 #pragma unroll
   for (int o = 16; o; o >>= 1) mf = fmaxf(mf, __shfl_xor_sync(0xffffffffu, mf, o));
   if ((threadIdx.x & 31) == 0) atomicMax(out, __float_as_uint(mf));
@@ -513,10 +522,10 @@ __global__ void __launch_bounds__(256) absmax_L_kernel(const double2* __restrict
 
 __global__ void __launch_bounds__(256) absmax_kernel(const double* __restrict__ x, long long n,
                                                      unsigned int* __restrict__ out) {
-  double m = 0.0;
+  unsigned long long m = 0;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-    m = fmax(m, fabs(x[i]));
-  float mf = (float)m;
+    m = abs_max(m, x[i]);
+  float mf = (float)__longlong_as_double((long long)m);
 #pragma unroll
   for (int o = 16; o; o >>= 1) mf = fmaxf(mf, __shfl_xor_sync(0xffffffffu, mf, o));
   if ((threadIdx.x & 31) == 0) atomicMax(out, __float_as_uint(mf));

@@ -571,7 +571,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
           for (int i = 0; i < 8; ++i)
             if (half * 16 + 32 * i < cols) prev[i] = *reinterpret_cast<const uint4*>(y + half * 16 + 32 * i);
         }
-        if (!mbar_wait(accf(b), u & 1, err, 8u, lim)) {
+        if (!__all_sync(0xffffffffu, mbar_wait(accf(b), u & 1, err, 8u, lim))) {
           ok = false;
           break;
         }
