@@ -211,72 +211,95 @@ __global__ void build_Cc_kernel(const double2* __restrict__ C, const int4* __res
 // Xt[t][IJ][row_base + (slot * naux + P) * nc + c] = split of sX (Z_ij + Z_ji).c for i >= j, where
 // each real component of Z_ij (complex) is a two-float pair ZT[slot][(P n + j) 2n + 2i + (re|im)].
 // (The factor s of L^q = s (Z + Z^T) is applied, squared, to the contraction's output.)
-constexpr int PK_P = 64, PK_B = 4;
+//
+// Bound by memory: 16 bytes of ZT in and 2 kSlices sizeof(T) / 2 out per complex element. A block takes 32 P of one 8 x 8
+// block of pairs, so that ZT is read in runs of 128 bytes on both sides of the transposition (blocks of 4 x 4 read half
+// lines). The Z_ij of a thread come through shared memory, its Z_ji stay in registers, and the slices go out through the
+// same shared memory as (re, im) pairs in runs of 32 P. The three launches of the h-BN-shaped problem (BF16x3, n = 104):
+// 290 us with blocks of 64 P x 4 x 4 and 2-byte stores, 173 now (1.2 GB: 6.8 TB/s); the NiO-shaped one (FP16x2, n = 119,
+// 113): 832 -> 424 us.
+constexpr int PK_P = 32, PK_B = 8;
 template <class PREC>
 __global__ void __launch_bounds__(256) pack_split_kernel(const float2* __restrict__ ZT, int naux, int n, int nc,
-                                                         typename PREC::T* __restrict__ Xt, long long sstride,
-                                                         long long Rtot, long long row_base,
+                                                         int nptiles, typename PREC::T* __restrict__ Xt,
+                                                         long long sstride, long long Rtot, long long row_base,
                                                          const float* __restrict__ psx) {
+  using T = typename PREC::T;
   const float sx = PREC::kScaled ? *psx : 1.f;
-  // (re.hi, re.lo, im.hi, im.lo) of (pl, ii, jj) at [pl][ii * PK_B + jj]; the odd row pitch puts
-  // consecutive pl (the lanes of the write phase) in different banks.
-  constexpr int kPitch = PK_B * PK_B + 1;
-  __shared__ float4 za[PK_P][kPitch];
-  __shared__ float4 zb[PK_P][kPitch];
+  constexpr int kPairs = PK_B * PK_B, kQ = PK_B * (PK_B + 1);  // (pitch 9 of ii: conflict-free both ways)
+  constexpr int NS = PREC::kSlices, kOutPitch = PK_P + 1;
+  // (re.hi, re.lo, im.hi, im.lo) of (pl, ii, jj) at [pl][ii * 9 + jj]; then the slices [t][pair][pl]
+  __shared__ float4 smem[PK_P * kQ];
+  static_assert(sizeof(Pair2<T>) * NS * kPairs * kOutPitch <= sizeof(smem), "the slices fit where Z was");
+  Pair2<T>* out = reinterpret_cast<Pair2<T>*>(smem);
   // pair-block decode: lower triangle of ceil(n / PK_B) blocks (an FP32 square root, made exact: every thread takes
   // it, and an FP64 one cost the 90 small launches of a batch of 24 problems 15% of their time, 986 -> 832 us)
-  const long long t = blockIdx.x;
+  const int t = blockIdx.x / nptiles;
   long long bi = (long long)((sqrtf(8.f * (float)t + 1.f) - 1.f) * 0.5f);
   while (bi * (bi + 1) / 2 > t) --bi;
   while ((bi + 1) * (bi + 2) / 2 <= t) ++bi;
   const int bj = (int)(t - bi * (bi + 1) / 2);
   const int i0 = (int)bi * PK_B, j0 = bj * PK_B;
-  const int P0 = blockIdx.y * PK_P;
-  const int slot = blockIdx.z;
+  const int P0 = (blockIdx.x % nptiles) * PK_P;
+  const int slot = blockIdx.y;
   const float4* z = reinterpret_cast<const float4*>(ZT + (long long)slot * naux * n * 2 * n);
-  // All loads of a thread are issued before any is stored (256 threads).
-  constexpr int kPer = PK_P * PK_B * PK_B / 256;
+  // All loads of a thread are issued before any is used. Its elements are (pl, a, b) = (w + 4 r, a, b) for the r-th.
+  constexpr int kPer = PK_P * kPairs / 256;
+  const int w = threadIdx.x / kPairs, a = (threadIdx.x / PK_B) % PK_B, b = threadIdx.x % PK_B;
   float4 va[kPer], vb[kPer];
 #pragma unroll
   for (int r = 0; r < kPer; ++r) {
-    const int e = threadIdx.x + r * 256;
-    const int pl = e / (PK_B * PK_B), a = (e / PK_B) % PK_B, b = e % PK_B;
-    const int P = P0 + pl;
-    // za[pl][ii][jj] = Z_{i j} with (ii, jj) = (b, a): consecutive e run over i for fixed j.
+    const int P = P0 + w + r * (256 / kPairs);
+    // Z_{i j} with (ii, jj) = (b, a): consecutive threads run over i for fixed j.
     va[r] = make_float4(0.f, 0.f, 0.f, 0.f);
     if (P < naux && i0 + b < n && j0 + a < n) va[r] = z[((long long)P * n + j0 + a) * n + i0 + b];
-    // zb[pl][ii][jj] = Z_{j i} with (ii, jj) = (a, b): consecutive e run over j for fixed i.
+    // Z_{j i} with (ii, jj) = (a, b): consecutive threads run over j for fixed i.
     vb[r] = make_float4(0.f, 0.f, 0.f, 0.f);
     if (P < naux && i0 + a < n && j0 + b < n) vb[r] = z[((long long)P * n + i0 + a) * n + j0 + b];
   }
 #pragma unroll
+  for (int r = 0; r < kPer; ++r) smem[(w + r * (256 / kPairs)) * kQ + b * (PK_B + 1) + a] = va[r];
+  __syncthreads();
+#pragma unroll
+  for (int r = 0; r < kPer; ++r) va[r] = smem[(w + r * (256 / kPairs)) * kQ + a * (PK_B + 1) + b];
+  __syncthreads();
+#pragma unroll
   for (int r = 0; r < kPer; ++r) {
-    const int e = threadIdx.x + r * 256;
-    const int pl = e / (PK_B * PK_B), a = (e / PK_B) % PK_B, b = e % PK_B;
-    za[pl][b * PK_B + a] = va[r];
-    zb[pl][a * PK_B + b] = vb[r];
+    T x[2][3];
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      const float ah = c == 0 ? va[r].x : va[r].z, al = c == 0 ? va[r].y : va[r].w;
+      const float bh = c == 0 ? vb[r].x : vb[r].z, bl = c == 0 ? vb[r].y : vb[r].w;
+      // (ah + al) + (bh + bl) as a two-float pair: TwoSum of the leading parts.
+      const float sh = ah + bh, bv = sh - ah;
+      const float sl = ((ah - (sh - bv)) + (bh - bv)) + (al + bl);
+      PREC::split(sh * sx, sl * sx, x[c]);
+    }
+#pragma unroll
+    for (int q = 0; q < NS; ++q)
+      out[(q * kPairs + a * PK_B + b) * kOutPitch + w + r * (256 / kPairs)] = Pair2<T>{x[0][q], x[1][q]};
   }
   __syncthreads();
-  const int nr = PK_P * nc;  // rows per pair in this block
-  for (int e = threadIdx.x; e < PK_B * PK_B * nr; e += blockDim.x) {
-    const int pr = e / nr, rl = e % nr;
-    const int ii = pr / PK_B, jj = pr % PK_B;
-    const int i = i0 + ii, j = j0 + jj;
-    const int pl = rl / nc, c = rl % nc;
-    const int P = P0 + pl;
-    if (i >= n || j > i || P >= naux) continue;
-    const float4 a = za[pl][ii * PK_B + jj], b = zb[pl][ii * PK_B + jj];
-    const float ah = c == 0 ? a.x : a.z, al = c == 0 ? a.y : a.w;
-    const float bh = c == 0 ? b.x : b.z, bl = c == 0 ? b.y : b.w;
-    // (ah + al) + (bh + bl) as a two-float pair: TwoSum of the leading parts.
-    const float sh = ah + bh, bv = sh - ah;
-    const float sl = ((ah - (sh - bv)) + (bh - bv)) + (al + bl);
-    const long long IJ = (long long)i * (i + 1) / 2 + j;
-    const long long idx = IJ * Rtot + row_base + ((long long)slot * naux + P) * nc + c;
-    typename PREC::T x[3];
-    PREC::split(sh * sx, sl * sx, x);
+  const int lane = threadIdx.x & 31, P = P0 + lane;
+  if (P >= naux) return;
+  const long long k0 = row_base + ((long long)slot * naux + P) * nc;
+  // (both components in one store where every row and slice starts on such a boundary)
+  const bool pairs = nc == 2 && ((row_base | Rtot | sstride) & 1) == 0 &&
+                     (reinterpret_cast<unsigned long long>(Xt) & (sizeof(Pair2<T>) - 1)) == 0;
+  for (int pr = threadIdx.x >> 5; pr < kPairs; pr += 8) {
+    const int i = i0 + pr / PK_B, j = j0 + pr % PK_B;
+    if (i >= n || j > i) continue;
+    T* row = Xt + ((long long)i * (i + 1) / 2 + j) * Rtot + k0;
 #pragma unroll
-    for (int q = 0; q < PREC::kSlices; ++q) Xt[idx + q * sstride] = x[q];
+    for (int q = 0; q < NS; ++q) {
+      const Pair2<T> v = out[(q * kPairs + pr) * kOutPitch + lane];
+      if (pairs) {
+        *reinterpret_cast<Pair2<T>*>(row + q * sstride) = v;
+      } else {
+        row[q * sstride] = v.a;
+        if (nc == 2) row[q * sstride + 1] = v.b;
+      }
+    }
   }
 }
 
@@ -289,12 +312,14 @@ __global__ void __launch_bounds__(256) pack_split_kernel(const float2* __restric
 // the bra rows against the ket rows, whose output row ij is (ij|kl) as (re, im) doubles over kl.
 // Z_ij of slot sl is the two-float pair ZT[sl][(P n + j) n + i] (re.hi, re.lo, im.hi, im.lo); the
 // factor s of L^q = s Z is applied, squared, to the contraction's output. One block stages a tile
-// of 32 P x 32 i at one j (reads coalesced over i), then writes runs of 32 consecutive P per row.
+// of 64 P x 16 i at one j (reads in runs of 256 bytes over i), then writes runs of 64 consecutive P per row, two P to
+// a lane. Bound by its writes, six per slice of each Z: one 16-bit element per lane and store left half of each
+// request empty (8 q of 220 x 104^2: 417 us; now 338).
 __device__ __forceinline__ float neg_of(float x) { return -x; }
 __device__ __forceinline__ __half neg_of(__half x) { return __hneg(x); }
 __device__ __forceinline__ __nv_bfloat16 neg_of(__nv_bfloat16 x) { return __hneg(x); }
 
-constexpr int PC_T = 32;
+constexpr int PC_P = 64, PC_I = 16;
 template <class PREC>
 __global__ void __launch_bounds__(256) pack_cplx_kernel(const float4* __restrict__ ZT, int naux, int n, int nq,
                                                         int q0, const int* __restrict__ neg,
@@ -302,33 +327,48 @@ __global__ void __launch_bounds__(256) pack_cplx_kernel(const float4* __restrict
                                                         long long Rtot, const float* __restrict__ psx) {
   using T = typename PREC::T;
   const float sx = PREC::kScaled ? *psx : 1.f;
-  __shared__ float4 z[PC_T][PC_T + 1];  // [i][P]
-  const int itiles = (n + PC_T - 1) / PC_T;
-  const int i0 = (blockIdx.x % itiles) * PC_T, j = blockIdx.x / itiles;
-  const int P0 = blockIdx.y * PC_T;
+  __shared__ float4 z[PC_I][PC_P + 1];  // [i][P]
+  const int itiles = (n + PC_I - 1) / PC_I;
+  const int i0 = (blockIdx.x % itiles) * PC_I, j = blockIdx.x / itiles;
+  const int P0 = blockIdx.y * PC_P;
   const int sl = blockIdx.z;
-  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
   const float4* zs = ZT + (long long)sl * naux * n * n;
 #pragma unroll
-  for (int r = 0; r < PC_T / 8; ++r) {
-    const int pl = ty + r * 8, P = P0 + pl, i = i0 + tx;
+  for (int r = 0; r < PC_P * PC_I / 256; ++r) {
+    const int il = threadIdx.x % PC_I, pl = threadIdx.x / PC_I + r * (256 / PC_I);
+    const int i = i0 + il, P = P0 + pl;
     float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
     if (P < naux && i < n) v = zs[((long long)P * n + j) * n + i];
-    z[tx][pl] = v;
+    z[il][pl] = v;
   }
   __syncthreads();
-  const int q = q0 + sl, P = P0 + tx;
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  const int q = q0 + sl, P = P0 + 2 * tx;
   if (P >= naux) return;
+  const bool two = P + 1 < naux;
+  // (the pair of P in one store where every block, row and slice starts on such a boundary)
+  const bool wide = two && ((naux | Rtot | sstride) & 1) == 0 &&
+                    (reinterpret_cast<unsigned long long>(Xt) & (sizeof(Pair2<T>) - 1)) == 0;
   const long long kb = (long long)q * 2 * naux + P, kn = (long long)neg[q] * 2 * naux + P;
   const long long n2 = (long long)n * n;
+  auto put = [&](T* dst, T x, T y) {
+    if (wide) {
+      *reinterpret_cast<Pair2<T>*>(dst) = Pair2<T>{x, y};
+    } else {
+      dst[0] = x;
+      if (two) dst[1] = y;
+    }
+  };
 #pragma unroll
-  for (int r = 0; r < PC_T / 8; ++r) {
+  for (int r = 0; r < PC_I / 8; ++r) {
     const int il = ty + r * 8, i = i0 + il;
     if (i >= n) break;
-    const float4 v = z[il][tx];
-    T re[3], im[3];
-    PREC::split(v.x * sx, v.y * sx, re);
-    PREC::split(v.z * sx, v.w * sx, im);
+    const float4 u = z[il][2 * tx], v = z[il][2 * tx + 1];
+    T re[3], im[3], re1[3], im1[3];
+    PREC::split(u.x * sx, u.y * sx, re);
+    PREC::split(u.z * sx, u.w * sx, im);
+    PREC::split(v.x * sx, v.y * sx, re1);
+    PREC::split(v.z * sx, v.w * sx, im1);
     const long long ij = (long long)i * n + j;
     T* a = Xt + ij * Rtot;
     T* b0 = Xt + (n2 + 2 * ij) * Rtot;
@@ -336,12 +376,12 @@ __global__ void __launch_bounds__(256) pack_cplx_kernel(const float4* __restrict
 #pragma unroll
     for (int t = 0; t < PREC::kSlices; ++t) {
       const long long o = t * sstride;
-      a[o + kb] = re[t];
-      a[o + kb + naux] = im[t];
-      b0[o + kn] = re[t];
-      b0[o + kn + naux] = neg_of(im[t]);
-      b1[o + kn] = im[t];
-      b1[o + kn + naux] = re[t];
+      put(a + o + kb, re[t], re1[t]);
+      put(a + o + kb + naux, im[t], im1[t]);
+      put(b0 + o + kn, re[t], re1[t]);
+      put(b0 + o + kn + naux, neg_of(im[t]), neg_of(im1[t]));
+      put(b1 + o + kn, im[t], im1[t]);
+      put(b1 + o + kn + naux, re[t], re1[t]);
     }
   }
 }
@@ -684,10 +724,12 @@ cudaError_t DMET_P(launch_build_Cc)(int prec, const double2* C, const int4* gath
 cudaError_t DMET_P(launch_pack_split)(int prec, const void* ZT, int nq, int naux, int n, int nc, void* Xt, long long sstride,
                               long long Rtot, long long row_base, const float* sx, cudaStream_t s) {
   const long long nb = (n + PK_B - 1) / PK_B;
-  const dim3 grid((unsigned)(nb * (nb + 1) / 2), (naux + PK_P - 1) / PK_P, nq);
+  const int pt = (naux + PK_P - 1) / PK_P;
+  if (nb * (nb + 1) / 2 * pt > 0x7fffffffLL || nq > 65535) return cudaErrorInvalidValue;
+  const dim3 grid((unsigned)(nb * (nb + 1) / 2 * pt), nq);
   return with_prec(prec, [&](auto tag) -> cudaError_t {
     using P = decltype(tag);
-    pack_split_kernel<P><<<grid, 256, 0, s>>>((const float2*)ZT, naux, n, nc, (typename P::T*)Xt, sstride, Rtot,
+    pack_split_kernel<P><<<grid, 256, 0, s>>>((const float2*)ZT, naux, n, nc, pt, (typename P::T*)Xt, sstride, Rtot,
                                               row_base, sx);
     return cudaGetLastError();
   });
@@ -695,9 +737,9 @@ cudaError_t DMET_P(launch_pack_split)(int prec, const void* ZT, int nq, int naux
 
 cudaError_t DMET_P(launch_pack_cplx)(int prec, const void* ZT, int nq, int naux, int n, int q0, const int* neg, void* Xt,
                              long long sstride, long long Rtot, const float* sx, cudaStream_t s) {
-  const long long gx = (long long)((n + PC_T - 1) / PC_T) * n;
-  if (gx > 0x7fffffffLL || nq > 65535 || (naux + PC_T - 1) / PC_T > 65535) return cudaErrorInvalidValue;
-  const dim3 grid((unsigned)gx, (naux + PC_T - 1) / PC_T, nq);
+  const long long gx = (long long)((n + PC_I - 1) / PC_I) * n;
+  if (gx > 0x7fffffffLL || nq > 65535 || (naux + PC_P - 1) / PC_P > 65535) return cudaErrorInvalidValue;
+  const dim3 grid((unsigned)gx, (naux + PC_P - 1) / PC_P, nq);
   return with_prec(prec, [&](auto tag) -> cudaError_t {
     using P = decltype(tag);
     pack_cplx_kernel<P><<<grid, 256, 0, s>>>((const float4*)ZT, naux, n, nq, q0, neg, (typename P::T*)Xt, sstride,
