@@ -216,7 +216,7 @@ __global__ void build_Cc_kernel(const double2* __restrict__ C, const int4* __res
 // block of pairs, so that ZT is read in runs of 128 bytes on both sides of the transposition (blocks of 4 x 4 read half
 // lines). The Z_ij of a thread come through shared memory, its Z_ji stay in registers, and the slices go out through the
 // same shared memory as (re, im) pairs in runs of 32 P. The three launches of the h-BN-shaped problem (BF16x3, n = 104):
-// 290 us with blocks of 64 P x 4 x 4 and 2-byte stores, 173 now (1.2 GB: 6.8 TB/s); the NiO-shaped one (FP16x2, n = 119,
+// 290 us with blocks of 64 P x 4 x 4 and 2-byte stores, 173 now (1.05 GB: 6.1 TB/s); the NiO-shaped one (FP16x2, n = 119,
 // 113): 832 -> 424 us.
 constexpr int PK_P = 32, PK_B = 8;
 template <class PREC>

@@ -321,7 +321,7 @@ __global__ void __launch_bounds__(256) rns_convert_kernel(const ConvArgs a) {
     else return element(r, u);
   };
   // a thread's share of the transpose of the tile of 32 pairs from u on: the next tile's is loaded before the current
-  // one is converted (22 880 x 520: 286 us without, 250 with)
+  // one is converted (22 880 x 520: 286 us without, 224 with)
   static_assert(RW * KL == 32, "a thread's share of a tile");
   double2 next[RW];
   auto fetch = [&](int u) {
@@ -380,10 +380,18 @@ struct GemmArgs {
   int row0;                 // first row of the launch in the row operand
   int jobs;                 // (clusters of tiles) per (modulus, batch)
   int nkb, seg;             // K blocks, and how many of them between reductions (at most kSegStages)
-  signed char* Y;           // [mod][batch][rows][ldy]
+  signed char* Y;           // [mod][batch] in tiles (y_tile)
   long long ymod;
   int ldy;
 };
+
+// Y, the products' residues, lies in tiles of 32 rows x 16 columns, a row's 16 bytes after the other's: a warp of the
+// GEMM's epilogue stores, and one of the reconstruction loads, 512 contiguous bytes with a lane per row. (Row by row
+// the same accesses touched 32 lines each: 5720 x 208 x 52 in 55 batches took 523 us for the GEMM and 509 for the
+// reconstruction, 357 and 324 now.) Offset of the tile with row group rg and column c (a multiple of 16) of a batch entry of `rows` rows.
+__host__ __device__ inline long long y_tile(int z, int rows, int ldy, int rg, int c) {
+  return (((long long)z * ((rows + 31) >> 5) + rg) * (ldy >> 4) + (c >> 4)) * 512;
+}
 
 struct Tile {
   int mod, z, m0, n0;
@@ -558,7 +566,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
       const Tile t = tile_of<CL>(g, jb, rank);
       const float p = kModF[t.mod], rp = 1.0f / p;
       const int row = t.m0 + quad * 32 + lane;
-      signed char* y = g.Y + (long long)t.mod * g.ymod + ((long long)t.z * g.rows + row) * g.ldy + t.n0;
+      signed char* y =
+          g.Y + (long long)t.mod * g.ymod + y_tile(t.z, g.rows, g.ldy, t.m0 / 32 + quad, t.n0) + lane * 16;
       const bool rok = row < g.rows;
       const int cols = min(g.bn, g.ldy - t.n0);
       for (int k0 = 0; k0 < g.nkb; k0 += g.seg, ++gs) {
@@ -569,7 +578,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
         if (k0 && rok) {
 #pragma unroll
           for (int i = 0; i < 8; ++i)
-            if (half * 16 + 32 * i < cols) prev[i] = *reinterpret_cast<const uint4*>(y + half * 16 + 32 * i);
+            if (half * 16 + 32 * i < cols) prev[i] = *reinterpret_cast<const uint4*>(y + (half + 2 * i) * 512);
         }
         if (!__all_sync(0xffffffffu, mbar_wait(accf(b), u & 1, err, 8u, lim))) {
           ok = false;
@@ -585,7 +594,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
           tmem_ld_32x32b_x16(tm + c, v);
           tmem_ld_wait();
           const uint4 w = reduce16(v, k0 != 0, prev[i], p, rp);
-          if (rok) *reinterpret_cast<uint4*>(y + c) = w;
+          if (rok) *reinterpret_cast<uint4*>(y + (half + 2 * i) * 512) = w;
         }
         tc_fence_before();
         __syncwarp();
@@ -745,8 +754,8 @@ __device__ __forceinline__ void store_complex(const CrtArgs& a, double2* D, cons
 
 // A warp takes 32 rows x 16 columns, a lane per row, 8 columns at a time (15 planes of 8 bytes in registers, so
 // that four CTAs fit an SM). Bound by issue (157 instructions per value, 45 of them the multiply-adds of the
-// fractions; IPC 2): 23.8 M values in 190 us. The same with the whole integer in 64-bit multiply-adds on
-// 30-bit limbs and 16 columns a time took 238 instructions at half the occupancy, 390 us.
+// fractions): 65.4 M values in 324 us. The same with the whole integer in 64-bit multiply-adds on
+// 30-bit limbs and 16 columns a time took 238 instructions at half the occupancy, twice the time.
 template <bool CPLX>
 __global__ void __launch_bounds__(256, 4) rns_crt_kernel(const CrtArgs a) {
   __shared__ double stage[8][32 * 17];
@@ -760,7 +769,7 @@ __global__ void __launch_bounds__(256, 4) rns_crt_kernel(const CrtArgs a) {
   if (rbase >= a.rows) return;                                     // (whole warps leave)
   if (!CPLX && a.tri && c0 > a.row0 + rbase + 31) return;
   const bool rok = row < a.rows;
-  const signed char* yp = a.Y + ((long long)z * a.rows + (rok ? row : 0)) * a.ldy + c0;
+  const signed char* yp = a.Y + y_tile(z, a.rows, a.ldy, rg, c0) + lane * 16;  // (rows past the end: padding)
   const int sa = rok ? a.ea[(long long)z * a.ea_rows + row] : 0;
   const int* ebp = a.eb + (long long)z * a.eb_rows;
   double* st = stage[warp];
@@ -947,7 +956,7 @@ ZPlan zplan(const ZgemmArgs& a, int al, bool cj, int bl) {
   p.ldy = (int)pad_to(2ll * p.cols.rows, 16);
   p.row_bytes = (size_t)p.rows.rows * p.Kp * 2 * kMods;
   p.col_bytes = (size_t)2 * p.cols.rows * p.Kp * 2 * kMods;
-  p.y_bytes = (size_t)p.rows.rows * p.ldy * kMods;
+  p.y_bytes = (size_t)pad_to(p.rows.rows, 32) * p.ldy * kMods;
   return p;
 }
 
@@ -960,7 +969,7 @@ size_t rns_need(const ZgemmArgs& a) {
 
 size_t rns_need(const DsyrkArgs& a) {
   const size_t kp = (size_t)pad_to(a.K, kBK), rows = (size_t)a.M + (a.mode ? a.N : 0);
-  return rows * kp * 2 * kMods + (size_t)a.M * pad_to(a.N, 16) * kMods + rows * 4 + 65536;
+  return rows * kp * 2 * kMods + (size_t)pad_to(a.M, 32) * pad_to(a.N, 16) * kMods + rows * 4 + 65536;
 }
 
 // Where the line between the two lies (fitted to shapes from 8 x 256 x 8 to 128 x 22 880 x 1024, single and batched): the
@@ -1003,7 +1012,7 @@ cudaError_t rns_zgemm(const ZgemmArgs& a, int al, bool cj, int bl, const RnsCtx&
       __nv_bfloat16* RB = (__nv_bfloat16*)w.take((size_t)smB * 2 * kMods);
       int* eb = (int*)w.take((size_t)n * p.cols.rows * 4);
       __nv_bfloat16* RA = (__nv_bfloat16*)w.take((size_t)smA * 2 * kMods);
-      signed char* Y = (signed char*)w.take((size_t)n * m * p.ldy * kMods);
+      signed char* Y = (signed char*)w.take((size_t)n * pad_to(m, 32) * p.ldy * kMods);
       int* ea = (int*)w.take((size_t)n * m * 4);
       if (w.p > w.end) return cudaErrorInvalidValue;
       cudaError_t e = cudaSuccess;
@@ -1043,7 +1052,7 @@ cudaError_t rns_zgemm(const ZgemmArgs& a, int al, bool cj, int bl, const RnsCtx&
       g.ct = (g.cols + g.bn - 1) / g.bn;
       g.nkb = p.Kp / kBK;
       g.Y = Y;
-      g.ymod = (long long)n * m * p.ldy;
+      g.ymod = (long long)n * pad_to(m, 32) * p.ldy;
       g.ldy = p.ldy;
       if ((e = gemm(RA, smA, RB, smB, g, p.Kp, m, c, s)) != cudaSuccess) return e;
       x.Y = Y;
@@ -1095,7 +1104,7 @@ cudaError_t rns_dsyrk(const DsyrkArgs& a, const RnsCtx& c, cudaStream_t s, int* 
     __nv_bfloat16* RB = tri ? RA : (__nv_bfloat16*)w.take((size_t)smB * 2 * kMods);
     int* ea = (int*)w.take((size_t)M * 4);
     int* eb = tri ? ea : (int*)w.take((size_t)N * 4);
-    signed char* Y = (signed char*)w.take((size_t)std::min((long long)nr, (long long)M) * ldy * kMods);
+    signed char* Y = (signed char*)w.take((size_t)std::min<long long>(nr, pad_to(M, 32)) * ldy * kMods);
     if (w.p > w.end) return cudaErrorInvalidValue;
     Side xs = X, ys = Yo;
     xs.base += k0 * a.ldx;
@@ -1122,7 +1131,7 @@ cudaError_t rns_dsyrk(const DsyrkArgs& a, const RnsCtx& c, cudaStream_t s, int* 
       g.ct = (N + g.bn - 1) / g.bn;
       g.nkb = Kp / kBK;
       g.Y = Y;
-      g.ymod = (long long)m * ldy;
+      g.ymod = pad_to(m, 32) * ldy;
       g.ldy = (int)ldy;
       e = gemm(RA, smA, RB, smB, g, Kp, M, c, s);
       if (e != cudaSuccess) return e;
