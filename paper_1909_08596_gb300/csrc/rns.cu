@@ -109,14 +109,37 @@ __host__ __device__ constexpr int chunk_weight(int i, int j) {
 }
 
 constexpr int kPoison = -(1 << 28);  // scale of a row that holds an infinity or a NaN
-constexpr float kMagic = 12582912.f;  // 1.5 * 2^23: adding it rounds to an integer
 
-// v - p * rint(v / p) for an integer |v| <= 2^24: a residue with |r| <= (p + 1) / 2 (the rounding of v / p
+// Two values at a time on the paired FP32 pipe, each rounded as the scalar form (x: the low half). Instructions bound
+// the conversion (issue at 79%): 22 880 x 520 in 224 us with the scalar form, 204 with this; the GEMM of
+// 5720 x 208 x 52 in 55 batches, bound by its epilogue, 357 and 315.
+using f32x2 = unsigned long long;
+constexpr f32x2 both(unsigned bits) { return ((f32x2)bits << 32) | bits; }
+__device__ __forceinline__ f32x2 pack2(float x, float y) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
+  return r;
+}
+__device__ __forceinline__ void unpack2(f32x2 v, float& x, float& y) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(v));
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+constexpr f32x2 both_of(float x) { return both(__builtin_bit_cast(unsigned, x)); }
+constexpr f32x2 kMagic2 = both(0x4B400000u), kMinusMagic2 = both(0xCB400000u);  // +- 1.5 * 2^23: rounds to an integer
+// v - p * rint(v / p) for integers |v| <= 2^24: a residue with |r| <= (p + 1) / 2 (the rounding of v / p
 // can pick the neighbour when v / p lies within 2^-9 of a half-integer), so at most 128 for p = 256 and
 // 127 for the others: it fits a byte, modulo 256 for p = 256. (p = 255 would reach 128 and is left out.)
-__device__ __forceinline__ float sym_mod(float v, float p, float rp) {
-  const float q = __fadd_rn(fmaf(v, rp, kMagic), -kMagic);
-  return fmaf(q, -p, v);
+__device__ __forceinline__ f32x2 sym_mod2(f32x2 v, f32x2 minus_p, f32x2 rp) {
+  return fma2(add2(fma2(v, rp, kMagic2), kMinusMagic2), minus_p, v);
 }
 
 __constant__ float kModF[kMods] = {256, 253, 251, 247, 241, 239, 233, 229, 227, 223, 217, 211, 199, 197, 193};
@@ -210,30 +233,49 @@ __device__ __forceinline__ void digits(long long a, float (&c)[4]) {
 }
 
 // |c_j w_j| <= 2^22 for j = 1, 2, 2^18 for j = 3 (|a| <= 2^59) and 2^15 for j = 0: the sum is exact.
-template <int I>
-__device__ __forceinline__ float residue(const float (&c)[4]) {
-  constexpr float w1 = (float)chunk_weight(I, 1), w2 = (float)chunk_weight(I, 2), w3 = (float)chunk_weight(I, 3);
-  constexpr float p = (float)mod_of(I), rp = 1.0f / p;
-  return sym_mod(fmaf(c[3], w3, fmaf(c[2], w2, fmaf(c[1], w1, c[0]))), p, rp);
+struct ModConst {
+  f32x2 w1, w2, w3, rp, minus_p;
+};
+constexpr ModConst mod_const(int i) {
+  return ModConst{both_of((float)chunk_weight(i, 1)), both_of((float)chunk_weight(i, 2)),
+                  both_of((float)chunk_weight(i, 3)), both_of(1.0f / (float)mod_of(i)), both_of(-(float)mod_of(i))};
+}
+struct ModTable {
+  ModConst m[kMods];
+};
+constexpr ModTable mod_table() {
+  ModTable t{};
+  for (int i = 0; i < kMods; ++i) t.m[i] = mod_const(i);
+  return t;
+}
+__constant__ ModTable kModTable = mod_table();
+
+__device__ __forceinline__ f32x2 residues(const f32x2 (&c)[4], const ModConst& m) {
+  return sym_mod2(fma2(c[3], m.w3, fma2(c[2], m.w2, fma2(c[1], m.w1, c[0]))), m.minus_p, m.rp);
 }
 
 // The residues of one (re, im) or (k, k + 1) pair of each of RW rows, modulus by modulus (rows side by side: their
-// chains overlap and share the plane's address; off: byte offset of a row's pair in a plane, 2 KiB planes and up
-// to 4 GiB, or ~0 for a row that is not stored).
-template <int SRC, int RW, int I>
-__device__ __forceinline__ void store_residues(const float (&cr)[RW][4], const float (&ci)[RW][4],
-                                               const unsigned (&off)[RW], char* plane, long long smod, unsigned row2) {
+// chains overlap and share the constants and the plane's address; off: byte offset of a row's pair in a plane, 2 KiB
+// planes and up to 4 GiB, or ~0 for a row that is not stored).
+// TABLE: the moduli's constants from constant memory, for the kernel that holds the next tile in registers beside four
+// rows (80 registers; as immediates 104, and 2 CTAs per SM: 22 880 x 520 in 225 us against 202); elsewhere as
+// immediates (5720 x 52 in 55 batches: 182 us, 226 from the table).
+template <int SRC, int RW, bool TABLE, int I>
+__device__ __forceinline__ void store_residues(const f32x2 (&c)[RW][4], const unsigned (&off)[RW], char* plane,
+                                               long long smod, unsigned row2) {
   if constexpr (I < kMods) {
+    constexpr ModConst imm = mod_const(I);
 #pragma unroll
     for (int i = 0; i < RW; ++i) {
-      const float re = residue<I>(cr[i]), im = residue<I>(ci[i]);
+      float re, im;
+      unpack2(TABLE ? residues(c[i], kModTable.m[I]) : residues(c[i], imm), re, im);
       if (off[i] != ~0u) {
         *reinterpret_cast<__nv_bfloat162*>(plane + off[i]) = __floats2bfloat162_rn(re, SRC == SRC_COMPLEX2 ? -im : im);
         if constexpr (SRC == SRC_COMPLEX2)
           *reinterpret_cast<__nv_bfloat162*>(plane + (off[i] + row2)) = __floats2bfloat162_rn(im, re);
       }
     }
-    store_residues<SRC, RW, I + 1>(cr, ci, off, plane + smod, smod, row2);
+    store_residues<SRC, RW, TABLE, I + 1>(c, off, plane + smod, smod, row2);
   }
 }
 
@@ -321,7 +363,7 @@ __global__ void __launch_bounds__(256) rns_convert_kernel(const ConvArgs a) {
     else return element(r, u);
   };
   // a thread's share of the transpose of the tile of 32 pairs from u on: the next tile's is loaded before the current
-  // one is converted (22 880 x 520: 286 us without, 224 with)
+  // one is converted (22 880 x 520: 286 us without, 224 with, both before the paired arithmetic)
   static_assert(RW * KL == 32, "a thread's share of a tile");
   double2 next[RW];
   auto fetch = [&](int u) {
@@ -338,7 +380,7 @@ __global__ void __launch_bounds__(256) rns_convert_kernel(const ConvArgs a) {
       if (u0 + 32 < upad) fetch(u0 + 32);
     }
     const int u = u0 + lane;
-    float cr[RW][4], ci[RW][4];
+    f32x2 c[RW][4];
     unsigned off[RW];
 #pragma unroll
     for (int i = 0; i < RW; ++i) {
@@ -351,11 +393,15 @@ __global__ void __launch_bounds__(256) rns_convert_kernel(const ConvArgs a) {
         ai = to_int(v.y, s);
         if (SRC != SRC_REAL && a.conj) ai = -ai;
       }
-      digits(ar, cr[i]);
-      digits(ai, ci[i]);
+      float cr[4], ci[4];
+      digits(ar, cr);
+      digits(ai, ci);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) c[i][j] = pack2(cr[j], ci[j]);
       off[i] = u < upad && r < a.rows ? (unsigned)((((long long)z * a.rows + r) * RR * a.Kp + 2 * u) * 2) : ~0u;
     }
-    store_residues<SRC, RW, 0>(cr, ci, off, reinterpret_cast<char*>(a.R), a.smod * 2, (unsigned)a.Kp * 2u);
+    store_residues<SRC, RW, rowfast && RW == 4, 0>(c, off, reinterpret_cast<char*>(a.R), a.smod * 2,
+                                                   (unsigned)a.Kp * 2u);
   }
 }
 
@@ -388,7 +434,8 @@ struct GemmArgs {
 // Y, the products' residues, lies in tiles of 32 rows x 16 columns, a row's 16 bytes after the other's: a warp of the
 // GEMM's epilogue stores, and one of the reconstruction loads, 512 contiguous bytes with a lane per row. (Row by row
 // the same accesses touched 32 lines each: 5720 x 208 x 52 in 55 batches took 523 us for the GEMM and 509 for the
-// reconstruction, 357 and 324 now.) Offset of the tile with row group rg and column c (a multiple of 16) of a batch entry of `rows` rows.
+// reconstruction, 357 and 324 so.) Offset of the tile with row group rg and column c (a multiple of 16) of a batch
+// entry of `rows` rows.
 __host__ __device__ inline long long y_tile(int z, int rows, int ldy, int rg, int c) {
   return (((long long)z * ((rows + 31) >> 5) + rg) * (ldy >> 4) + (c >> 4)) * 512;
 }
@@ -427,19 +474,21 @@ __device__ __forceinline__ Tile tile_of(const GemmArgs& g, int job, int rank) {
 }
 
 // 16 accumulator columns to bytes: v (+ the running residue) modulo p.
-__device__ __forceinline__ uint4 reduce16(const uint32_t (&v)[16], bool add, uint4 prev, float p, float rp) {
+__device__ __forceinline__ uint4 reduce16(const uint32_t (&v)[16], bool add, uint4 prev, f32x2 minus_p, f32x2 rp) {
   uint32_t w[4];
   const uint32_t pv[4] = {prev.x, prev.y, prev.z, prev.w};
 #pragma unroll
   for (int g = 0; g < 4; ++g) {
-    uint32_t b[4];
+    float b[4];
 #pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      float x = __uint_as_float(v[4 * g + c]);
-      if (add) x += (float)(int)(signed char)(pv[g] >> (8 * c));
-      b[c] = __float_as_uint(__fadd_rn(sym_mod(x, p, rp), kMagic));  // the low byte is the residue's
+    for (int c = 0; c < 4; c += 2) {
+      f32x2 x = pack2(__uint_as_float(v[4 * g + c]), __uint_as_float(v[4 * g + c + 1]));
+      if (add)
+        x = add2(x, pack2((float)(int)(signed char)(pv[g] >> (8 * c)), (float)(int)(signed char)(pv[g] >> (8 * c + 8))));
+      unpack2(add2(sym_mod2(x, minus_p, rp), kMagic2), b[c], b[c + 1]);  // the low byte is the residue's
     }
-    w[g] = __byte_perm(__byte_perm(b[0], b[1], 0x0040), __byte_perm(b[2], b[3], 0x0040), 0x5410);
+    w[g] = __byte_perm(__byte_perm(__float_as_uint(b[0]), __float_as_uint(b[1]), 0x0040),
+                       __byte_perm(__float_as_uint(b[2]), __float_as_uint(b[3]), 0x0040), 0x5410);
   }
   return make_uint4(w[0], w[1], w[2], w[3]);
 }
@@ -564,7 +613,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
     int gs = 0;
     for (int jb = job0; jb < njobs && ok; jb += njob) {
       const Tile t = tile_of<CL>(g, jb, rank);
-      const float p = kModF[t.mod], rp = 1.0f / p;
+      const float p = kModF[t.mod];
+      const f32x2 minus_p = pack2(-p, -p), rp = pack2(1.0f / p, 1.0f / p);
       const int row = t.m0 + quad * 32 + lane;
       signed char* y =
           g.Y + (long long)t.mod * g.ymod + y_tile(t.z, g.rows, g.ldy, t.m0 / 32 + quad, t.n0) + lane * 16;
@@ -593,7 +643,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
           uint32_t v[16];
           tmem_ld_32x32b_x16(tm + c, v);
           tmem_ld_wait();
-          const uint4 w = reduce16(v, k0 != 0, prev[i], p, rp);
+          const uint4 w = reduce16(v, k0 != 0, prev[i], minus_p, rp);
           if (rok) *reinterpret_cast<uint4*>(y + (half + 2 * i) * 512) = w;
         }
         tc_fence_before();
