@@ -229,7 +229,7 @@ DMET_API dmet_status_t dmet_emb_status(dmet_emb_plan_t plan, int32_t problem, do
  *   gamma    FP64 [n][n], symmetric, spin-summed, in the embedding basis;
  *   fock_out FP64 [n][n] (the real part of F0, whose imaginary part vanishes for real orbitals).
  * FP64 throughout; queued on the plan's stream; grows a plan-owned scratch buffer on first use
- * (about 16 Nk n_AO n + 16 Nk n^2 bytes). */
+ * (about 16 Nk n_AO n + 16 Nk n^2 + 300 n^2 bytes). */
 DMET_API dmet_status_t dmet_emb_fock(dmet_emb_plan_t plan, int32_t problem, const void* F, const void* C,
                                      const double* eri, const double* gamma, double* fock_out);
 
@@ -276,7 +276,9 @@ DMET_API dmet_status_t dmet_emb_bath(dmet_emb_plan_t plan, int32_t problem, int3
  *   gamma  complex128 [n][n], the embedding density;
  *   J, K   complex128 [n][n], written (real for real orbitals and a real gamma).
  * FP64 throughout (batched complex GEMMs over the (q, P) entries in chunks, and reductions); queued
- * on the plan's stream; grows a plan-owned scratch buffer of at most about 1 GiB on first use. */
+ * on the plan's stream; grows a plan-owned scratch buffer of at most about 1 GiB on first use; for
+ * larger n (integer products, as for DMET_PREC_FP64) of about 700 MiB beside 256 MiB or the 16 n_aux n^2
+ * bytes of one q, and where that much is not to be had the products run as FMAs. */
 DMET_API dmet_status_t dmet_emb_jk_df(dmet_emb_plan_t plan, int32_t problem, int32_t spin, const void* Lq,
                                       const void* gamma, void* J, void* K);
 
@@ -293,8 +295,8 @@ DMET_API dmet_status_t dmet_emb_jk_df(dmet_emb_plan_t plan, int32_t problem, int
  * dmet_emb_eri), then exp(-i q.r), the forward DFT over the grid, the Coulomb kernel 4 pi / |q + G|^2
  * (the plane waves and kernel of dmet_fftdf_plane_waves, 0 at q + G = 0), the inverse DFT,
  * exp(+i q.r), and (ij|kl) += Omega / (N_g Nk) sum_r w(r)_ij (r|0k 0l)^{-q} with the inverse DFT
- * normalised by 1/N_g (Omega the cell volume). The DFTs are dense per grid axis (batched complex
- * GEMMs). FP64 throughout; queued on the plan's stream; grows a plan-owned scratch buffer on first use
+ * normalised by 1/N_g (Omega the cell volume). The DFTs run axis by axis, as FFTs in registers where
+ * every axis has at most 32 points and no prime factor above 7 (else dense, as batched complex GEMMs). FP64 throughout; queued on the plan's stream; grows a plan-owned scratch buffer on first use
  * (2 N_g n^2 complex values). */
 DMET_API dmet_status_t dmet_emb_eri_fftdf(dmet_emb_plan_t plan, int32_t problem, const void* rho,
                                           const void* const* C, const int32_t* grid, const double* lattice,

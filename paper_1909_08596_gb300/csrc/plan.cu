@@ -2012,7 +2012,6 @@ dmet_status_t dmet_emb_plan(const dmet_emb_desc_t* descs, int32_t n_problems, vo
       alloc((void**)&W.X[s], &W.X_b[s], need.X[s]);
       alloc((void**)&W.lq_all[s], &W.lq_all_b[s], need.lq_all[s]);
     }
-    if (st == DMET_OK && rsz[i]) alloc(&W.rns, &W.rns_b, rsz[i]);
     alloc(&W.Ls, &W.Ls_b, mn.Ls);
     alloc(&W.Cc, &W.Cc_b, mn.Cc);
     alloc(&W.A2, &W.A2_b, mn.A2);
@@ -2029,6 +2028,9 @@ dmet_status_t dmet_emb_plan(const dmet_emb_desc_t* descs, int32_t n_problems, vo
       if (st == DMET_OK && W.Xt[s] && cudaMemset(W.Xt[s], 0, W.Xt_b[s]) != cudaSuccess)
         st = fail(DMET_ERR_CUDA, "memset");
   }
+  // (last, and a plan does without it rather than fail)
+  for (size_t i = 0; st == DMET_OK && i < P->ws.size(); ++i)
+    if (rsz[i] && ensure(&P->ws[i].rns, &P->ws[i].rns_b, rsz[i]) == DMET_ERR_OOM) clear_error();
   if (st == DMET_OK && concurrent) {
     const int nside = std::min(n_problems, 8);
     P->side.assign(nside, nullptr);
@@ -3054,7 +3056,11 @@ static dmet_status_t jk_residues(dmet_emb_plan_s* P, Prob& pr, int n, const doub
   c.scratch = (void*)16;  // (only tested for being there)
   c.bytes = rb;
   if (!rns_takes_zgemm(z1, c) || !rns_takes_zgemm(z2, c)) return DMET_OK;
-  TRY(ensure(&P->jk_ws, &P->jk_ws_b, oR + rb));
+  if (const dmet_status_t st = ensure(&P->jk_ws, &P->jk_ws_b, oR + rb); st != DMET_OK) {
+    if (st != DMET_ERR_OOM) return st;
+    clear_error();
+    return DMET_OK;  // (the FMA form asks for less)
+  }
   char* w = (char*)P->jk_ws;
   double2* W = (double2*)w;
   double2* part = (double2*)(w + oP);

@@ -1026,7 +1026,8 @@ size_t rns_need(const DsyrkArgs& a) {
 // FP64 kernel takes 0.27 us per k and 16 x 16 complex tile and SM (less where a tile has few rows); the residues
 // take 28 us for their four launches, 85 ns per k of a conversion that few CTAs share, 34 ps per complex
 // result (reconstruction and epilogue) and 12 ps per converted real element, and the MMAs. A 128 x 4096 product:
-// K = 8, 35 against 43 us; K = 16, 64 against 44; K = 64, 238 against 48.
+// K = 8, 35 against 43 us; K = 16, 64 against 44; K = 64, 238 against 48. (At large sizes a result
+// takes 20 ps and a converted element 9 since Y lies in tiles; the line, where the launches count, is where it was.)
 bool rns_takes_zgemm(const ZgemmArgs& a, const RnsCtx& c) {
   if (!c.scratch || a.lower || a.M <= 0 || a.N <= 0 || a.K <= 0 || a.batch <= 0) return false;
   const ZPlan p = zplan(a, A_KM, false, B_KN);
