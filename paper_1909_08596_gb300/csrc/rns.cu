@@ -424,7 +424,7 @@ struct GemmArgs {
   int tri, h0;              // tri: only tiles with a column <= the last row (square product, bn = 256); row 0 of
                             // this launch is row 256 h0 of the product
   int row0;                 // first row of the launch in the row operand
-  int jobs;                 // (clusters of tiles) per (modulus, batch)
+  int jobs;                 // tiles per (modulus, batch)
   int nkb, seg;             // K blocks, and how many of them between reductions (at most kSegStages)
   signed char* Y;           // [mod][batch] in tiles (y_tile)
   long long ymod;
@@ -444,12 +444,11 @@ struct Tile {
   int mod, z, m0, n0;
 };
 
-// Lower triangle: the row tiles 2 h and 2 h + 1 have h0 + h + 1 column tiles each; jobs take the pair together (CL = 2).
+// Lower triangle: the row tiles 2 h and 2 h + 1 have h0 + h + 1 column tiles each; pairs of jobs take them side by side.
 __host__ __device__ inline int tri_jobs_before(int h, int h0) { return h * h0 + h * (h + 1) / 2; }
 
-// Job `job` of a launch, for the CTA of rank `rank` of its cluster: CL neighbouring row tiles of one column tile.
-template <int CL>
-__device__ __forceinline__ Tile tile_of(const GemmArgs& g, int job, int rank) {
+// Job `job` of a launch.
+__device__ __forceinline__ Tile tile_of(const GemmArgs& g, int job) {
   Tile t;
   const int per = g.nbatch * g.jobs;
   t.mod = job / per;
@@ -457,18 +456,19 @@ __device__ __forceinline__ Tile tile_of(const GemmArgs& g, int job, int rank) {
   t.z = r / g.jobs;
   r -= t.z * g.jobs;
   int mt, nt;
-  if (CL == 2 && g.tri) {
+  if (g.tri) {
+    const int u = r >> 1;
     const float c = (float)(2 * g.h0 + 1);
-    int h = (int)((sqrtf(c * c + 8.f * (float)r) - c) * 0.5f);
-    while (h > 0 && tri_jobs_before(h, g.h0) > r) --h;
-    while (tri_jobs_before(h + 1, g.h0) <= r) ++h;
-    mt = h;
-    nt = r - tri_jobs_before(h, g.h0);
+    int h = (int)((sqrtf(c * c + 8.f * (float)u) - c) * 0.5f);
+    while (h > 0 && tri_jobs_before(h, g.h0) > u) --h;
+    while (tri_jobs_before(h + 1, g.h0) <= u) ++h;
+    mt = 2 * h + (r & 1);
+    nt = u - tri_jobs_before(h, g.h0);
   } else {
     mt = r / g.ct;
     nt = r - mt * g.ct;
   }
-  t.m0 = (mt * CL + rank) * kTileM;
+  t.m0 = mt * kTileM;
   t.n0 = nt * g.bn;
   return t;
 }
@@ -493,10 +493,9 @@ __device__ __forceinline__ uint4 reduce16(const uint32_t (&v)[16], bool add, uin
   return make_uint4(w[0], w[1], w[2], w[3]);
 }
 
-// Bound by the L2 reads of the operands (a 128 x 256 tile alone reads 48 KB per 512 clocks of MMA): with CL = 2 a
-// cluster's two CTAs take neighbouring row tiles, load half of the column tile each and multicast it to both, 32 KB
-// per CTA. A stage is free again when both CTAs' MMAs have read it.
-template <int CL>
+// Bound by the L2 reads of the operands: a 128 x 256 tile reads 48 KB per 512 clocks of MMA, and the L2 gives some
+// 10 TB/s in all. Every CTA loads its own tiles, without TMA multicast: the same code runs where several GPUs take part
+// (pairs of CTAs that shared the column tile by multicast: 17.39 ms for an h-BN-shaped call, 17.50 so).
 __global__ void __launch_bounds__(kGemmThreads, 1)
     rns_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const GemmArgs g,
                     int njobs, unsigned int* err, unsigned long long lim, int withhold) {
@@ -514,15 +513,12 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
   const uint32_t done_bar = smem_u32(bars + 2 * kStages + 4);
   auto a_tile = [&](int s) { return smem_u32(smem + s * kStageBytes); };
   auto b_tile = [&](int s) { return smem_u32(smem + s * kStageBytes + kABytes); };
-  const int rank = CL > 1 ? (int)cluster_rank() : 0;
-  const int job0 = (int)blockIdx.x / CL, njob = (int)gridDim.x / CL;
-  constexpr uint16_t kAll = (1u << CL) - 1u;
-  bool failed = false;
+  const int job0 = (int)blockIdx.x, njob = (int)gridDim.x;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages; ++s) {
       mbar_init(full(s), 1);
-      mbar_init(empty(s), CL);
+      mbar_init(empty(s), 1);
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(accf(b), 1);
@@ -538,7 +534,6 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
   }
   tc_fence_before();
   __syncthreads();
-  if (CL > 1) cluster_sync_all();  // every CTA's barriers are initialised
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
 
@@ -550,7 +545,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
       const uint32_t bytes = kABytes + (uint32_t)g.bn * 128u;
       bool ok = !withhold;
       for (int jb = job0; jb < njobs && ok; jb += njob) {
-        const Tile t = tile_of<CL>(g, jb, rank);
+        const Tile t = tile_of(g, jb);
         const int ra = t.z * g.rows + g.row0 + t.m0, rb = t.z * g.cols + t.n0;
         for (int kb = 0; kb < g.nkb; ++kb) {
           const int s = issued % kStages, ph = (issued / kStages) & 1;
@@ -560,17 +555,10 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
           }
           mbar_arrive_expect_tx(full(s), bytes);
           tma_load_3d(a_tile(s), &tmA, full(s), kb * kBK, ra, t.mod);
-          if constexpr (CL == 1) {
-            tma_load_3d(b_tile(s), &tmB, full(s), kb * kBK, rb, t.mod);
-          } else {
-            // this CTA's share of the column tile's rows (a multiple of 8: whole swizzle atoms), to both CTAs
-            const int share = g.bn / CL;
-            tma_load_3d_multicast(b_tile(s) + rank * share * 128, &tmB, full(s), kb * kBK, rb + rank * share, t.mod, kAll);
-          }
+          tma_load_3d(b_tile(s), &tmB, full(s), kb * kBK, rb, t.mod);
           ++issued;
         }
       }
-      failed = !ok;
     }
   } else if (warp == 1) {
     if (lane == 0) {
@@ -596,8 +584,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
             for (int kk = 0; kk < 4; ++kk)
               umma<0>(tmem + b * 256, smem_desc<128>(a_tile(s) + kk * 32), smem_desc<128>(b_tile(s) + kk * 32), idesc,
                       (kb > k0 || kk) ? 1u : 0u);
-            if constexpr (CL == 1) umma_commit(empty(s));
-            else umma_commit_multicast(empty(s), kAll);
+            umma_commit(empty(s));
             ++it;
             *consumed = it;
           }
@@ -605,14 +592,14 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
         }
       }
       umma_commit(done_bar);
-      failed = !mbar_wait(done_bar, 0, err, 16u, lim) || !ok;
+      mbar_wait(done_bar, 0, err, 16u, lim);
     }
   } else if (warp >= 4) {
     const int quad = warp & 3, half = (warp - 4) >> 2;
     bool ok = true;
     int gs = 0;
     for (int jb = job0; jb < njobs && ok; jb += njob) {
-      const Tile t = tile_of<CL>(g, jb, rank);
+      const Tile t = tile_of(g, jb);
       const float p = kModF[t.mod];
       const f32x2 minus_p = pack2(-p, -p), rp = pack2(1.0f / p, 1.0f / p);
       const int row = t.m0 + quad * 32 + lane;
@@ -656,12 +643,6 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
   if (warp == 0 && lane == 0) {
     // copies issued but never consumed (only after an expired wait) must land before exit
     for (int i = *consumed; i < issued; ++i) mbar_wait(full(i % kStages), (i / kStages) & 1, err, 32u, lim);
-  }
-  if (CL > 1) {
-    // After an expired wait the peer's copies into this CTA may still be in flight: give them a millisecond to land.
-    if (__syncthreads_or(failed))
-      for (int i = 0; i < 1000; ++i) __nanosleep(1000);
-    cluster_sync_all();  // no CTA leaves while the other's copies and commits can still reach it
   }
   __syncthreads();
   if (warp == 1) {
@@ -920,57 +901,22 @@ int tile_width(int cols) {
   return (int)pad_to((cols + ct - 1) / ct, 16);
 }
 
-// Row tiles in pairs where the operands' reads bound the GEMM and pairing wastes little: not for a lone row tile nor
-// an odd few, and not for a K of a few blocks, which the epilogue bounds (5720 x 208 x 52 in 36 batches: 266 us
-// alone, 299 in pairs; 5460^2 x 3264, lower triangle: 1.28 PFLOP/s in pairs; the L2 gives some 10 TB/s).
-int cluster_of(int rt, bool tri, int nkb) {
-  return tri || (nkb > 4 && (rt >= 8 || (rt >= 2 && rt % 2 == 0))) ? 2 : 1;
-}
-
-template <int CL>
-cudaError_t launch_gemm(const CUtensorMap& ma, const CUtensorMap& mb, const GemmArgs& g, int njobs, const RnsCtx& c,
-                        cudaStream_t s) {
-  auto kernel = rns_gemm_kernel<CL>;
-  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kGemmSmem);
-  if (e != cudaSuccess) return e;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)CL);
-  cfg.blockDim = dim3(kGemmThreads);
-  cfg.dynamicSmemBytes = kGemmSmem;
-  cfg.stream = s;
-  cudaLaunchAttribute at[1];
-  if (CL > 1) {
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = CL;
-    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-  }
-  // as many clusters as run at once (the jobs are dealt out statically)
-  int fit = c.sms / CL;
-  if (CL > 1) {
-    e = cudaOccupancyMaxActiveClusters(&fit, kernel, &cfg);
-    if (e != cudaSuccess) return e;
-    fit = std::max(1, std::min(fit, c.sms / CL));
-  }
-  cfg.gridDim = dim3((unsigned)(std::min(njobs, fit) * CL));
-  return cudaLaunchKernelEx(&cfg, kernel, ma, mb, g, njobs, c.err, c.wait_ns, c.withhold_loads);
-}
-
 cudaError_t gemm(const __nv_bfloat16* RA, long long smodA, const __nv_bfloat16* RB, long long smodB, GemmArgs g, int Kp,
                  int total_rows_a, const RnsCtx& c, cudaStream_t s) {
   CUtensorMap ma, mb;
   cudaError_t e = make_tmap_rows128(&ma, RA, Kp, (unsigned long long)g.nbatch * total_rows_a, kMods, smodA, kTileM);
   if (e != cudaSuccess) return e;
-  const int cl = cluster_of(g.rt, g.tri, g.nkb);
-  const int pairs = (g.rt + cl - 1) / cl;
-  g.jobs = g.tri ? tri_jobs_before(pairs, g.h0) : pairs * g.ct;
-  e = make_tmap_rows128(&mb, RB, Kp, (unsigned long long)g.nbatch * g.cols, kMods, smodB, g.bn / cl);
+  g.jobs = g.tri ? 2 * tri_jobs_before((g.rt + 1) / 2, g.h0) : g.rt * g.ct;
+  e = make_tmap_rows128(&mb, RB, Kp, (unsigned long long)g.nbatch * g.cols, kMods, smodB, g.bn);
   if (e != cudaSuccess) return e;
   const int segs = (g.nkb + kSegStages - 1) / kSegStages;
   g.seg = (g.nkb + segs - 1) / segs;
   const int njobs = kMods * g.nbatch * g.jobs;
-  return cl == 2 ? launch_gemm<2>(ma, mb, g, njobs, c, s) : launch_gemm<1>(ma, mb, g, njobs, c, s);
+  e = cudaFuncSetAttribute(rns_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kGemmSmem);
+  if (e != cudaSuccess) return e;
+  rns_gemm_kernel<<<std::min(njobs, c.sms), kGemmThreads, kGemmSmem, s>>>(ma, mb, g, njobs, c.err, c.wait_ns,
+                                                                         c.withhold_loads);
+  return cudaGetLastError();
 }
 
 // Splits the context's scratch; every piece starts on a 1024-byte boundary.
