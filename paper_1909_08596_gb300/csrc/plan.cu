@@ -321,7 +321,7 @@ struct dmet_emb_plan_s {
   std::vector<cudaEvent_t> join;
   Workspace* W = nullptr;          // workspace of the problem being enqueued
   cudaStream_t cs = nullptr;       // stream of the problem being enqueued
-  cudaStream_t chk = nullptr;      // the orbital checks' stream (fork_checks)
+  cudaStream_t chk = nullptr;      // the orbital checks' stream (Checks)
   cudaEvent_t chk_fork = nullptr, chk_join = nullptr;
   double* dstats = nullptr;        // [n_problems][8]
   unsigned int* derr = nullptr;
@@ -690,26 +690,46 @@ dmet_status_t run_orbital_checks(dmet_emb_plan_s* P, Prob& pr, int p, const doub
 
 // The orbital checks read only C and write only the problem's statistics, so they run beside the transforms on a
 // stream of their own (135 us of an h-BN-shaped call, on the FP64 pipe, under operand splitting that is bound by
-// memory): forked from the problem's stream here, joined back by join_checks before the call's work ends. Problems
-// on side streams of their own keep them there: they already overlap, and one stream for the checks of a batch is
-// slower (24 problems in grouped launches: 5.49 against 5.32 ms).
-dmet_status_t fork_checks(dmet_emb_plan_s* P, Prob& pr, int p, const double2* const* C, bool beside) {
-  if (!beside) return run_orbital_checks(P, pr, p, C);
-  CK(cudaEventRecord(P->chk_fork, P->cs));
-  CK(cudaStreamWaitEvent(P->chk, P->chk_fork, 0));
-  const cudaStream_t cs = P->cs;
-  P->cs = P->chk;
-  const dmet_status_t st = run_orbital_checks(P, pr, p, C);
-  P->cs = cs;
-  // (recorded on a failure too: a captured fork has to be joined)
-  CK(cudaEventRecord(P->chk_join, P->chk));
-  return st;
-}
+// memory): forked from the problem's stream by fork, joined back by join or, on every return before it, by the
+// destructor, so that what the caller queues next (another call's statistics, a change of C, the end of a capture)
+// follows them. Problems on side streams of their own keep them there: they already overlap, and one stream for the
+// checks of a batch is slower (24 problems in grouped launches: 5.49 against 5.32 ms).
+class Checks {
+ public:
+  explicit Checks(dmet_emb_plan_s* P) : P_(P) {}
+  ~Checks() {
+    if (forked_) cudaStreamWaitEvent(into_, P_->chk_join, 0);
+  }
+  Checks(const Checks&) = delete;
+  Checks& operator=(const Checks&) = delete;
 
-dmet_status_t join_checks(dmet_emb_plan_s* P, cudaStream_t s) {
-  CK(cudaStreamWaitEvent(s, P->chk_join, 0));
-  return DMET_OK;
-}
+  dmet_status_t fork(Prob& pr, int p, const double2* const* C, bool beside) {
+    if (!beside) return run_orbital_checks(P_, pr, p, C);
+    const cudaStream_t cs = P_->cs;
+    CK(cudaEventRecord(P_->chk_fork, cs));
+    CK(cudaStreamWaitEvent(P_->chk, P_->chk_fork, 0));
+    P_->cs = P_->chk;
+    const dmet_status_t st = run_orbital_checks(P_, pr, p, C);
+    P_->cs = cs;
+    // (on a failure too: a part of the checks may be queued, and a captured fork has to be joined)
+    CK(cudaEventRecord(P_->chk_join, P_->chk));
+    into_ = cs;
+    forked_ = true;
+    return st;
+  }
+
+  dmet_status_t join() {
+    if (!forked_) return DMET_OK;
+    forked_ = false;
+    CK(cudaStreamWaitEvent(into_, P_->chk_join, 0));
+    return DMET_OK;
+  }
+
+ private:
+  dmet_emb_plan_s* P_;
+  cudaStream_t into_ = nullptr;
+  bool forked_ = false;
+};
 
 dmet_status_t run_l_check(dmet_emb_plan_s* P, Prob& pr, int p, const double2* L) {
   if (pr.d.sym != DMET_SYM_REAL || !pr.d.check_l) return DMET_OK;
@@ -2191,7 +2211,8 @@ dmet_status_t dmet_emb_transform_3idx(dmet_emb_plan_t P, int32_t problem, const 
   const double2* Cd[2] = {nullptr, nullptr};
   TRY(stage_inputs(P, pr, L, C, &Ld, Cd));
   CK(cudaMemsetAsync(P->dstats + 8 * problem, 0, 8 * sizeof(double), P->cs));
-  TRY(fork_checks(P, pr, problem, Cd, true));
+  Checks checks(P);
+  TRY(checks.fork(pr, problem, Cd, true));
   TRY(run_l_check(P, pr, problem, Ld));
   double2* out[2] = {nullptr, nullptr};
   size_t ob[2] = {0, 0}, need = 0;
@@ -2230,7 +2251,7 @@ dmet_status_t dmet_emb_transform_3idx(dmet_emb_plan_t P, int32_t problem, const 
   } else {
     TRY(transform_range(P, pr, Ld, Cd, q_begin, q_end, out, pr.bq));
   }
-  TRY(join_checks(P, P->cs));
+  TRY(checks.join());
   if (need) {
     for (int s = 0; s < pr.nspin; ++s)
       if (ohost[s]) {
@@ -2257,8 +2278,8 @@ static dmet_status_t enqueue_problem(dmet_emb_plan_s* P, int p, const void* L, c
   const double2* Cd[2] = {nullptr, nullptr};
   TRY(stage_inputs(P, pr, L, C, &Ld, Cd, /*subset=*/true));
   CK(cudaMemsetAsync(P->dstats + 8 * p, 0, 8 * sizeof(double), P->cs));
-  const bool beside = P->side.empty();
-  TRY(fork_checks(P, pr, p, Cd, beside));
+  Checks checks(P);
+  TRY(checks.fork(pr, p, Cd, P->side.empty()));
   TRY(run_l_check(P, pr, p, Ld));
   const int nblk = pr.nspin == 1 ? 1 : 3;
   void* out[3] = {nullptr, nullptr, nullptr};
@@ -2285,8 +2306,8 @@ static dmet_status_t enqueue_problem(dmet_emb_plan_s* P, int p, const void* L, c
   else if (pr.pack == DMET_PACK_S8) st = eri_s8(P, pr, Ld, Cd, out);
   else st = eri_full(P, pr, Ld, Cd, out);
   P->xpending = false;
-  if (beside) TRY(join_checks(P, P->cs));
   TRY(st);
+  TRY(checks.join());
   if (need) {
     for (int b = 0; b < nblk; ++b)
       if (ohost[b]) {
@@ -3345,7 +3366,8 @@ dmet_status_t dmet_emb_eri_fftdf(dmet_emb_plan_t P, int32_t problem, const void*
   const double2* Cd[2] = {(const double2*)C[0], pr.nspin == 2 ? (const double2*)C[1] : nullptr};
   P->W = &P->ws[P->ws_of[problem]];
   CK(cudaMemsetAsync(P->dstats + 8 * problem, 0, 8 * sizeof(double), P->cs));
-  TRY(fork_checks(P, pr, problem, Cd, true));
+  Checks checks(P);
+  TRY(checks.fork(pr, problem, Cd, true));
   double2* lq[2] = {P->W->lq_all[0], P->W->lq_all[1]};
   TRY(transform_range(P, pr, (const double2*)rho, Cd, 0, nk, lq, pr.bq));
   for (int b = 0; b < nblk; ++b) CK(cudaMemsetAsync(eri_out[b], 0, eri_bytes_of(pr.d, b), P->cs));
@@ -3412,7 +3434,7 @@ dmet_status_t dmet_emb_eri_fftdf(dmet_emb_plan_t P, int32_t problem, const void*
       }
     }
   }
-  TRY(join_checks(P, P->cs));
+  TRY(checks.join());
   CK(cudaGetLastError());
   return DMET_OK;
 }
