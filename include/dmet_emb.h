@@ -80,7 +80,10 @@ typedef enum {
   DMET_PREC_FP64 = 0,    /* FP64 inputs, results and intermediates. Small products run as IEEE FP64
                             FMAs; larger ones round each operand row once to 58-bit integers
                             (relative to the row's 2-norm), multiply those exactly and round each
-                            result to FP64, which is no less accurate than the chain of FMAs. An
+                            result to FP64. Results that this would leave less accurate than FMAs,
+                            those whose sum of magnitudes sum |a| |b| is small beside the rows'
+                            norms (graded or localised operands), are formed as FMAs, so that
+                            every result is within the error bound of the chain of FMAs. An
                             infinity or NaN in an operand row gives NaN in every result of that
                             row there. Products whose scratch the workspace limit does not leave
                             run as FMAs. */

@@ -11,17 +11,27 @@
 // GEMM of symmetric residues (bf16, |r| <= 128) per modulus, and the product recovered modulo
 // P = prod p_i > 2 * 2^(2 kBeta). The only errors are the rounding of the operands to integers, half
 // a unit of 2^-kBeta of the row's norm (5 bits below the FP64 rounding of an element of the row's
-// size), and one rounding of the result, so it is closer to the exact product than a chain of FP64
-// FMAs, whose error grows with sqrt(K).
+// size), and one rounding of the result: some 2^-59 |a| |b| of the rows' norms, whatever K.
 //
-//   1. rns_convert_kernel: per operand row, the scale from its norm; then residues [mod][batch][row][K],
-//      K-major (complex operands as interleaved (re, im) pairs along K; the column operand of a
-//      complex product as two rows, (re, -im) for the real and (im, re) for the imaginary part).
-//   2. rns_gemm_kernel: tcgen05 (128 x up to 256 tiles, TMA-fed), one job per (modulus, batch, tile).
+// That is below the rounding of a chain of FP64 FMAs, about 2^-54 S with S = sum_k |A(m, k)| |B(n, k)|, while S is at
+// least 2^-5 of the norms' bounds, as it is for operands whose large elements meet (S is 0.6 |a| |b| for random ones).
+// Rows that are graded over many decades can have results far below their norms, which FMAs get right and a grid
+// relative to the norm does not. So the engine forms S as well, in one more product: the magnitudes as bf16, rounded
+// down, go through the GEMM as a plane beside the residues, and the reconstruction replaces every result with too small
+// an S by the chain of FMAs over the original operands (fma_results). Where S is zero the result is, exactly.
+// Measured against quads, two half transforms of K = 48, worst element and rms in units of 2^-53 S: random operands
+// 0.16 and 0.025 (FMAs 0.78 and 0.12), elements spread over two decades 1.0 and 0.09 (3.4 and 0.39), four 3.9 and 0.28
+// (7.9 and 0.85), eight 8.6 and 0.82 (9.3 and 1.4). The plane costs 8% of an h-BN-shaped call (17.5 -> 18.95 ms); the
+// same with operands graded over 4 / 8 / 40 decades takes 30 / 149 / 262 ms (some 390 on the FP64 pipe alone).
+//
+//   1. rns_convert_kernel: per operand row, the scale from its norm; then residues [plane][batch][row][K], the
+//      magnitudes as the last plane, K-major (complex operands as interleaved (re, im) pairs along K; the column
+//      operand of a complex product as two rows, (re, -im) for the real and (im, re) for the imaginary part).
+//   2. rns_gemm_kernel: tcgen05 (128 x up to 256 tiles, TMA-fed), one job per (plane, batch, tile).
 //      After every kSegStages K blocks the FP32 sums, exact below 2^24, are reduced modulo p and the
-//      running residue is kept as one byte per element in Y [mod][batch][row][col].
+//      running residue is kept as one byte per element in Y [plane][batch][row][col] (of S: see count16).
 //   3. rns_crt_kernel: recovers the signed 117-bit integer as a 64-bit fraction of P, rounds it to FP64, undoes the
-//      scales and writes the caller's layout.
+//      scales, takes the results with a small S from FMAs and writes the caller's layout.
 //
 // A row with an infinity or a NaN gives NaN in every result it enters.
 
@@ -44,6 +54,7 @@ namespace {
 using namespace tc;
 
 constexpr int kMods = 15;
+constexpr int kPlanes = kMods + 1;  // the residues, then the magnitudes
 constexpr int kBeta = 58;
 __host__ __device__ constexpr int mod_of(int i) {
   constexpr int p[kMods] = {256, 253, 251, 247, 241, 239, 233, 229, 227, 223, 217, 211, 199, 197, 193};
@@ -156,8 +167,8 @@ struct ConvArgs {
   long long s_row, s_k;   // strides of a row and of a k index, in elements
   int rows, K, Kp;        // Kp: real K, padded to the GEMM's K block
   int conj;
-  __nv_bfloat16* R;       // [mod][batch][rows (x 2 for SRC_COMPLEX2)][Kp]
-  long long smod;         // elements per modulus plane
+  __nv_bfloat16* R;       // [plane][batch][rows (x 2 for SRC_COMPLEX2)][Kp]
+  long long smod;         // elements per plane
   int* exps;              // [batch][rows]
 };
 
@@ -219,6 +230,16 @@ __device__ __forceinline__ long long to_int(double x, int s) {
   const int r = min(max(1081 - s - (e ? e : 1), 0), 63);
   const long long t = (long long)((m + ((1ull << r) >> 1)) >> r);
   return (int)hi < 0 ? -t : t;
+}
+
+// |x| 2^(s - kBeta), at most 1, as a bf16 rounded down; what is below 2^-62 (or subnormal, whose exponent says less)
+// counts as that, so that products of two are normal in FP32 and only a zero gives a zero.
+constexpr int kMagMin = -62;
+__device__ __forceinline__ unsigned magnitude(double x, int s) {
+  const unsigned hi = (unsigned)__double2hiint(x) & 0x7fffffffu;
+  const int e = (int)(hi >> 20), E = e ? e - 1023 + s - kBeta : kMagMin - 1;
+  const unsigned b = E < kMagMin ? (unsigned)(kMagMin + 127) << 7 : ((unsigned)(E + 127) << 7) | ((hi >> 13) & 0x7fu);
+  return (hi | (unsigned)__double2loint(x)) ? b : 0u;
 }
 
 // Four signed 16-bit digits of a, as floats: a = sum c_j 2^(16 j).
@@ -399,6 +420,12 @@ __global__ void __launch_bounds__(256) rns_convert_kernel(const ConvArgs a) {
 #pragma unroll
       for (int j = 0; j < 4; ++j) c[i][j] = pack2(cr[j], ci[j]);
       off[i] = u < upad && r < a.rows ? (unsigned)((((long long)z * a.rows + r) * RR * a.Kp + 2 * u) * 2) : ~0u;
+      if (off[i] != ~0u) {
+        const unsigned mx = magnitude(v.x, s), my = magnitude(v.y, s);
+        char* at = reinterpret_cast<char*>(a.R) + (long long)kMods * a.smod * 2 + off[i];
+        *reinterpret_cast<unsigned*>(at) = mx | (my << 16);
+        if constexpr (SRC == SRC_COMPLEX2) *reinterpret_cast<unsigned*>(at + (unsigned)a.Kp * 2u) = my | (mx << 16);
+      }
     }
     store_residues<SRC, RW, rowfast && RW == 4, 0>(c, off, reinterpret_cast<char*>(a.R), a.smod * 2,
                                                    (unsigned)a.Kp * 2u);
@@ -424,9 +451,9 @@ struct GemmArgs {
   int tri, h0;              // tri: only tiles with a column <= the last row (square product, bn = 256); row 0 of
                             // this launch is row 256 h0 of the product
   int row0;                 // first row of the launch in the row operand
-  int jobs;                 // tiles per (modulus, batch)
+  int jobs;                 // tiles per (plane, batch)
   int nkb, seg;             // K blocks, and how many of them between reductions (at most kSegStages)
-  signed char* Y;           // [mod][batch] in tiles (y_tile)
+  signed char* Y;           // [plane][batch] in tiles (y_tile)
   long long ymod;
   int ldy;
 };
@@ -489,6 +516,24 @@ __device__ __forceinline__ uint4 reduce16(const uint32_t (&v)[16], bool add, uin
     }
     w[g] = __byte_perm(__byte_perm(__float_as_uint(b[0]), __float_as_uint(b[1]), 0x0040),
                        __byte_perm(__float_as_uint(b[2]), __float_as_uint(b[3]), 0x0040), 0x5410);
+  }
+  return make_uint4(w[0], w[1], w[2], w[3]);
+}
+
+// 16 sums of magnitudes to bytes: 2 floor(128 S) (a segment's share rounded down, at most 254) + (S != 0).
+__device__ __forceinline__ uint4 count16(const uint32_t (&v)[16], bool add, uint4 prev) {
+  uint32_t w[4];
+  const uint32_t pv[4] = {prev.x, prev.y, prev.z, prev.w};
+#pragma unroll
+  for (int g = 0; g < 4; ++g) {
+    w[g] = 0;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      const float f = __uint_as_float(v[4 * g + c]);
+      const unsigned old = add ? (pv[g] >> (8 * c)) & 255u : 0u;
+      const unsigned n = min((unsigned)(f * 128.f) + (old >> 1), 127u);
+      w[g] |= (n << 1 | (f > 0.f ? 1u : 0u) | (old & 1u)) << (8 * c);
+    }
   }
   return make_uint4(w[0], w[1], w[2], w[3]);
 }
@@ -600,7 +645,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
     int gs = 0;
     for (int jb = job0; jb < njobs && ok; jb += njob) {
       const Tile t = tile_of(g, jb);
-      const float p = kModF[t.mod];
+      const bool mags = t.mod == kMods;
+      const float p = kModF[mags ? 0 : t.mod];
       const f32x2 minus_p = pack2(-p, -p), rp = pack2(1.0f / p, 1.0f / p);
       const int row = t.m0 + quad * 32 + lane;
       signed char* y =
@@ -630,7 +676,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
           uint32_t v[16];
           tmem_ld_32x32b_x16(tm + c, v);
           tmem_ld_wait();
-          const uint4 w = reduce16(v, k0 != 0, prev[i], minus_p, rp);
+          const uint4 w = mags ? count16(v, k0 != 0, prev[i]) : reduce16(v, k0 != 0, prev[i], minus_p, rp);
           if (rok) *reinterpret_cast<uint4*>(y + (half + 2 * i) * 512) = w;
         }
         tc_fence_before();
@@ -652,6 +698,13 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
 }
 
 // ---------------- reconstruction ----------------
+
+// An operand of the product, for the results that are taken from FMAs.
+struct FmaSide {
+  const double* src;           // the launch's first row
+  long long sbatch, s_row, s_k;
+  int sel, conj;               // as in ConvArgs
+};
 
 struct CrtArgs {
   const signed char* Y;
@@ -675,6 +728,8 @@ struct CrtArgs {
   double alpha;
   int scaled;               // alpha != 1 (tested as an integer: the FP64 pipe is slow)
   int beta;
+  FmaSide rside, cside;
+  int rows_are_m, K;
 };
 
 struct Frac {
@@ -783,14 +838,101 @@ __device__ __forceinline__ void store_complex(const CrtArgs& a, double2* D, cons
   __syncwarp();
 }
 
+// Results whose S is below kMinCount / 128 of the norms' bounds come from FMAs: the residues' error, about 2^-59 of
+// those bounds, is then above the 2^-54 S of a chain.
+constexpr unsigned kMinCount = 4;
+
+// Bit 4 h + i (real: element i of the word) or 2 h + i (complex: pair i, by the larger modulus bound S_re + S_im) of
+// the result for results with a small S. w: four bytes of count16.
+template <bool CPLX>
+__device__ __forceinline__ unsigned small_sums(unsigned w) {
+  const unsigned n = (w >> 1) & 0x7f7f7f7fu;
+  if constexpr (CPLX) {
+    constexpr unsigned add = 0x8000u - 2 * kMinCount;
+    const unsigned sum = (n & 0x00ff00ffu) + ((n >> 8) & 0x00ff00ffu), any = (w | w >> 8) & 0x00010001u;
+    const unsigned ok = (sum + (add << 16 | add)) | ((any ^ 0x00010001u) << 15);
+    return ((~ok >> 15) & 1u) | ((~ok >> 30) & 2u);
+  } else {
+    const unsigned ok = (n + 0x01010101u * (0x80u - kMinCount)) | ((~w & 0x01010101u) << 7), bad = ~ok & 0x80808080u;
+    return ((bad >> 7) & 1u) | ((bad >> 14) & 2u) | ((bad >> 21) & 4u) | ((bad >> 28) & 8u);
+  }
+}
+
+// The results of a warp's 32 x 16 (8 complex) that `flags` marks, a bit per column and lane (row), as the FP64 kernels
+// form them: listed in order of columns, a lane per result.
+template <bool CPLX>
+__device__ __noinline__ void fma_results(const CrtArgs& a, double* st, unsigned short* list, unsigned flags, int c0,
+                                         int rbase, int z) {
+  const int lane = threadIdx.x & 31, cbase = CPLX ? c0 >> 1 : c0;
+  int n = 0;
+#pragma unroll 1
+  for (int c = 0; c < (CPLX ? 8 : 16); ++c) {
+    const bool f = (flags >> c & 1u) && rbase + lane < a.rows && (cbase + c) * (CPLX ? 2 : 1) < a.cols &&
+                   !(a.tri && cbase + c > a.row0 + rbase + lane);
+    const unsigned b = __ballot_sync(0xffffffffu, f);
+    if (f) list[n + __popc(b & ((1u << lane) - 1u))] = (unsigned short)(c << 5 | lane);
+    n += __popc(b);
+  }
+  __syncwarp();
+  long long zr = z, zc = z;
+  int K = a.K;
+  if (CPLX && a.tab) {
+    const int4 t = a.tab[a.tab0 + z];
+    zr = a.rside.sel ? t.y : t.x;
+    zc = a.cside.sel ? t.y : t.x;
+    K = t.w;
+  }
+#pragma unroll 1
+  for (int t = lane; t < n; t += 32) {
+    const int r = list[t] & 31, c = list[t] >> 5;
+    const long long ro = zr * a.rside.sbatch + (rbase + r) * a.rside.s_row;
+    const long long co = zc * a.cside.sbatch + (cbase + c) * a.cside.s_row;
+    if constexpr (CPLX) {
+      const double2* p = reinterpret_cast<const double2*>(a.rside.src) + ro;
+      const double2* q = reinterpret_cast<const double2*>(a.cside.src) + co;
+      long long ps = a.rside.s_k, qs = a.cside.s_k;
+      if (!a.rows_are_m) {
+        const double2* x = p;
+        p = q;
+        q = x;
+        ps = a.cside.s_k;
+        qs = a.rside.s_k;
+      }
+      const bool cj = a.rside.conj | a.cside.conj;  // (of the m operand)
+      double re = 0.0, im = 0.0;
+#pragma unroll 4
+      for (int k = 0; k < K; ++k) {
+        double2 u = p[k * ps];
+        const double2 v = q[k * qs];
+        if (cj) u.y = -u.y;
+        re = fma(u.x, v.x, re);
+        im = fma(u.x, v.y, im);
+        re = fma(-u.y, v.y, re);
+        im = fma(u.y, v.x, im);
+      }
+      st[r * 17 + 2 * c] = re;
+      st[r * 17 + 2 * c + 1] = im;
+    } else {
+      const double* p = a.rside.src + ro;
+      const double* q = a.cside.src + co;
+      double v = 0.0;
+#pragma unroll 4
+      for (int k = 0; k < K; ++k) v = fma(p[k * a.rside.s_k], q[k * a.cside.s_k], v);
+      st[r * 17 + c] = v;
+    }
+  }
+  __syncwarp();
+}
+
 // A warp takes 32 rows x 16 columns, a lane per row, 8 columns at a time (15 planes of 8 bytes in registers, so
 // that four CTAs fit an SM). Bound by issue (157 instructions per value, 45 of them the multiply-adds of the
 // fractions): 65.4 M values in 324 us. The same with the whole integer in 64-bit multiply-adds on
 // 30-bit limbs and 16 columns a time took 238 instructions at half the occupancy, twice the time.
 template <bool CPLX>
-__global__ void __launch_bounds__(256, 4) rns_crt_kernel(const CrtArgs a) {
+__global__ void __launch_bounds__(256, 4) rns_crt_kernel(const __grid_constant__ CrtArgs a) {
   __shared__ double stage[8][32 * 17];
   __shared__ long long radrs[CPLX ? 8 : 1][32];
+  __shared__ unsigned short list[8][CPLX ? 256 : 512];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int z = blockIdx.y;
   const long long item = (long long)blockIdx.x * 8 + warp;
@@ -804,6 +946,7 @@ __global__ void __launch_bounds__(256, 4) rns_crt_kernel(const CrtArgs a) {
   const int sa = rok ? a.ea[(long long)z * a.ea_rows + row] : 0;
   const int* ebp = a.eb + (long long)z * a.eb_rows;
   double* st = stage[warp];
+  unsigned flags = 0;
 #pragma unroll 1
   for (int h = 0; h < 2; ++h) {
     if (c0 + 8 * h >= a.cols) break;
@@ -814,6 +957,9 @@ __global__ void __launch_bounds__(256, 4) rns_crt_kernel(const CrtArgs a) {
       y[i].x ^= 0x80808080u;
       y[i].y ^= 0x80808080u;
     }
+    const uint2 m = *reinterpret_cast<const uint2*>(yp + (long long)kMods * a.ymod + 8 * h);
+    flags |= CPLX ? (small_sums<CPLX>(m.x) | small_sums<CPLX>(m.y) << 2) << (4 * h)
+                  : (small_sums<CPLX>(m.x) | small_sums<CPLX>(m.y) << 4) << (8 * h);
 #pragma unroll
     for (int c = 0; c < 8; ++c) {
       Frac f = frac_start();
@@ -823,6 +969,7 @@ __global__ void __launch_bounds__(256, 4) rns_crt_kernel(const CrtArgs a) {
     }
   }
   __syncwarp();
+  if (__any_sync(0xffffffffu, flags != 0)) fma_results<CPLX>(a, st, list[warp], flags, c0, rbase, z);
   if constexpr (CPLX) {
     double2* D = a.D + (a.tab ? (long long)a.tab[a.tab0 + z].z : (long long)z) * a.sD;
     store_complex(a, D, st, radrs[warp], c0, rbase, lane);
@@ -857,12 +1004,17 @@ struct Side {
   int rows, conj;
 };
 
+// `o` from row r0 on, for the chunk of batch entries from batch0 on.
+FmaSide fma_side(const Side& o, int r0, const int4* tab, long long batch0) {
+  const int w = o.src == SRC_REAL ? 1 : 2;
+  return {o.base + (long long)w * (r0 * o.s_row + (tab ? 0 : batch0 * o.sbatch)), o.sbatch, o.s_row, o.s_k, o.sel, o.conj};
+}
+
 cudaError_t convert(const Side& o, int r0, int nrows, const int4* tab, int tab0, int K, int Kp, int nb,
                     long long batch0, __nv_bfloat16* R, long long smod, int* exps, int sms, cudaStream_t s) {
   ConvArgs a;
   std::memset(&a, 0, sizeof(a));
-  const int w = o.src == SRC_REAL ? 1 : 2;
-  a.src = o.base + (long long)w * (r0 * o.s_row + (tab ? 0 : batch0 * o.sbatch));
+  a.src = fma_side(o, r0, tab, batch0).src;
   a.tab = tab;
   a.tab0 = tab0;
   a.sel = o.sel;
@@ -904,14 +1056,14 @@ int tile_width(int cols) {
 cudaError_t gemm(const __nv_bfloat16* RA, long long smodA, const __nv_bfloat16* RB, long long smodB, GemmArgs g, int Kp,
                  int total_rows_a, const RnsCtx& c, cudaStream_t s) {
   CUtensorMap ma, mb;
-  cudaError_t e = make_tmap_rows128(&ma, RA, Kp, (unsigned long long)g.nbatch * total_rows_a, kMods, smodA, kTileM);
+  cudaError_t e = make_tmap_rows128(&ma, RA, Kp, (unsigned long long)g.nbatch * total_rows_a, kPlanes, smodA, kTileM);
   if (e != cudaSuccess) return e;
   g.jobs = g.tri ? 2 * tri_jobs_before((g.rt + 1) / 2, g.h0) : g.rt * g.ct;
-  e = make_tmap_rows128(&mb, RB, Kp, (unsigned long long)g.nbatch * g.cols, kMods, smodB, g.bn);
+  e = make_tmap_rows128(&mb, RB, Kp, (unsigned long long)g.nbatch * g.cols, kPlanes, smodB, g.bn);
   if (e != cudaSuccess) return e;
   const int segs = (g.nkb + kSegStages - 1) / kSegStages;
   g.seg = (g.nkb + segs - 1) / segs;
-  const int njobs = kMods * g.nbatch * g.jobs;
+  const int njobs = kPlanes * g.nbatch * g.jobs;
   e = cudaFuncSetAttribute(rns_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kGemmSmem);
   if (e != cudaSuccess) return e;
   rns_gemm_kernel<<<std::min(njobs, c.sms), kGemmThreads, kGemmSmem, s>>>(ma, mb, g, njobs, c.err, c.wait_ns,
@@ -950,9 +1102,9 @@ ZPlan zplan(const ZgemmArgs& a, int al, bool cj, int bl) {
   p.K = a.K;
   p.Kp = (int)pad_to(2ll * a.K, kBK);
   p.ldy = (int)pad_to(2ll * p.cols.rows, 16);
-  p.row_bytes = (size_t)p.rows.rows * p.Kp * 2 * kMods;
-  p.col_bytes = (size_t)2 * p.cols.rows * p.Kp * 2 * kMods;
-  p.y_bytes = (size_t)pad_to(p.rows.rows, 32) * p.ldy * kMods;
+  p.row_bytes = (size_t)p.rows.rows * p.Kp * 2 * kPlanes;
+  p.col_bytes = (size_t)2 * p.cols.rows * p.Kp * 2 * kPlanes;
+  p.y_bytes = (size_t)pad_to(p.rows.rows, 32) * p.ldy * kPlanes;
   return p;
 }
 
@@ -965,7 +1117,7 @@ size_t rns_need(const ZgemmArgs& a) {
 
 size_t rns_need(const DsyrkArgs& a) {
   const size_t kp = (size_t)pad_to(a.K, kBK), rows = (size_t)a.M + (a.mode ? a.N : 0);
-  return rows * kp * 2 * kMods + (size_t)pad_to(a.M, 32) * pad_to(a.N, 16) * kMods + rows * 4 + 65536;
+  return rows * kp * 2 * kPlanes + (size_t)pad_to(a.M, 32) * pad_to(a.N, 16) * kPlanes + rows * 4 + 65536;
 }
 
 // Where the line between the two lies (fitted to shapes from 8 x 256 x 8 to 128 x 22 880 x 1024, single and batched): the
@@ -977,11 +1129,11 @@ size_t rns_need(const DsyrkArgs& a) {
 bool rns_takes_zgemm(const ZgemmArgs& a, const RnsCtx& c) {
   if (!c.scratch || a.lower || a.M <= 0 || a.N <= 0 || a.K <= 0 || a.batch <= 0) return false;
   const ZPlan p = zplan(a, A_KM, false, B_KN);
-  if (p.col_bytes + 2 * kBK * (size_t)p.Kp * 2 * kMods + 256 * (size_t)p.ldy * kMods + (4 << 20) > c.bytes) return false;
+  if (p.col_bytes + 2 * kBK * (size_t)p.Kp * 2 * kPlanes + 256 * (size_t)p.ldy * kPlanes + (4 << 20) > c.bytes) return false;
   const double ctas = std::ceil((double)((a.M + 15) / 16) * ((a.N + 15) / 16) * a.batch / c.sms);
   const double fp64 = 5 + 0.27 * a.K * ctas * std::min(16, (a.M + 1) / 2 * 2) / 16.0;
   const double mn = (double)a.M * a.N * a.batch, conv = ((double)p.rows.rows + 2.0 * p.cols.rows) * p.Kp * a.batch;
-  return fp64 > 28 + 0.085 * a.K + 34e-6 * mn + 12e-6 * conv + 8.0 * kMods / 1.2e9 * mn * a.K;
+  return fp64 > 28 + 0.085 * a.K + 34e-6 * mn + 12e-6 * conv + 8.0 * kPlanes / 1.2e9 * mn * a.K;
 }
 
 cudaError_t rns_zgemm(const ZgemmArgs& a, int al, bool cj, int bl, const RnsCtx& c, cudaStream_t s, int* launches) {
@@ -995,7 +1147,7 @@ cudaError_t rns_zgemm(const ZgemmArgs& a, int al, bool cj, int bl, const RnsCtx&
   if (nb < 1) {
     nb = 1;
     const size_t fixed = p.col_bytes + exps;
-    const size_t per_row = (size_t)p.Kp * 2 * kMods + (size_t)p.ldy * kMods;
+    const size_t per_row = (size_t)p.Kp * 2 * kPlanes + (size_t)p.ldy * kPlanes;
     nr = (int)std::min<size_t>((size_t)p.rows.rows, (avail - fixed) / per_row / 128 * 128);
     if (nr < 1) return cudaErrorInvalidValue;
   }
@@ -1006,10 +1158,10 @@ cudaError_t rns_zgemm(const ZgemmArgs& a, int al, bool cj, int bl, const RnsCtx&
       Carve w{(char*)c.scratch, (char*)c.scratch + c.bytes};
       const long long smA = (long long)n * m * p.Kp, smB = (long long)n * 2 * p.cols.rows * p.Kp;
       // (the column operand first: it stays in place over the row chunks of an entry)
-      __nv_bfloat16* RB = (__nv_bfloat16*)w.take((size_t)smB * 2 * kMods);
+      __nv_bfloat16* RB = (__nv_bfloat16*)w.take((size_t)smB * 2 * kPlanes);
       int* eb = (int*)w.take((size_t)n * p.cols.rows * 4);
-      __nv_bfloat16* RA = (__nv_bfloat16*)w.take((size_t)smA * 2 * kMods);
-      signed char* Y = (signed char*)w.take((size_t)n * pad_to(m, 32) * p.ldy * kMods);
+      __nv_bfloat16* RA = (__nv_bfloat16*)w.take((size_t)smA * 2 * kPlanes);
+      signed char* Y = (signed char*)w.take((size_t)n * pad_to(m, 32) * p.ldy * kPlanes);
       int* ea = (int*)w.take((size_t)n * m * 4);
       if (w.p > w.end) return cudaErrorInvalidValue;
       cudaError_t e = cudaSuccess;
@@ -1039,6 +1191,10 @@ cudaError_t rns_zgemm(const ZgemmArgs& a, int al, bool cj, int bl, const RnsCtx&
       x.alpha = a.alpha;
       x.scaled = a.alpha != 1.0;
       x.beta = a.beta;
+      x.rside = fma_side(p.rows, r0, a.tab, b0);
+      x.cside = fma_side(p.cols, 0, a.tab, b0);
+      x.rows_are_m = p.rows_are_m;
+      x.K = p.K;
       GemmArgs g;
       std::memset(&g, 0, sizeof(g));
       g.nbatch = n;
@@ -1071,10 +1227,10 @@ bool rns_takes_dsyrk(const DsyrkArgs& a, const RnsCtx& c) {
   const double tm = (a.M + 15) / 16, tn = (a.N + 15) / 16, ctas = a.mode == 0 ? tm * (tm + 1) / 2 : tm * tn;
   const double fp64 = 5 + 0.068 * a.K * std::ceil(ctas / c.sms), mn = (a.mode == 0 ? 0.5 : 1.0) * a.M * (double)a.N;
   const double conv = ((double)a.M + (a.mode ? a.N : 0)) * a.K;
-  if (fp64 < 26 + (a.mode ? 8 : 0) + 0.024 * a.K + 17e-6 * mn + 12e-6 * conv + 2.0 * kMods / 1.2e9 * mn * a.K)
+  if (fp64 < 26 + (a.mode ? 8 : 0) + 0.024 * a.K + 17e-6 * mn + 12e-6 * conv + 2.0 * kPlanes / 1.2e9 * mn * a.K)
     return false;
   // at least one K block of both operands and 256 rows of Y
-  const size_t ops = ((size_t)a.M + (a.mode ? a.N : 0)) * kBK * 2 * kMods, y = (size_t)256 * pad_to(a.N, 16) * kMods;
+  const size_t ops = ((size_t)a.M + (a.mode ? a.N : 0)) * kBK * 2 * kPlanes, y = (size_t)256 * pad_to(a.N, 16) * kPlanes;
   return ops + y + ((size_t)a.M + a.N) * 4 + (1 << 20) <= c.bytes;
 }
 
@@ -1086,22 +1242,22 @@ cudaError_t rns_dsyrk(const DsyrkArgs& a, const RnsCtx& c, cudaStream_t s, int* 
   const size_t avail = c.bytes - exps;
   // K in chunks whose residues take at most half of the scratch (or what the smallest row chunk
   // leaves), rows of the result in chunks of what is left; every chunk adds into the output
-  const size_t ymin = (size_t)256 * ldy * kMods;
-  const size_t opmax = std::max(avail / 2, opsrow * kBK * 2 * kMods);
-  long long Kc = std::min<long long>(pad_to(a.K, kBK), (long long)(std::min(opmax, avail - ymin) / (opsrow * 2 * kMods)) / kBK * kBK);
-  const size_t yav = avail - opsrow * Kc * 2 * kMods;
-  const int nr = (int)std::min<size_t>((size_t)pad_to(M, 256), yav / ((size_t)ldy * kMods) / 256 * 256);
+  const size_t ymin = (size_t)256 * ldy * kPlanes;
+  const size_t opmax = std::max(avail / 2, opsrow * kBK * 2 * kPlanes);
+  long long Kc = std::min<long long>(pad_to(a.K, kBK), (long long)(std::min(opmax, avail - ymin) / (opsrow * 2 * kPlanes)) / kBK * kBK);
+  const size_t yav = avail - opsrow * Kc * 2 * kPlanes;
+  const int nr = (int)std::min<size_t>((size_t)pad_to(M, 256), yav / ((size_t)ldy * kPlanes) / 256 * 256);
   if (Kc < kBK || nr < 256) return cudaErrorInvalidValue;
   const Side X{SRC_REAL, a.X, 0, 0, 1, a.ldx, M, 0}, Yo{SRC_REAL, a.Y, 0, 0, 1, a.ldy, N, 0};
   for (long long k0 = 0; k0 < a.K; k0 += Kc) {
     const int K = (int)std::min<long long>(Kc, a.K - k0), Kp = (int)pad_to(K, kBK);
     Carve w{(char*)c.scratch, (char*)c.scratch + c.bytes};
     const long long smA = (long long)M * Kp, smB = (long long)N * Kp;
-    __nv_bfloat16* RA = (__nv_bfloat16*)w.take((size_t)smA * 2 * kMods);
-    __nv_bfloat16* RB = tri ? RA : (__nv_bfloat16*)w.take((size_t)smB * 2 * kMods);
+    __nv_bfloat16* RA = (__nv_bfloat16*)w.take((size_t)smA * 2 * kPlanes);
+    __nv_bfloat16* RB = tri ? RA : (__nv_bfloat16*)w.take((size_t)smB * 2 * kPlanes);
     int* ea = (int*)w.take((size_t)M * 4);
     int* eb = tri ? ea : (int*)w.take((size_t)N * 4);
-    signed char* Y = (signed char*)w.take((size_t)std::min<long long>(nr, pad_to(M, 32)) * ldy * kMods);
+    signed char* Y = (signed char*)w.take((size_t)std::min<long long>(nr, pad_to(M, 32)) * ldy * kPlanes);
     if (w.p > w.end) return cudaErrorInvalidValue;
     Side xs = X, ys = Yo;
     xs.base += k0 * a.ldx;
@@ -1146,6 +1302,9 @@ cudaError_t rns_dsyrk(const DsyrkArgs& a, const RnsCtx& c, cudaStream_t s, int* 
       x.ldo = a.ldo;
       x.tri = tri;
       x.alpha = a.alpha;
+      x.rside = fma_side(xs, r0, nullptr, 0);
+      x.cside = fma_side(tri ? xs : ys, 0, nullptr, 0);
+      x.K = K;
       const dim3 grid(crt_blocks(m, N), 1);
       rns_crt_kernel<false><<<grid, 256, 0, s>>>(x);
       if ((e = cudaGetLastError()) != cudaSuccess) return e;
