@@ -83,10 +83,9 @@ typedef enum {
                             result to FP64. Results that this would leave less accurate than FMAs,
                             those whose sum of magnitudes sum |a| |b| is small beside the rows'
                             norms (graded or localised operands), are formed as FMAs, so that
-                            every result is within the error bound of the chain of FMAs. An
-                            infinity or NaN in an operand row gives NaN in every result of that
-                            row there. Products whose scratch the workspace limit does not leave
-                            run as FMAs. */
+                            every result is within the error bound of the chain of FMAs.
+                            Results of rows with an infinity or a NaN are FMAs too. Products whose
+                            scratch the workspace limit does not leave run as FMAs. */
   DMET_PREC_BF16X3 = 1,  /* three bf16 slices per operand, six slice products per multiply-add */
   DMET_PREC_TF32 = 2,    /* one TF32 slice, one product (about 2^-11 relative per product) */
   DMET_PREC_TF32X3 = 3,  /* two TF32 slices, three products (about 2^-22), half the 16-bit rate */

@@ -33,7 +33,8 @@
 //   3. rns_crt_kernel: recovers the signed 117-bit integer as a 64-bit fraction of P, rounds it to FP64, undoes the
 //      scales, takes the results with a small S from FMAs and writes the caller's layout.
 //
-// A row with an infinity or a NaN gives NaN in every result it enters.
+// A row with an infinity or a NaN has no scale. Its magnitudes count as the smallest, so its results come from FMAs,
+// except where its elements meet zeros only: NaN, as an infinity or NaN times zero is.
 
 #include <cuda.h>
 #include <cuda_bf16.h>
