@@ -769,8 +769,8 @@ __device__ __noinline__ double scaled_value(unsigned long long r, int e, bool po
 }
 
 // x 2^-s from the signed fraction f = 2^64 x / P: |f| P in integers (the FP64 pipe would take a conversion and a
-// multiplication per value, each 1/64 of the rate), rounded to FP64. The fraction is good to 2^-64, that is
-// to 2^-62 of the product of the two rows' norm bounds, below the rounding of the operands.
+// multiplication per value, each 1/64 of the rate), rounded to FP64. The fraction is good to 2^-62.7 of P, that is
+// to 2^-61.3 of the product of the two rows' norm bounds, below the rounding of the operands.
 __device__ __forceinline__ double crt_value(unsigned long long f, int s) {
   constexpr unsigned long long P64 = (unsigned long long)(mod_product() >> 54);
   const unsigned sign = (unsigned)(f >> 32) & 0x80000000u;
