@@ -1086,7 +1086,7 @@ struct Carve {
 struct ZPlan {
   Side rows, cols;
   int K, Kp, ldy;
-  size_t row_bytes, col_bytes, y_bytes;  // per batch entry: row residues, column residues, Y
+  size_t row_bytes, col_bytes, y_bytes, exps;  // per batch entry: row residues, column residues, Y, the rows' scales
   bool rows_are_m;
 };
 
@@ -1106,14 +1106,38 @@ ZPlan zplan(const ZgemmArgs& a, int al, bool cj, int bl) {
   p.row_bytes = (size_t)p.rows.rows * p.Kp * 2 * kPlanes;
   p.col_bytes = (size_t)2 * p.cols.rows * p.Kp * 2 * kPlanes;
   p.y_bytes = (size_t)pad_to(p.rows.rows, 32) * p.ldy * kPlanes;
+  p.exps = ((size_t)p.rows.rows + p.cols.rows) * 4 + 4096;
   return p;
+}
+
+// How a product runs in the scratch there is: chunks of nb whole batch entries, or of nr rows of one entry. False: not
+// at all (less than 128 rows fit beside the column operand and the scales).
+struct ZChunks {
+  int nb, nr;
+  long long launches;  // chunks
+};
+bool zchunks(const ZPlan& p, int batch, size_t bytes, ZChunks* c) {
+  if (bytes <= 16384) return false;
+  const size_t avail = bytes - 16384, fixed = p.col_bytes + p.exps;
+  const int rows = p.rows.rows;
+  c->nb = (int)std::min<size_t>((size_t)batch, avail / (p.row_bytes + p.col_bytes + p.y_bytes + p.exps));
+  c->nr = rows;
+  if (c->nb < 1) {
+    c->nb = 1;
+    if (fixed >= avail) return false;
+    const size_t per_row = ((size_t)p.Kp * 2 + p.ldy) * kPlanes;
+    c->nr = (int)std::min<size_t>((size_t)rows, (avail - fixed) / per_row / 128 * 128);
+    if (c->nr < 1) return false;
+  }
+  c->launches = (long long)((batch + c->nb - 1) / c->nb) * ((rows + c->nr - 1) / c->nr);
+  return true;
 }
 
 }  // namespace
 
 size_t rns_need(const ZgemmArgs& a) {
   const ZPlan p = zplan(a, A_KM, false, B_KN);
-  return (p.row_bytes + p.col_bytes + p.y_bytes + ((size_t)p.rows.rows + p.cols.rows) * 4 + 4096) * a.batch + 16384;
+  return (p.row_bytes + p.col_bytes + p.y_bytes + p.exps) * a.batch + 16384;
 }
 
 size_t rns_need(const DsyrkArgs& a) {
@@ -1127,31 +1151,23 @@ size_t rns_need(const DsyrkArgs& a) {
 // result (reconstruction and epilogue) and 12 ps per converted real element, and the MMAs. A 128 x 4096 product:
 // K = 8, 35 against 43 us; K = 16, 64 against 44; K = 64, 238 against 48. (At large sizes a result
 // takes 20 ps and a converted element 9 since Y lies in tiles; the line, where the launches count, is where it was.)
+// A product that the scratch only lets run in chunks pays the launches for each: where that is many, FMAs are faster.
 bool rns_takes_zgemm(const ZgemmArgs& a, const RnsCtx& c) {
   if (!c.scratch || a.lower || a.M <= 0 || a.N <= 0 || a.K <= 0 || a.batch <= 0) return false;
   const ZPlan p = zplan(a, A_KM, false, B_KN);
-  if (p.col_bytes + 2 * kBK * (size_t)p.Kp * 2 * kPlanes + 256 * (size_t)p.ldy * kPlanes + (4 << 20) > c.bytes) return false;
+  ZChunks ch;
+  if (!zchunks(p, a.batch, c.bytes, &ch)) return false;
   const double ctas = std::ceil((double)((a.M + 15) / 16) * ((a.N + 15) / 16) * a.batch / c.sms);
   const double fp64 = 5 + 0.27 * a.K * ctas * std::min(16, (a.M + 1) / 2 * 2) / 16.0;
   const double mn = (double)a.M * a.N * a.batch, conv = ((double)p.rows.rows + 2.0 * p.cols.rows) * p.Kp * a.batch;
-  return fp64 > 28 + 0.085 * a.K + 34e-6 * mn + 12e-6 * conv + 8.0 * kPlanes / 1.2e9 * mn * a.K;
+  return fp64 > 28.0 * ch.launches + 0.085 * a.K + 34e-6 * mn + 12e-6 * conv + 8.0 * kPlanes / 1.2e9 * mn * a.K;
 }
 
 cudaError_t rns_zgemm(const ZgemmArgs& a, int al, bool cj, int bl, const RnsCtx& c, cudaStream_t s, int* launches) {
   const ZPlan p = zplan(a, al, cj, bl);
-  const size_t exps = ((size_t)p.rows.rows + p.cols.rows) * 4 + 4096;
-  // chunks of whole batch entries, or of rows of one entry
-  const size_t per = p.row_bytes + p.col_bytes + p.y_bytes + exps;
-  const size_t avail = c.bytes - 16384;
-  int nb = (int)std::min<size_t>((size_t)a.batch, avail / per);
-  int nr = p.rows.rows;
-  if (nb < 1) {
-    nb = 1;
-    const size_t fixed = p.col_bytes + exps;
-    const size_t per_row = (size_t)p.Kp * 2 * kPlanes + (size_t)p.ldy * kPlanes;
-    nr = (int)std::min<size_t>((size_t)p.rows.rows, (avail - fixed) / per_row / 128 * 128);
-    if (nr < 1) return cudaErrorInvalidValue;
-  }
+  ZChunks ch;
+  if (!zchunks(p, a.batch, c.bytes, &ch)) return cudaErrorInvalidValue;  // (rns_takes_zgemm tells first)
+  const int nb = ch.nb, nr = ch.nr;
   for (int b0 = 0; b0 < a.batch; b0 += nb) {
     const int n = std::min(nb, a.batch - b0);
     for (int r0 = 0; r0 < p.rows.rows; r0 += nr) {
