@@ -278,9 +278,9 @@ DMET_API dmet_status_t dmet_emb_bath(dmet_emb_plan_t plan, int32_t problem, int3
  *   gamma  complex128 [n][n], the embedding density;
  *   J, K   complex128 [n][n], written (real for real orbitals and a real gamma).
  * FP64 throughout (batched complex GEMMs over the (q, P) entries in chunks, and reductions); queued
- * on the plan's stream; grows a plan-owned scratch buffer of at most about 1 GiB on first use; for
- * larger n (integer products, as for DMET_PREC_FP64) of about 700 MiB beside 256 MiB or the 16 n_aux n^2
- * bytes of one q, and where that much is not to be had the products run as FMAs. */
+ * on the plan's stream; grows a plan-owned scratch buffer of at most about 1 GiB on first use (or
+ * the 32 n^2 bytes of one aux function beside 700 MiB), and where that much is not to be had for larger n (integer
+ * products, as for DMET_PREC_FP64) the products run as FMAs. */
 DMET_API dmet_status_t dmet_emb_jk_df(dmet_emb_plan_t plan, int32_t problem, int32_t spin, const void* Lq,
                                       const void* gamma, void* J, void* K);
 

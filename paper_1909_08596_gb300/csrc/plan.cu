@@ -3029,22 +3029,27 @@ dmet_status_t dmet_emb_bath(dmet_emb_plan_t P, int32_t problem, int32_t spin, co
   return DMET_OK;
 }
 
-// J and K of dmet_emb_jk_df through residue products, q by q in chunks: W = L^q_P gamma for every P, stored [P][l][i], then
-// K += (1/Nk) sum over (P, l) of W[(P, l)][i] L^{-q}[(P, l)][j] as one product of K = n_aux n per q, split into
-// parts of the aux functions that fill the GPU. *done = false: the products are too small for it (nothing queued).
+// J and K of dmet_emb_jk_df through residue products, in chunks of whole q or, where one is larger, of some aux functions
+// of a q: W = L^q_P gamma for every P, stored [P][l][i], then K += (1/Nk) sum over (P, l) of W[(P, l)][i] L^{-q}[(P, l)][j] as
+// one product per q, split into parts of the aux functions that fill the GPU. *done = false: the products are too
+// small for it (nothing queued).
 static dmet_status_t jk_residues(dmet_emb_plan_s* P, Prob& pr, int n, const double2* Lq, const double2* gamma,
                                  double2* J, double2* K, bool* done) {
   *done = false;
   const int nk = pr.nk, naux = pr.naux;
   const long long nn = (long long)n * n;
   if ((long long)naux * n > INT_MAX / 4 || nk > 65535) return DMET_OK;
-  const size_t wq = (size_t)naux * nn * 16;  // W of one q
-  const int cq = (int)std::max<size_t>(1, std::min<size_t>(nk, ((size_t)256 << 20) / wq));
-  // Parts of some 480 K (complex): as many parts then fit a chunk of the scratch as its conversions (one CTA per 32
-  // rows and part) need to fill the GPU twice. h-BN-shaped, 10 parts of K = 2912 a chunk: each conversion took
-  // 306 or 258 us at 130 CTAs, two thirds of the call.
-  const int pl = std::max(1, std::min(naux, 480 / n)), parts = (naux + pl - 1) / pl;
-  if ((long long)cq * parts > 65535) return DMET_OK;
+  // Parts of some 960 K (complex): enough of them fit a chunk of the residues' scratch for its conversions (one CTA
+  // per 32 rows and part) to fill the GPU, and few enough that the parts' reconstructions and their sum, n^2 each, stay small.
+  // (36 q, 220 aux functions, n = 104) / (4, 500, 160) / (2, 600, 256) / (2, 900, 300) / (1, 1200, 400): 480 K 15.6 /
+  // 8.8 / 14.3 / 35.1 / 42.3 ms, 960 14.9 / 9.0 / 13.3 / 31.8 / 39.5, 1920 16.3 / 9.7 / 14.1 / 33.5 / 43.0.
+  const int pl = std::max(1, std::min(naux, 960 / n));
+  // W and the parts of a chunk take at most 320 MiB, and 704 the residues
+  const size_t wp = (size_t)nn * 16;  // W of one aux function
+  const int fit = (int)std::min<size_t>((size_t)INT_MAX / 2, ((size_t)320 << 20) / (wp + (wp + pl - 1) / pl));
+  const int pa = std::min(naux, std::max(1, fit / pl) * pl), cq = std::max(1, std::min(nk, fit / naux));
+  const int parts = cq * ((pa + pl - 1) / pl);  // of a chunk
+  if (parts > 65535) return DMET_OK;
   ZgemmArgs z1 = zargs(), z2 = zargs();
   z1.A = gamma;  // opA(b, l) = gamma[l][b], opB(l, (P, a)) = L[(P, a)][l], stored at [P][b][a]
   z1.M = n;
@@ -3055,7 +3060,7 @@ static dmet_status_t jk_residues(dmet_emb_plan_s* P, Prob& pr, int n, const doub
   z1.dn_div = n;
   z1.dn_hi = nn;
   z1.dn_lo = 1;
-  z1.N = (int)std::min<long long>((long long)cq * naux * n, INT_MAX / 4);
+  z1.N = cq * pa * n;
   z2.M = n;      // opA((P, l), i) = W[P][l][i], opB((P, l), j) = L^{-q}[P][l][j]
   z2.N = n;
   z2.K = pl * n;
@@ -3067,11 +3072,22 @@ static dmet_status_t jk_residues(dmet_emb_plan_s* P, Prob& pr, int n, const doub
   z2.dm_lo = n;
   z2.dn_lo = 1;
   z2.alpha = 1.0 / nk;
-  z2.batch = cq * parts;
+  z2.batch = parts;
+  std::vector<int4> t;     // the parts of every chunk, in order
+  std::vector<int> first;  // where a chunk's begin
+  for (int q0 = 0; q0 < nk; q0 += cq)
+    for (int a0 = 0; a0 < naux; a0 += pa) {
+      first.push_back((int)t.size());
+      const int np = std::min(pa, naux - a0);
+      for (int q = q0, h = 0; q < std::min(nk, q0 + cq); ++q)
+        for (int p0 = 0; p0 < np; p0 += pl, ++h)
+          t.push_back(make_int4((q - q0) * np + p0, pr.s.neg[q] * naux + a0 + p0, h, std::min(pl, np - p0) * n));
+    }
+  first.push_back((int)t.size());
   // scratch: W, the parts of K, the entry table, the Coulomb pass, the residues
-  const size_t oP = ((size_t)cq * wq + 255) / 256 * 256, oT = oP + (size_t)cq * parts * nn * 16;
-  const size_t oG = oT + (size_t)nk * parts * sizeof(int4), oV = oG + (size_t)nn * 16;
-  const size_t oJ = oV + (size_t)nk * naux * 16, oR = (oJ + (size_t)jk_coulomb_parts(nn) * nn * 16 + 1023) / 1024 * 1024;
+  const size_t oP = ((size_t)cq * pa * wp + 255) / 256 * 256, oT = oP + (size_t)parts * wp;
+  const size_t oG = oT + t.size() * sizeof(int4), oV = oG + wp;
+  const size_t oJ = oV + (size_t)nk * naux * 16, oR = (oJ + (size_t)jk_coulomb_parts(nn) * wp + 1023) / 1024 * 1024;
   const size_t rb = std::min<size_t>((size_t)704 << 20, std::max(rns_need(z1), rns_need(z2)));
   RnsCtx c = rns_ctx(P);
   c.scratch = (void*)16;  // (only tested for being there)
@@ -3087,36 +3103,30 @@ static dmet_status_t jk_residues(dmet_emb_plan_s* P, Prob& pr, int n, const doub
   double2* part = (double2*)(w + oP);
   int4* tab = (int4*)(w + oT);
   c.scratch = w + oR;
-  std::vector<int4> t((size_t)nk * parts);
-  for (int q = 0; q < nk; ++q)
-    for (int h = 0; h < parts; ++h) {
-      const int p0 = h * pl, p1 = std::min(naux, p0 + pl);
-      t[(size_t)q * parts + h] = make_int4(q * naux + p0, pr.s.neg[q] * naux + p0, (q % cq) * parts + h, (p1 - p0) * n);
-    }
   // flops: the two products and the two reductions of every (q, P)
   Timed tm(P, KC_JK_DF, 8.0 * nk * naux * (2.0 * nn * n + 2.0 * nn), 16.0 * nk * naux * nn * 5, 4);
   CK(cudaMemcpyAsync(tab, t.data(), t.size() * sizeof(int4), cudaMemcpyHostToDevice, P->cs));
   CK(cudaMemsetAsync(J, 0, (size_t)nn * 16, P->cs));
   CK(cudaMemsetAsync(K, 0, (size_t)nn * 16, P->cs));
-  int launches = 0;
+  int launches = 0, chunk = 0;
   CK(launch_jk_coulomb(Lq, pr.d_neg, nk, naux, n, gamma, 1.0 / nk, (double2*)(w + oG), (double2*)(w + oV),
                        (double2*)(w + oJ), J, P->cs));
-  for (int q0 = 0; q0 < nk; q0 += cq) {
-    const int nq = std::min(cq, nk - q0);
-    z1.B = Lq + (long long)q0 * naux * nn;
-    z1.D = W;
-    z1.N = nq * naux * n;
-    CK(rns_zgemm(z1, A_KM, false, B_NK, c, P->cs, &launches));
-    z2.A = W - (long long)q0 * naux * nn;  // (the table holds absolute q)
-    z2.B = Lq;
-    z2.D = part;
-    z2.tab = tab;
-    z2.tab0 = q0 * parts;
-    z2.batch = nq * parts;
-    CK(rns_zgemm(z2, A_KM, false, B_KN, c, P->cs, &launches));
-    CK(launch_sum_parts(part, nq * parts, nn, K, P->cs));
-    ++launches;
-  }
+  for (int q0 = 0; q0 < nk; q0 += cq)
+    for (int a0 = 0; a0 < naux; a0 += pa, ++chunk) {
+      z1.B = Lq + ((long long)q0 * naux + a0) * nn;
+      z1.D = W;
+      z1.N = std::min(cq, nk - q0) * std::min(pa, naux - a0) * n;
+      CK(rns_zgemm(z1, A_KM, false, B_NK, c, P->cs, &launches));
+      z2.A = W;
+      z2.B = Lq;
+      z2.D = part;
+      z2.tab = tab;
+      z2.tab0 = first[chunk];
+      z2.batch = first[chunk + 1] - first[chunk];
+      CK(rns_zgemm(z2, A_KM, false, B_KN, c, P->cs, &launches));
+      CK(launch_sum_parts(part, z2.batch, nn, K, P->cs));
+      ++launches;
+    }
   tm.more(launches);
   *done = true;
   return DMET_OK;
