@@ -298,8 +298,10 @@ DMET_API dmet_status_t dmet_emb_jk_df(dmet_emb_plan_t plan, int32_t problem, int
  * (the plane waves and kernel of dmet_fftdf_plane_waves, 0 at q + G = 0), the inverse DFT,
  * exp(+i q.r), and (ij|kl) += Omega / (N_g Nk) sum_r w(r)_ij (r|0k 0l)^{-q} with the inverse DFT
  * normalised by 1/N_g (Omega the cell volume). The DFTs run axis by axis, as FFTs in registers where
- * every axis has at most 32 points and no prime factor above 7 (else dense, as batched complex GEMMs). FP64 throughout; queued on the plan's stream; grows a plan-owned scratch buffer on first use
- * (2 N_g n^2 complex values). */
+ * every axis has at most 32 points and no prime factor above 7 (else dense, as batched complex GEMMs).
+ * FP64 throughout; queued on the plan's stream; grows a plan-owned scratch buffer on first use: N_g n^2 complex
+ * values per q, twice that for the dense form, of as many q as fit 4 GiB (at least one), and the split contraction's
+ * partial blocks of at most 1 GiB. */
 DMET_API dmet_status_t dmet_emb_eri_fftdf(dmet_emb_plan_t plan, int32_t problem, const void* rho,
                                           const void* const* C, const int32_t* grid, const double* lattice,
                                           void* const* eri_out);

@@ -290,6 +290,9 @@ __global__ void __launch_bounds__(256) sum_parts_kernel(const double2* __restric
 
 }  // namespace
 
+// Every length up to 32 that the FFTs take is faster than dense; whole calls with one cell or two and a cubic grid, dense
+// against FFTs, in us: 2: 225 and 92, 5: 430 and 154, 7: 598 and 193, 9: 789 and 283, 12: 1819 and 482, 16: 2552 and 775,
+// 18: 3087 and 1214, 20: 1652 and 563, 24: 2138 and 822, 28: 4031 and 1258, 30: 7138 and 4208, 32: 4813 and 1753.
 bool fftdf_fft_axis(int g) {
   if (g < 1 || g > kMaxDftAxis) return false;
   for (int p : {2, 3, 5, 7})

@@ -3319,8 +3319,11 @@ dmet_status_t dmet_emb_eri_fftdf(dmet_emb_plan_t P, int32_t problem, const void*
   // so a chunk of consecutive q' pairs the transformed factors of q = -q' (computed in that order)
   // with a contiguous run of the untransformed ones: one GEMM over K = qc N_g per chunk and spin pair.
   const long long g0 = grid[0], g1 = grid[1], g2 = grid[2];
+  // The FFTs run in place, the dense form between two buffers; they stay within 4 GiB.
+  const bool ffts = fftdf_fft_axis(grid[0]) && fftdf_fft_axis(grid[1]) && fftdf_fft_axis(grid[2]);
+  const int nbuf = ffts ? 1 : 2;
   int qc = nk;
-  while (qc > 1 && ((size_t)qc * ng * nx_max * 16 * 2 > ((size_t)4 << 30) || (long long)qc * g0 * g1 > 65535 ||
+  while (qc > 1 && ((size_t)qc * ng * nx_max * 16 * nbuf > ((size_t)4 << 30) || (long long)qc * g0 * g1 > 65535 ||
                     (long long)qc * ng > INT_MAX))
     qc = (qc + 1) / 2;
   if ((long long)qc * g0 * g1 > 65535 || (long long)qc * ng > INT_MAX)
@@ -3332,7 +3335,6 @@ dmet_status_t dmet_emb_eri_fftdf(dmet_emb_plan_t P, int32_t problem, const void*
     std::memcpy(vp.data() + (size_t)qq * ng, vq.data() + (size_t)qtab[qq] * ng, sizeof(double) * ng);
   }
   // exp(-i q.r) = prod_d exp(-2 pi i j_d n_d / (N_d g_d)), tabulated per axis for q = -q', for the FFT passes
-  const bool ffts = fftdf_fft_axis(grid[0]) && fftdf_fft_axis(grid[1]) && fftdf_fft_axis(grid[2]);
   std::vector<double2> ph;
   size_t ph_off[3];
   for (int d = 0; d < 3; ++d) {
@@ -3353,16 +3355,16 @@ dmet_status_t dmet_emb_eri_fftdf(dmet_emb_plan_t P, int32_t problem, const void*
   while (kparts < 64 && tiles_min * kparts < 2 * 152 && ktot % (2 * kparts) == 0 && ktot / (2 * kparts) >= 64 &&
          (size_t)(2 * kparts) * nx_max * nx_max * 16 <= ((size_t)1 << 30))
     kparts *= 2;
-  // scratch: two [qc][grid][n^2] buffers, the DFT matrices, the kernels, the q table, the K parts
-  const size_t bbuf = (size_t)qc * ng * nx_max * 16, oF = 2 * bbuf, oV = oF + (F.size() * 16 + 255) / 256 * 256;
+  // scratch: one or two [qc][grid][n^2] buffers, the DFT matrices, the kernels, the q table, the phases, the K parts
+  const size_t bbuf = (size_t)qc * ng * nx_max * 16, oF = nbuf * bbuf, oV = oF + (F.size() * 16 + 255) / 256 * 256;
   const size_t oQ = oV + (vp.size() * 8 + 255) / 256 * 256;
   const size_t oH = oQ + (qtab.size() * sizeof(int) + 255) / 256 * 256;
   const size_t oP = oH + (ph.size() * 16 + 255) / 256 * 256;
   P->cs = P->stream;
   TRY(ensure(&P->fft_ws, &P->fft_ws_b, oP + (kparts > 1 ? (size_t)kparts * nx_max * nx_max * 16 : 0)));
   char* w = (char*)P->fft_ws;
-  double2* buf0 = (double2*)w;
-  double2* buf1 = (double2*)(w + bbuf);
+  double2* buf1 = (double2*)w;
+  double2* buf0 = ffts ? nullptr : (double2*)(w + bbuf);  // (of the dense form)
   double2* dF = (double2*)(w + oF);
   double* dV = (double*)(w + oV);
   int* dQ = (int*)(w + oQ);
