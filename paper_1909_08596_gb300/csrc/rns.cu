@@ -20,9 +20,10 @@
 // down, go through the GEMM as a plane beside the residues, and the reconstruction replaces every result with too small
 // an S by the chain of FMAs over the original operands (fma_results). Where S is zero the result is, exactly.
 // Measured against quads, two half transforms of K = 48, worst element and rms in units of 2^-53 S: random operands
-// 0.16 and 0.025 (FMAs 0.78 and 0.12), elements spread over two decades 1.0 and 0.09 (3.4 and 0.39), four 3.9 and 0.28
-// (7.9 and 0.85), eight 8.6 and 0.82 (9.3 and 1.4). The plane costs 8% of an h-BN-shaped call (17.5 -> 18.95 ms); the
-// same with operands graded over 4 / 8 / 40 decades takes 30 / 149 / 262 ms (some 390 on the FP64 pipe alone).
+// 0.16 and 0.025 (FMAs 0.78 and 0.12), elements spread over two decades 0.9 and 0.09 (3.4 and 0.39), four 3.9 and 0.28
+// (7.9 and 0.85), eight 7.5 and 0.82 (9.3 and 1.4). The plane costs 8% of an h-BN-shaped call (17.4 -> 18.8 ms); the
+// same with L and C falling by 2 / 4 / 20 decades from their diagonals takes 24 / 140 / 256 ms (some 390 on the FP64
+// pipe alone).
 //
 //   1. rns_convert_kernel: per operand row, the scale from its norm; then residues [plane][batch][row][K], the
 //      magnitudes as the last plane, K-major (complex operands as interleaved (re, im) pairs along K; the column
@@ -859,8 +860,9 @@ __device__ __forceinline__ unsigned small_sums(unsigned w) {
   }
 }
 
-// The results of a warp's 32 x 16 (8 complex) that `flags` marks, a bit per column and lane (row), as the FP64 kernels
-// form them: listed in order of columns, a lane per result.
+// The results of a warp's 32 x 16 (8 complex) that `flags` marks, a bit per column and lane (row), as FMAs: listed in
+// order of columns, a lane per result while there are 32, 32 / n lanes for each of the last n (one lane each: 400 us
+// more for an FFTDF call of 2.1 ms with a few results of K = 432, and the h-BN-shaped call of 2 decades 30 ms, now 24).
 template <bool CPLX>
 __device__ __noinline__ void fma_results(const CrtArgs& a, double* st, unsigned short* list, unsigned flags, int c0,
                                          int rbase, int z) {
@@ -884,10 +886,15 @@ __device__ __noinline__ void fma_results(const CrtArgs& a, double* st, unsigned 
     K = t.w;
   }
 #pragma unroll 1
-  for (int t = lane; t < n; t += 32) {
-    const int r = list[t] & 31, c = list[t] >> 5;
+  for (int t0 = 0; t0 < n; t0 += 32) {
+    int g = 1;  // lanes per result
+    while ((n - t0) * g <= 16) g *= 2;
+    const int t = t0 + lane / g, k0 = lane & (g - 1);
+    const int item = t < n ? list[t] : 0, r = item & 31, c = item >> 5;
     const long long ro = zr * a.rside.sbatch + (rbase + r) * a.rside.s_row;
     const long long co = zc * a.cside.sbatch + (cbase + c) * a.cside.s_row;
+    const int Kt = t < n ? K : 0;
+    double re = 0.0, im = 0.0;
     if constexpr (CPLX) {
       const double2* p = reinterpret_cast<const double2*>(a.rside.src) + ro;
       const double2* q = reinterpret_cast<const double2*>(a.cside.src) + co;
@@ -900,9 +907,8 @@ __device__ __noinline__ void fma_results(const CrtArgs& a, double* st, unsigned 
         qs = a.rside.s_k;
       }
       const bool cj = a.rside.conj | a.cside.conj;  // (of the m operand)
-      double re = 0.0, im = 0.0;
 #pragma unroll 4
-      for (int k = 0; k < K; ++k) {
+      for (int k = k0; k < Kt; k += g) {
         double2 u = p[k * ps];
         const double2 v = q[k * qs];
         if (cj) u.y = -u.y;
@@ -911,15 +917,19 @@ __device__ __noinline__ void fma_results(const CrtArgs& a, double* st, unsigned 
         re = fma(-u.y, v.y, re);
         im = fma(u.y, v.x, im);
       }
-      st[r * 17 + 2 * c] = re;
-      st[r * 17 + 2 * c + 1] = im;
     } else {
       const double* p = a.rside.src + ro;
       const double* q = a.cside.src + co;
-      double v = 0.0;
 #pragma unroll 4
-      for (int k = 0; k < K; ++k) v = fma(p[k * a.rside.s_k], q[k * a.cside.s_k], v);
-      st[r * 17 + c] = v;
+      for (int k = k0; k < Kt; k += g) re = fma(p[k * a.rside.s_k], q[k * a.cside.s_k], re);
+    }
+    for (int o = g >> 1; o; o >>= 1) {
+      re += __shfl_xor_sync(0xffffffffu, re, o);
+      if constexpr (CPLX) im += __shfl_xor_sync(0xffffffffu, im, o);
+    }
+    if (t < n && k0 == 0) {
+      st[r * 17 + (CPLX ? 2 * c : c)] = re;
+      if constexpr (CPLX) st[r * 17 + 2 * c + 1] = im;
     }
   }
   __syncwarp();
