@@ -231,7 +231,7 @@ DMET_API dmet_status_t dmet_emb_status(dmet_emb_plan_t plan, int32_t problem, do
  *   gamma    FP64 [n][n], symmetric, spin-summed, in the embedding basis;
  *   fock_out FP64 [n][n] (the real part of F0, whose imaginary part vanishes for real orbitals).
  * FP64 throughout; queued on the plan's stream; grows a plan-owned scratch buffer on first use
- * (about 16 Nk n_AO n + 16 Nk n^2 + 300 n^2 bytes). */
+ * (about 16 Nk n_AO n + 16 Nk n^2 + 150 n^2 bytes). */
 DMET_API dmet_status_t dmet_emb_fock(dmet_emb_plan_t plan, int32_t problem, const void* F, const void* C,
                                      const double* eri, const double* gamma, double* fock_out);
 

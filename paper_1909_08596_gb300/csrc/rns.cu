@@ -6,8 +6,8 @@
 // cores about 1500 times that, and 16-bit integers up to 2^7 multiply and add exactly in their FP32
 // accumulators. So every row of A and of B is scaled by a power of two to integers of about kBeta
 // bits (a 2-norm of at most 2^kBeta, so that no inner product exceeds 2^(2 kBeta)), and the integer
-// product is formed exactly by the Chinese remainder theorem (the number-theoretic form of the
-// error-free matrix products of Ozaki et al.): kMods pairwise coprime moduli of at most 8 bits, one
+// product is formed exactly by the Chinese remainder theorem (the modular form of the
+// error-free matrix products: K. Ozaki, Y. Uchino, T. Imamura, "Ozaki Scheme II", arXiv:2504.08009, 2025): kMods pairwise coprime moduli of at most 8 bits, one
 // GEMM of symmetric residues (bf16, |r| <= 128) per modulus, and the product recovered modulo
 // P = prod p_i > 2 * 2^(2 kBeta). The only errors are the rounding of the operands to integers, half
 // a unit of 2^-kBeta of the row's norm (5 bits below the FP64 rounding of an element of the row's
@@ -21,7 +21,7 @@
 // an S by the chain of FMAs over the original operands (fma_results). Where S is zero the result is, exactly.
 // Measured against quads, two half transforms of K = 48, worst element and rms in units of 2^-53 S: random operands
 // 0.16 and 0.025 (FMAs 0.78 and 0.12), elements spread over two decades 0.9 and 0.09 (3.4 and 0.39), four 3.9 and 0.28
-// (7.9 and 0.85), eight 7.5 and 0.82 (9.3 and 1.4). The plane costs 8% of an h-BN-shaped call (17.4 -> 18.8 ms); the
+// (7.9 and 0.85), eight 7.5 and 0.82 (9.3 and 1.4). The plane costs 6% of an h-BN-shaped call (17.5 -> 18.6 ms); the
 // same with L and C falling by 2 / 4 / 20 decades from their diagonals takes 24 / 140 / 256 ms (some 390 on the FP64
 // pipe alone).
 //
@@ -522,20 +522,28 @@ __device__ __forceinline__ uint4 reduce16(const uint32_t (&v)[16], bool add, uin
   return make_uint4(w[0], w[1], w[2], w[3]);
 }
 
-// 16 sums of magnitudes to bytes: 2 floor(128 S) (a segment's share rounded down, at most 254) + (S != 0).
+// 16 sums of magnitudes to bytes: 2 n + (S != 0), n = 127 S rounded down (within one), a segment added to the next: S is
+// at most 1 over all of K, so n stays below 128. An S other than zero is at least 2^-124, so its upper byte is not zero.
+// (With conversions to integers instead of the rounding constant the GEMM of 2465 x 61 x 17 in 76 batches took 189 us, 184
+// so, and an h-BN-shaped call 18.60 ms, 18.57.)
 __device__ __forceinline__ uint4 count16(const uint32_t (&v)[16], bool add, uint4 prev) {
+  constexpr f32x2 scale = both_of(127.f), minus_half = both_of(-0.5f);
   uint32_t w[4];
   const uint32_t pv[4] = {prev.x, prev.y, prev.z, prev.w};
 #pragma unroll
   for (int g = 0; g < 4; ++g) {
-    w[g] = 0;
+    float b[4];
 #pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      const float f = __uint_as_float(v[4 * g + c]);
-      const unsigned old = add ? (pv[g] >> (8 * c)) & 255u : 0u;
-      const unsigned n = min((unsigned)(f * 128.f) + (old >> 1), 127u);
-      w[g] |= (n << 1 | (f > 0.f ? 1u : 0u) | (old & 1u)) << (8 * c);
+    for (int c = 0; c < 4; c += 2) {
+      const f32x2 x = pack2(__uint_as_float(v[4 * g + c]), __uint_as_float(v[4 * g + c + 1]));
+      unpack2(add2(fma2(x, scale, minus_half), kMagic2), b[c], b[c + 1]);  // the low byte is n
     }
+    const uint32_t n = __byte_perm(__byte_perm(__float_as_uint(b[0]), __float_as_uint(b[1]), 0x0040),
+                                   __byte_perm(__float_as_uint(b[2]), __float_as_uint(b[3]), 0x0040), 0x5410);
+    const uint32_t t = __byte_perm(__byte_perm(v[4 * g], v[4 * g + 1], 0x0073),
+                                   __byte_perm(v[4 * g + 2], v[4 * g + 3], 0x0073), 0x5410);
+    w[g] = (n << 1) | (((t + 0x7f7f7f7fu) >> 7) & 0x01010101u);
+    if (add) w[g] = (w[g] + (pv[g] & 0xfefefefeu)) | (pv[g] & 0x01010101u);
   }
   return make_uint4(w[0], w[1], w[2], w[3]);
 }
@@ -671,16 +679,21 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
         }
         tc_fence_after();
         const uint32_t tm = tmem + b * 256 + ((uint32_t)(quad * 32) << 16);
+        auto drain = [&](auto to_bytes) {
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          const int c = half * 16 + 32 * i;
-          if (c >= cols) break;  // (uniform)
-          uint32_t v[16];
-          tmem_ld_32x32b_x16(tm + c, v);
-          tmem_ld_wait();
-          const uint4 w = mags ? count16(v, k0 != 0, prev[i]) : reduce16(v, k0 != 0, prev[i], minus_p, rp);
-          if (rok) *reinterpret_cast<uint4*>(y + (half + 2 * i) * 512) = w;
-        }
+          for (int i = 0; i < 8; ++i) {
+            const int c = half * 16 + 32 * i;
+            if (c >= cols) break;  // (uniform)
+            uint32_t v[16];
+            tmem_ld_32x32b_x16(tm + c, v);
+            tmem_ld_wait();
+            const uint4 w = to_bytes(v, prev[i]);
+            if (rok) *reinterpret_cast<uint4*>(y + (half + 2 * i) * 512) = w;
+          }
+        };
+        // (two loops: with the choice within one an h-BN-shaped call took 18.83 ms, so 18.60)
+        if (mags) drain([&](const uint32_t (&v)[16], uint4 o) { return count16(v, k0 != 0, o); });
+        else drain([&](const uint32_t (&v)[16], uint4 o) { return reduce16(v, k0 != 0, o, minus_p, rp); });
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(acce(b));
@@ -840,7 +853,7 @@ __device__ __forceinline__ void store_complex(const CrtArgs& a, double2* D, cons
   __syncwarp();
 }
 
-// Results whose S is below kMinCount / 128 of the norms' bounds come from FMAs: the residues' error, about 2^-59 of
+// Results whose S is below kMinCount / 127 of the norms' bounds come from FMAs: the residues' error, about 2^-59 of
 // those bounds, is then above the 2^-54 S of a chain.
 constexpr unsigned kMinCount = 4;
 
