@@ -43,7 +43,7 @@ import synth  # noqa: E402
 METRIC = "embedded-ERI transform TFLOP/s and ms/problem at stated error vs FP64; % of roofline"
 DEFAULT_WORKLOAD = "nio_4x4x4_uhf"
 SMS = 152
-RESIDUE_PRODUCTS = 15  # moduli of the FP64 products (csrc/rns.cu)
+RESIDUE_PRODUCTS = 16  # planes of the FP64 products: 15 moduli and the magnitudes (csrc/rns.cu)
 DFMA_PER_SM_CLK = 2  # FP64 FMA lanes per SM per clock on GB300 (1.25 TFLOP/s nominal at 2.07 GHz)
 REF_SAMPLE_ORBITALS = 24
 # dmet_prec_t codes, and each tensor-core precision's tensor rate relative to dense bf16 (the recipe's
@@ -365,11 +365,24 @@ def measured_peaks():
 
 
 def residue_peak():
-    """FP64 flops per second if every product ran as RESIDUE_PRODUCTS integer products on the bf16 tensor cores."""
+    """FP64 flops per second if every product ran as RESIDUE_PRODUCTS products on the bf16 tensor cores."""
     peaks, src = measured_peaks()
     return peaks["bf16_tflops"] / RESIDUE_PRODUCTS, (
-        f"{src} bf16_tflops / {RESIDUE_PRODUCTS} (FP64 products as {RESIDUE_PRODUCTS} products of residues on the tensor "
-        "cores; the FP64 pipe's own peak is 1.26 TFLOP/s)")
+        f"{src} bf16_tflops / {RESIDUE_PRODUCTS} (FP64 products as 15 products of residues and one of magnitudes "
+        "on the tensor cores; the FP64 pipe's own peak is 1.26 TFLOP/s)")
+
+
+def fp64_pipe_peak():
+    return SMS * DFMA_PER_SM_CLK * 2 * 2070e6 / 1e12, "derived FP64 peak (152 SMs x 2 FMA/clk x 2 x 2070 MHz)"
+
+
+def fp64_roofline(achieved):
+    """(bound, peak, its source) of a rate of FP64 products: above the FP64 pipe's peak only the residue products can
+    have run; a rate below it is held to that pipe."""
+    peak, text = fp64_pipe_peak()
+    if achieved <= peak:
+        return "alu", peak, text
+    return ("tensor", *residue_peak())
 
 
 def roofline(spec, prec, kstats, sustained=False):
@@ -377,9 +390,9 @@ def roofline(spec, prec, kstats, sustained=False):
     top = max(kstats, key=lambda k: k["ms"])
     avg_ms = top["ms"] / max(top["launches"], 1)
     if prec == "fp64":
-        peak, peak_text = residue_peak()
         achieved = top["flops"] / (top["ms"] / 1e3) / 1e12 if top["ms"] > 0 else 0.0
-        return {"bound": "tensor", "kernel": top["name"], "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
+        bound, peak, peak_text = fp64_roofline(achieved)
+        return {"bound": bound, "kernel": top["name"], "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                 "frac": achieved / peak, "traffic": traffic_of((spec.name, prec, top["name"])),
                 "flops_counted": "algorithmic FP64 flops",
                 "peak_source": peak_text,
@@ -525,14 +538,14 @@ def measure_fock_and_bath(dm, torch, spec, Cd, eri0):
                   if k["name"] == "embedding_fock"][0]
             dm.dmet_emb_profile(plan, False)
             f_ms = ef0.elapsed_time(ef1) / reps
-            f_peak = SMS * DFMA_PER_SM_CLK * 2 * 2070e6 / 1e12
+            f_peak, f_text = fp64_pipe_peak()
             f_tf = fk["flops"] / reps / (f_ms / 1e3) / 1e12
             fock = {"ms": f_ms, "launches_per_call": fk["launches"] // reps,
                     "roofline": {"bound": "alu", "achieved": f_tf, "peak": f_peak, "unit": "TFLOP/s",
                                  "frac": f_tf / f_peak,
-                                 "flops_counted": "FP64 flops the kernels execute (transform GEMMs; 2 n^2 exchange "
-                                                  "and n(n+1)/2 Coulomb multiply-adds per ERI pair row)",
-                                 "peak_source": "derived FP64 peak (152 SMs x 2 FMA/clk x 2 x 2070 MHz)"}}
+                                 "flops_counted": "FP64 flops the kernels execute (transform GEMMs; four exchange "
+                                                  "and two Coulomb multiply-adds per stored ERI element)",
+                                 "peak_source": f_text}}
     finally:
         dm.dmet_emb_destroy(plan)
     # The bath: the same cell and mesh, its n_AO LOs as the impurity and 8 of them as the valence
@@ -1017,7 +1030,6 @@ def run_rows_f(args):
     from paper_1909_08596_gb300 import build as libbuild
     libbuild.build()
     stream = torch.cuda.current_stream()
-    f_peak, f_text = residue_peak()
     reps = max(args.steps, 1)
     out = {"metric": METRIC, "workload": "rows_f (density-fitted J/K at the h-BN size; FFTDF on a 2x2x2 mesh)",
            "dtype": "f64"}
@@ -1051,11 +1063,13 @@ def run_rows_f(args):
     Jr, Kr = oracle.coulomb_exchange_df(Lq.cpu().numpy(), gam.cpu().numpy(), spec.mesh)
     scale = float(np.abs(Jr).max())
     tf = ks["flops"] / reps / (ms / 1e3) / 1e12
+    bound, f_peak, f_text = fp64_roofline(tf)
     out["jk_df"] = {"config": {"mesh": list(spec.mesh), "n_aux": spec.n_aux, "n_emb": n}, "ms_per_call": ms,
                     "launches_per_call": ks["launches"] // reps, "status": st,
-                    "roofline": {"bound": "tensor", "achieved": tf, "peak": f_peak, "unit": "TFLOP/s",
+                    "roofline": {"bound": bound, "achieved": tf, "peak": f_peak, "unit": "TFLOP/s",
                                  "frac": tf / f_peak,
-                                 "flops_counted": "FP64 flops of the batched complex GEMMs (L^q gamma L^-q) and traces",
+                                 "flops_counted": "FP64 flops of L^q gamma for every (q, P), of its product with L^-q "
+                                                  "over (P, l), and of the Coulomb traces and sums",
                                  "peak_source": f_text},
                     "max_abs_err_over_max_J": {"J": float(np.abs(J.cpu().numpy() - Jr).max()) / scale,
                                                "K": float(np.abs(K.cpu().numpy() - Kr).max()) / scale}}
@@ -1089,18 +1103,27 @@ def run_rows_f(args):
     ms = e0.elapsed_time(e1) / reps
     ref = of.embedded_eri_fftdf(rho, Cg, gspec.mesh, gspec.lattice, gspec.grid).ravel()
     got = eo.cpu().numpy()
-    # the roofline of the FFTDF steps themselves (the phases, the per-axis FFTs, the kernel and the
-    # contraction over the grid) over their own event time; the half transforms before them are Algorithm 1's
-    tf = ks["flops"] / (ks["ms"] / 1e3) / 1e12 if ks["ms"] > 0 else 0.0
+    # the roofline of the FFTDF steps themselves (the per-axis FFTs with the phases and the kernel in them, and the
+    # contraction over the grid) over their own event time; the half transforms before them are Algorithm 1's. Held to
+    # the larger of the HBM time of their bytes and the FP64 pipe's time of the FFTs' flops; the contraction, whose
+    # products can run on the tensor cores, beside it (its time is in the class's).
+    nk_g, n_g = int(np.prod(gspec.mesh)), gspec.n_emb
+    con_fl = 8.0 * nk_g * ng * n_g ** 4
+    secs = ks["ms"] / reps / 1e3
+    fft_fl, by = ks["flops"] / reps - con_fl, ks["bytes"] / reps
+    hbm, (pipe, pipe_text) = measured_peaks()[0]["hbm_gbs"], fp64_pipe_peak()
+    if by / (hbm * 1e9) >= fft_fl / (pipe * 1e12):
+        roof = {"bound": "hbm", "achieved": by / secs / 1e9, "peak": hbm, "unit": "GB/s", "peak_source": "hbm_gbs"}
+    else:
+        roof = {"bound": "alu", "achieved": fft_fl / secs / 1e12, "peak": pipe, "unit": "TFLOP/s",
+                "peak_source": pipe_text}
     out["fftdf"] = {"config": {"mesh": list(gspec.mesh), "n_ao": gspec.n_ao, "grid": list(gspec.grid),
                                "n_emb": gspec.n_emb}, "ms_per_call": ms,
                     "launches_per_call": sum(k["launches"] for k in kern_f.values()) // reps,
                     "status": st, "kernels": kern_f,
-                    "roofline": {"bound": "tensor", "kernel": "fftdf_grid", "achieved": tf, "peak": f_peak,
-                                 "unit": "TFLOP/s", "frac": tf / f_peak,
-                                 "flops_counted": "FP64 flops of the per-axis FFTs (10 N log2 N), the phases and the "
-                                                  "contraction over the grid",
-                                 "peak_source": f_text},
+                    "roofline": {**roof, "kernel": "fftdf_grid", "frac": roof["achieved"] / roof["peak"],
+                                 "bytes_counted": "FFT passes in and out, and the split contraction's partial blocks",
+                                 "fft_gflop": fft_fl / 1e9, "contraction_gflop": con_fl / 1e9},
                     "max_abs_err_over_max": float(np.abs(got - ref).max() / np.abs(ref).max())}
     print(json.dumps(out), flush=True)
     return 0
