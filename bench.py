@@ -58,9 +58,9 @@ PREC_DTYPE = {"fp64": "f64", "bf16x3": "bf16x3", "fp16x2": "fp16x2", "tf32": "tf
 # (kernel_sources_digest); after any change to the kernels or their job tables, traffic is null.
 KERNEL_SOURCES = ["tc_gemm.cuh", "tc_common.cuh", "prec.cuh", "split.cuh", "mixed_impl.cuh", "plan.cu"]
 TRAFFIC = {
-    # one-pass ncu capture of the contraction launches of one NiO-shaped call with job pacing (aa 526.2 GB,
-    # ab 1022.9 GB, bb 529.4 GB read + written) over the class's 5 launches per call
-    ("nio_4x4x4_uhf", "bf16x3", "tc_contract"): (2078.5e9 / 5, "9350c8854e55ec2d"),
+    # one-pass ncu capture of the contraction launches of one NiO-shaped call with job pacing (aa 526.1 GB,
+    # ab 1023.0 GB, bb 526.1 GB read + written) over the class's 5 launches per call
+    ("nio_4x4x4_uhf", "bf16x3", "tc_contract"): (2075.2e9 / 5, "e29d81a1f3b220d8"),
 }
 
 
