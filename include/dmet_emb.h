@@ -81,9 +81,10 @@ typedef enum {
                             FMAs; larger ones round each operand row once to 58-bit integers
                             (relative to the row's 2-norm), multiply those exactly and round each
                             result to FP64. Results that this would leave less accurate than FMAs,
-                            those whose sum of magnitudes sum |a| |b| is small beside the rows'
-                            norms (graded or localised operands), are formed as FMAs, so that
-                            every result is within the error bound of the chain of FMAs.
+                            those whose sum of magnitudes sum |a| |b| (moduli, for complex
+                            operands) is small beside the rows' norms, as for graded or localised
+                            operands, are formed as FMAs, so that the error of every result stays
+                            within the bound of a chain of FMAs in that sum.
                             Results of rows with an infinity or a NaN are FMAs too. Products whose
                             scratch the workspace limit does not leave run as FMAs. */
   DMET_PREC_BF16X3 = 1,  /* three bf16 slices per operand, six slice products per multiply-add */
